@@ -4,13 +4,16 @@
 // For facet q with Z_q = P_q + D_q S~_q Xcheck (N~_q x L):
 //   (I - prox_{alpha ||.||_*,theta})(Z) = U diag(min(s_j, alpha_j)) V^T = Z V diag(m) V^T,
 //   m_j = min(1, alpha_j / s_j), Z^T Z = V diag(s^2) V^T.
-// Three kernels:
-//   k_gram   : partial Gram matrices Z^T Z of pixel chunks (FP32, staged in smem);
-//   k_eig    : FP64 sum of the partials in fixed order, cyclic Jacobi
-//              eigen-solve of the L x L Gram, M_q = V diag(m) V^T (or weights);
+// Kernels:
+//   k_gram   : partial Gram matrices Z^T Z of pixel chunks (float pairs, staged in smem);
+//   k_eig    : FP64 sum of the partials in fixed order (k_gram_sum first where there are
+//              many), cyclic Jacobi eigen-solve of the L x L Gram in float pairs,
+//              M_q = V diag(m) V^T (or weights);
 //   k_apply  : pixel-driven: for each pixel and each facet covering it,
 //              P_q <- Z_q M_q and A += zeta D_q P_q (every A pixel written once).
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "fhs_internal.h"
 
@@ -37,17 +40,25 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // errors ~eps * lambda_max, which wipes out singular values below
 // sqrt(eps) s_max.)  Thread owns an LB x LB block of G; Lp = L rounded up to a
 // multiple of LB.  Output: FP64 partials [Q][nchunk_max][L][L].
-template <int LB>
+//
+// W64 (weights mode of Algorithm 1, once per reweighting cycle): z = wy wx x from the FP64
+// windows as a float pair, so that the small singular values entering
+// theta_bar = mu_bar / (s + mu_bar) are not limited by rounding z to FP32; the products
+// take the pairs' cross terms along (1.68 ms in FP64, 0.24 ms at 36 facets of 85^2 pixels and
+// 38 channels).
+template <int LB, bool W64>
 __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __restrict__ xc, const float* __restrict__ P,
                                               const NucFacet* __restrict__ facets, const float* __restrict__ win,
+                                              const double* __restrict__ win64,
                                               int n1, int n2, int L, int use_P, double* __restrict__ part,
                                               int nchunk_max) {
   // the staged sub-chunk and, after the last one, the per-group partial sums
   __shared__ union {
-    float z[kGramSub][kMaxL + 1];
+    float z[W64 ? 2 : 1][kGramSub][kMaxL + 1];
     double red[256 * LB * LB];
   } sm;
-  auto& z = sm.z;
+  auto& z = sm.z[0];
+  auto& zl = sm.z[W64 ? 1 : 0];
   auto& red = sm.red;
   const int q = blockIdx.y;
   const NucFacet f = facets[q];
@@ -102,13 +113,26 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
       pre[k] = val;
     }
   };
-  constexpr bool PF = LB <= 2;         // prefetch (registers permitting)
+  constexpr bool PF = LB <= 2 && !W64;         // prefetch (registers permitting)
   if (PF) fetch(p0);
   for (int s0 = p0; s0 < p1; s0 += kGramSub) {
     if constexpr (PF) {
 #pragma unroll
       for (int k = 0; k < NPT; ++k)
         if (sl0 + 4 * k < Lp) z[spix][sl0 + 4 * k] = pre[k];
+    } else if constexpr (W64) {
+      const int p = s0 + spix;
+      const int rr = p < p1 ? p / w : 0, cc = p < p1 ? p - rr * w : 0;
+      const double d64 = win64[f.wy_off + rr] * win64[f.wx_off + cc];
+      const float dh = (float)d64, dl = (float)(d64 - (double)dh);
+      const size_t xo = (size_t)(f.r0 + rr) * n2 + (f.c0 + cc);
+#pragma unroll 4
+      for (int l = sl0; l < Lp; l += 4) {
+        const float x = p < p1 && l < L ? xc[l * N + xo] : 0.f;
+        const float h = __fmul_rn(dh, x);
+        z[spix][l] = h;
+        zl[spix][l] = __fmaf_rn(dl, x, __fmaf_rn(dh, x, -h));
+      }
     } else {
 #pragma unroll 4
       for (int idx = threadIdx.x; idx < kGramSub * Lp; idx += blockDim.x) {
@@ -133,12 +157,20 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
         for (int i = 0; i < LB; ++i) a[i] = z[pix][ta * LB + i];
 #pragma unroll
         for (int j = 0; j < LB; ++j) b[j] = z[pix][tb * LB + j];
+        float al[LB], bl[LB];
+        if constexpr (W64) {
+#pragma unroll
+          for (int i = 0; i < LB; ++i) al[i] = zl[pix][ta * LB + i];
+#pragma unroll
+          for (int j = 0; j < LB; ++j) bl[j] = zl[pix][tb * LB + j];
+        }
 #pragma unroll
         for (int i = 0; i < LB; ++i)
 #pragma unroll
           for (int j = 0; j < LB; ++j) {
             float pr = __fmul_rn(a[i], b[j]);
             float pe = __fmaf_rn(a[i], b[j], -pr);
+            if constexpr (W64) pe = __fmaf_rn(al[i], b[j], __fmaf_rn(a[i], bl[j], pe));
             float s, e;
             two_sum(hi[i][j], pr, s, e);
             hi[i][j] = s;
@@ -170,221 +202,442 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
   }
 }
 
-// FP64 partial Gram of D_q S~_q x (weights mode of Algorithm 1, once per
-// reweighting cycle): z = wy * wx * x formed and multiplied in FP64 so that
-// the small singular values entering theta_bar = mu_bar / (s + mu_bar) are not
-// limited by rounding z to FP32.
-__global__ void __launch_bounds__(256) k_gram_f64(const float* __restrict__ xc, const NucFacet* __restrict__ facets,
-                                                  const double* __restrict__ win64, int n1, int n2, int L,
-                                                  double* __restrict__ part, int nchunk_max) {
-  __shared__ double z[kGramSub / 2][kMaxL + 1];
-  constexpr int SUB = kGramSub / 2;
-  const int q = blockIdx.y;
+// ------------------------------------------------------------ eigen-solve
+// A GB300 SM issues one FP64 warp instruction per 64 clocks and sub-partition, whatever
+// the number of active lanes (measured: 64 clk per dependent or independent DFMA, 431 for
+// 1/x or rsqrt, 1.7 lanes/clk per SM), 76 times below FP32.  The Jacobi eigen-solve
+// therefore runs on pairs of floats (hi + lo, about 2^-47), and FP64 keeps what the pairs
+// would lose: the sums of the chunk partials, m_j, and, for the weights, the
+// eigenvalues themselves (Rayleigh quotients, whose error is second order in the
+// eigenvectors').
+struct ff {
+  float h, l;
+};
+
+__device__ __forceinline__ ff ff_of(double x) {
+  const float h = (float)x;
+  return {h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ double ff_val(ff a) { return (double)a.h + (double)a.l; }
+
+// c a + s b.
+__device__ __forceinline__ ff ff_lin(ff c, ff a, ff s, ff b) {
+  const float p = __fmul_rn(c.h, a.h), q = __fmul_rn(s.h, b.h);
+  float pe = __fmaf_rn(c.h, a.h, -p), qe = __fmaf_rn(s.h, b.h, -q);
+  pe = __fmaf_rn(c.l, a.h, __fmaf_rn(c.h, a.l, pe));
+  qe = __fmaf_rn(s.l, b.h, __fmaf_rn(s.h, b.l, qe));
+  float t, e;
+  two_sum(p, q, t, e);
+  e = __fadd_rn(e, __fadd_rn(pe, qe));
+  const float h = __fadd_rn(t, e);
+  return {h, __fsub_rn(e, __fsub_rn(h, t))};
+}
+
+__device__ __forceinline__ ff ff_mul(ff a, ff b) {
+  const float p = __fmul_rn(a.h, b.h);
+  const float e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
+  const float h = __fadd_rn(p, e);
+  return {h, __fsub_rn(e, __fsub_rn(h, p))};
+}
+
+// u^-1/2 (u > 0): one Newton step from the FP32 value with the residual 1 - u y^2 formed
+// as a pair.
+__device__ __forceinline__ ff ff_rsqrt(ff u) {
+  const float y = rsqrtf(u.h);
+  const float q = __fmul_rn(y, y), qe = __fmaf_rn(y, y, -q);
+  const float w = __fmul_rn(u.h, q);
+  const float we = __fmaf_rn(u.l, q, __fmaf_rn(u.h, qe, __fmaf_rn(u.h, q, -w)));
+  const float r = __fsub_rn(__fsub_rn(1.f, w), we);
+  const float cor = y * fmaf(0.375f * r, r, 0.5f * r);
+  const float h = __fadd_rn(y, cor);
+  return {h, __fsub_rn(cor, __fsub_rn(h, y))};
+}
+
+// Plane rotation (c, s) that annihilates gpr of [[gpp, gpr], [gpr, grr]] up to the FP32
+// accuracy of its tangent (the remainder is annihilated in the next sweep); c and s are
+// float pairs with c^2 + s^2 = 1 to about 2^-46.  False (identity) when gpr is below the
+// accuracy of the pairs relative to the larger diagonal entry, or not a number.
+__device__ __forceinline__ bool ff_rotation(ff gpp, ff gpr, ff grr, ff& c, ff& s) {
+  c = {1.f, 0.f};
+  s = {0.f, 0.f};
+  const float g = gpr.h + gpr.l;
+  const float big = fmaxf(fabsf(gpp.h), fabsf(grr.h));
+  if (!(fabsf(g) > 5.7e-14f * big) || !(fabsf(g) > 1e-30f)) return false;       // 2^-44
+  const float d = __fadd_rn(__fsub_rn(grr.h, gpp.h), __fsub_rn(grr.l, gpp.l));
+  // tan = g / (|d|/2 + sqrt(d^2/4 + g^2)) with the sign of d; it may be off by a few ulp
+  // and is taken as exact from here on
+  const float h2 = 0.5f * fabsf(d);
+  float root;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(h2, h2, g * g)));
+  const float t = __fdividef(copysignf(1.f, d) * g, h2 + root);
+  // c = (1 + t^2)^-1/2, s = t c
+  const float p = __fmul_rn(t, t), pe = __fmaf_rn(t, t, -p);
+  const float uh = __fadd_rn(1.f, p);
+  c = ff_rsqrt({uh, __fadd_rn(__fsub_rn(p, __fsub_rn(uh, 1.f)), pe)});
+  const float sp = __fmul_rn(t, c.h);
+  const float se = __fmaf_rn(t, c.l, __fmaf_rn(t, c.h, -sp));
+  s.h = __fadd_rn(sp, se);
+  s.l = __fsub_rn(se, __fsub_rn(s.h, sp));
+  return true;
+}
+
+constexpr int kEigRows = 3;        // eigenvector-row items per worker thread, at most
+constexpr int kEigParts = 32;      // partial Grams per facet after k_gram_sum
+constexpr int kEigDirect = 64;     // up to this many partials k_eig adds them itself
+
+// Adds the chunk partials of a facet in a fixed order down to kEigParts: CTA g sums the
+// chunks g, g + kEigParts, ... into chunk g (facets of more than kEigDirect chunks, where
+// one CTA of k_eig would read megabytes alone).
+__global__ void __launch_bounds__(256) k_gram_sum(double* __restrict__ part, int nchunk_max,
+                                                  const NucFacet* __restrict__ facets, int L) {
+  __shared__ double acc[256];
+  const int q = blockIdx.y, g = blockIdx.x;
   const NucFacet f = facets[q];
-  const int h = f.r1 - f.r0, w = f.c1 - f.c0;
-  const int Nq = h * w;
-  const int p0 = blockIdx.x * kGramChunk;
-  if (p0 >= Nq) return;
-  const int p1 = min(Nq, p0 + kGramChunk);
-  const int LB = L <= 16 ? 1 : (L <= 32 ? 2 : 4);
-  const int Lp = (L + LB - 1) / LB * LB;
-  const int nb = Lp / LB;
-  const int ta = threadIdx.x / nb, tb = threadIdx.x % nb;
-  const bool active = ta < nb && ta <= tb;
-  double acc[4][4];
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  const size_t N = (size_t)n1 * n2;
-  for (int s0 = p0; s0 < p1; s0 += SUB) {
-    for (int idx = threadIdx.x; idx < SUB * Lp; idx += blockDim.x) {
-      int pix = idx % SUB, l = idx / SUB;
-      int p = s0 + pix;
-      double val = 0.0;
-      if (p < p1 && l < L) {
-        int rr = p / w, cc = p % w;
-        val = win64[f.wy_off + rr] * win64[f.wx_off + cc] * (double)xc[l * N + (size_t)(f.r0 + rr) * n2 + (f.c0 + cc)];
+  const int nch = ((f.r1 - f.r0) * (f.c1 - f.c0) + kGramChunk - 1) / kGramChunk;
+  if (nch <= kEigParts || g >= nch) return;
+  double* pq = part + (size_t)q * nchunk_max * L * L;
+  const int LL = L * L;
+  // up to 128 entries: thread -> (entry, share of the chunks), shares added in order
+  const int share = LL <= 128 ? 256 / LL : 1;
+  const int per = share > 1 ? LL : 256;
+  const int e0 = threadIdx.x % per, sh = threadIdx.x / per;
+  for (int eb = 0; eb < LL; eb += per) {
+    const int e = eb + e0;
+    double s = 0.0;
+    if (e < LL && sh < share) {
+      int c = g + kEigParts * sh;
+      for (; c + 3 * kEigParts * share < nch; c += 4 * kEigParts * share) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = pq[(size_t)(c + k * kEigParts * share) * LL + e];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s += v[k];
       }
-      z[pix][l] = val;
+      for (; c < nch; c += kEigParts * share) s += pq[(size_t)c * LL + e];
     }
-    __syncthreads();
-    if (active) {
-      for (int pix = 0; pix < SUB; ++pix)
-        for (int i = 0; i < LB; ++i)
-          for (int j = 0; j < LB; ++j) acc[i][j] = fma(z[pix][ta * LB + i], z[pix][tb * LB + j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  if (active) {
-    double* out = part + ((size_t)q * nchunk_max + blockIdx.x) * L * L;
-    for (int i = 0; i < LB; ++i)
-      for (int j = 0; j < LB; ++j) {
-        int a = ta * LB + i, b = tb * LB + j;
-        if (a < L && b < L) {
-          out[a * L + b] = acc[i][j];
-          out[b * L + a] = acc[i][j];
-        }
+    if (share == 1) {
+      if (e < LL) pq[(size_t)g * LL + e] = s;
+    } else {
+      acc[threadIdx.x] = s;
+      __syncthreads();
+      if (sh == 0 && e < LL) {
+        for (int k = 1; k < share; ++k) s += acc[k * per + e0];
+        pq[(size_t)g * LL + e] = s;
       }
+    }
   }
 }
 
-// One warp per facet: G = sum of partial Grams (FP64, fixed order), cyclic
-// Jacobi eigen-decomposition G = V diag(lambda) V^T, s = sqrt(max(lambda, 0))
-// sorted descending, then either M = V diag(m) V^T with
-// m_j = min(1, alpha_j / s_j), alpha_j = (mu_bar_q / zeta) theta_bar_q[rank j]
-// (dual mode), or theta_bar_q[rank] = mu_bar_q / (s + mu_bar_q) (weights mode).
-__global__ void __launch_bounds__(32) k_eig(const double* __restrict__ part, int nchunk_max,
-                                            const NucFacet* __restrict__ facets, int L,
-                                            const float* __restrict__ theta_bar, const float* __restrict__ mubar,
-                                            float inv_zeta, float* __restrict__ Mout, float* __restrict__ tb_out,
-                                            int weights_mode, int max_sweeps) {
-  extern __shared__ double sh[];
-  const int Ls = L + 1;
-  double* G = sh;                 // [L][L+1]
-  double* V = sh + L * Ls;        // [L][L+1]
-  double* lam = V + L * Ls;       // [L]
-  double* rc = lam + L;           // [L/2 + 1] rotation cosines of a round
-  double* rs = rc + (L / 2 + 1);  // [L/2 + 1] sines
-  int* rank = (int*)(rs + (L / 2 + 1));   // [L]
-  int* rp = rank + L;             // [L/2 + 1] pair indices
-  int* rr = rp + (L / 2 + 1);
-  const int q = blockIdx.x, lane = threadIdx.x;
+// Threads of k_eig: warp 0 (rotations, diagonal blocks) and two threads per 2 x 2 block of G
+// above the diagonal blocks, which rotate the eigenvector rows as well.
+static int eig_threads(int L) {
+  const int H = (L + 1) / 2, nB = H * (H - 1) / 2;
+  const int work = std::max(2 * nB, (H * L + kEigRows - 1) / kEigRows);
+  return 32 + std::max(32, (work + 31) & ~31);
+}
+static size_t eig_smem(int L, bool weights) {
+  const size_t Le = (L + 1) & ~1, H = Le / 2;
+  const size_t b = 2 * Le * (Le + 1) * sizeof(float2) + 2 * H * (sizeof(float4) + sizeof(int2)) +
+                   L * (2 * sizeof(float2) + sizeof(float) + sizeof(int));
+  return ((b + 15) & ~(size_t)15) + (weights ? 3 * (size_t)L * L * sizeof(double) : 0);
+}
+
+// One CTA per facet: G = sum of the partial Grams (FP64, chunk order), cyclic Jacobi
+// eigen-decomposition G = V diag(lambda) V^T in float pairs, s = sqrt(max(lambda, 0))
+// sorted descending, then either M = V diag(m) V^T with m_j = min(1, alpha_j / s_j),
+// alpha_j = (mu_bar_q / zeta) theta_bar_q[rank j] (dual mode), or
+// theta_bar_q[rank] = mu_bar_q / (s + mu_bar_q) (weights mode).
+//
+// Bound by the latency of a round: the rotations of H = Le/2 disjoint index pairs (warp 0,
+// about 500 clk), a barrier, every 2 x 2 block of G transformed in place from both
+// sides by two threads, a barrier; the eigenvector rows of a round are rotated
+// beside the next round's rotations.  One warp in FP64 took 1.09 ms at 20
+// channels (16 facets), 3.74 ms at 32 (64 facets) and, for the weights, 6.48 ms at 38 (36
+// facets); this kernel takes 0.098, 0.24 and 0.33 ms (device times of one launch).
+__global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, int nchunk_max, int nparts_max,
+                                             const NucFacet* __restrict__ facets, int L,
+                                             const float* __restrict__ theta_bar, const float* __restrict__ mubar,
+                                             float inv_zeta, float* __restrict__ Mout, float* __restrict__ tb_out,
+                                             int weights_mode, int max_sweeps) {
+  extern __shared__ __align__(16) unsigned char eig_smem_raw[];
+  __shared__ int s_emax;
+  const int Le = (L + 1) & ~1, H = Le / 2, Ls = Le + 1;
+  float4* rot = reinterpret_cast<float4*>(eig_smem_raw);          // [2][H] (c, s) of a round
+  int2* pr = reinterpret_cast<int2*>(rot + 2 * H);                // [2][H] index pairs of a round
+  float2* G = reinterpret_cast<float2*>(pr + 2 * H);              // [Le][Ls] pairs, index L (odd L): zeros
+  float2* V = G + Le * Ls;                                        // [Le][Ls], row j = eigenvector j
+  float2* lam = V + Le * Ls;                                      // [L]
+  float2* tm = lam + L;                                           // [L] m_j
+  float* tbq = reinterpret_cast<float*>(tm + L);                  // [L]
+  int* rank = reinterpret_cast<int*>(tbq + L);                    // [L]
+  double* G64 = reinterpret_cast<double*>(
+      eig_smem_raw + (((unsigned char*)(rank + L) - eig_smem_raw + 15) & ~(size_t)15));   // weights: [L][L]
+  const int q = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const NucFacet f = facets[q];
   const int Nq = (f.r1 - f.r0) * (f.c1 - f.c0);
-  const int nch = (Nq + kGramChunk - 1) / kGramChunk;
-  // sum of the chunk partials, chunk 0 first: eight entries of the lane at a time, so
-  // that each chunk's eight loads are in flight together (the order of the additions of
-  // an entry is the chunk order either way)
-  constexpr int kEigBatch = 8;
-  for (int e0 = lane; e0 < L * L; e0 += 32 * kEigBatch) {
-    double s[kEigBatch];
-#pragma unroll
-    for (int k = 0; k < kEigBatch; ++k) s[k] = 0.0;
-    const double* pq = part + (size_t)q * nchunk_max * L * L;
-    for (int c = 0; c < nch; ++c) {
-      const double* pc = pq + (size_t)c * L * L;
-#pragma unroll
-      for (int k = 0; k < kEigBatch; ++k) {
-        const int idx = e0 + 32 * k;
-        if (idx < L * L) s[k] += pc[idx];
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kEigBatch; ++k) {
-      const int idx = e0 + 32 * k;
-      if (idx < L * L) {
-        const int a = idx / L, b = idx % L;
-        G[a * Ls + b] = s[k];
-        V[a * Ls + b] = (a == b) ? 1.0 : 0.0;
-      }
-    }
-  }
-  __syncwarp();
-  // symmetrise (the partial Grams are symmetric up to rounding order)
-  for (int idx = lane; idx < L * L; idx += 32) {
-    int a = idx / L, b = idx % L;
-    if (a < b) {
-      double m = 0.5 * (G[a * Ls + b] + G[b * Ls + a]);
-      G[a * Ls + b] = m;
-      G[b * Ls + a] = m;
-    }
-  }
-  __syncwarp();
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    __syncwarp();
-    double off = 0.0, dia = 0.0;
-    for (int idx = lane; idx < L * L; idx += 32) {
-      int a = idx / L, b = idx % L;
-      double g = G[a * Ls + b];
-      if (a == b) dia += g * g; else off += g * g;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      off += __shfl_xor_sync(0xffffffffu, off, o);
-      dia += __shfl_xor_sync(0xffffffffu, dia, o);
-    }
-    if (off <= 1e-30 * dia || off == 0.0) break;
-    // one sweep = Le - 1 rounds of the round-robin tournament over Le = L rounded up to
-    // even (index L is a dummy); a round rotates Le/2 disjoint pairs at once: lane j
-    // computes pair j's rotation from the round's G, then rows and columns are
-    // updated for all pairs (the pairs are disjoint, so this is exact)
-    const int Le = (L + 1) & ~1, H = Le / 2;
-    for (int rnd = 0; rnd < Le - 1; ++rnd) {
-      auto player = [&](int k) { return k == 0 ? 0 : ((k - 1 + rnd) % (Le - 1)) + 1; };
-      __syncwarp();
-      for (int j = lane; j < H; j += 32) {
-        int p = player(j), r = player(Le - 1 - j);
-        if (p > r) { int t = p; p = r; r = t; }
-        double c = 1.0, sn = 0.0;
-        if (r < L) {
-          const double gpr = G[p * Ls + r], gpp = G[p * Ls + p], grr = G[r * Ls + r];
-          if (fabs(gpr) > 1e-300 && fabs(gpr) > 1e-18 * sqrt(fabs(gpp * grr))) {
-            const double th = (grr - gpp) / (2.0 * gpr);
-            const double t = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
-            c = 1.0 / sqrt(1.0 + t * t);
-            sn = t * c;
-          }
-        }
-        rp[j] = p; rr[j] = r; rc[j] = c; rs[j] = sn;
-      }
-      __syncwarp();
-      for (int idx = lane; idx < H * L; idx += 32) {     // rows p, r
-        const int j = idx / L, k = idx - j * L;
-        const int p = rp[j], r = rr[j];
-        if (r >= L || rs[j] == 0.0) continue;
-        const double c = rc[j], sn = rs[j];
-        const double a = G[p * Ls + k], b = G[r * Ls + k];
-        G[p * Ls + k] = c * a - sn * b;
-        G[r * Ls + k] = sn * a + c * b;
-      }
-      __syncwarp();
-      for (int idx = lane; idx < H * L; idx += 32) {     // columns p, r and eigenvectors
-        const int j = idx / L, k = idx - j * L;
-        const int p = rp[j], r = rr[j];
-        if (r >= L || rs[j] == 0.0) continue;
-        const double c = rc[j], sn = rs[j];
-        const double a = G[k * Ls + p], b = G[k * Ls + r];
-        G[k * Ls + p] = c * a - sn * b;
-        G[k * Ls + r] = sn * a + c * b;
-        const double va = V[k * Ls + p], vb = V[k * Ls + r];
-        V[k * Ls + p] = c * va - sn * vb;
-        V[k * Ls + r] = sn * va + c * vb;
-      }
-    }
-  }
-  __syncwarp();
-  for (int j = lane; j < L; j += 32) lam[j] = G[j * Ls + j];
-  __syncwarp();
-  for (int j = lane; j < L; j += 32) {
-    int rk = 0;
-    for (int k = 0; k < L; ++k) rk += (lam[k] > lam[j]) || (lam[k] == lam[j] && k < j);
-    rank[j] = rk;
-  }
-  __syncwarp();
+  const int nch = min((Nq + kGramChunk - 1) / kGramChunk, nparts_max);
   const float mb = mubar[q];
-  if (weights_mode) {
-    for (int j = lane; j < L; j += 32) {
-      double s = sqrt(fmax(lam[j], 0.0));
-      tb_out[(size_t)q * L + rank[j]] = (float)((double)mb / (s + (double)mb));
+  if (tid == 0) s_emax = 0;
+  for (int k = tid; k < Le * Ls; k += nt) {
+    const int a = k / Ls, b = k - a * Ls;
+    G[k] = make_float2(0.f, 0.f);
+    V[k] = make_float2(a == b ? 1.f : 0.f, 0.f);
+  }
+  if (!weights_mode)
+    for (int j = tid; j < L; j += nt) tbq[j] = theta_bar[(size_t)q * L + j];
+  __syncthreads();
+  // ---- G (upper triangle; the partials are symmetric), kept in FP64 registers until the
+  // scale 4^-k that takes the largest diagonal entry into [1, 4) is known
+  const int nE = L * (L + 1) / 2;
+  constexpr int kHold = 5;                       // nE <= kHold nt for every L <= 64
+  double g64[kHold];
+  const double* pq = part + (size_t)q * nchunk_max * L * L;
+  auto entry = [](int e, int& a, int& b) {       // e -> (a, b), a <= b
+    b = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+    while (b * (b + 1) / 2 > e) --b;
+    while ((b + 1) * (b + 2) / 2 <= e) ++b;
+    a = e - b * (b + 1) / 2;
+  };
+#pragma unroll
+  for (int u = 0; u < kHold; ++u) {
+    const int e = tid + u * nt;
+    g64[u] = 0.0;
+    if (e >= nE) continue;
+    int a, b;
+    entry(e, a, b);
+    double s = 0.0;
+    int c = 0;
+    for (; c + 8 <= nch; c += 8) {
+      double v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = pq[(size_t)(c + k) * L * L + a * L + b];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s += v[k];
     }
-    return;
+    for (; c < nch; ++c) s += pq[(size_t)c * L * L + a * L + b];
+    g64[u] = s;
+    if (a == b) {
+      const int ex = (__double2hiint(s) >> 20) & 0x7ff;
+      if (ex != 0x7ff) atomicMax(&s_emax, ex);
+    }
   }
-  // m_j stored in lam
-  __syncwarp();
-  for (int j = lane; j < L; j += 32) {
-    double s = sqrt(fmax(lam[j], 0.0));
-    double alpha = (double)mb * (double)inv_zeta * (double)theta_bar[(size_t)q * L + rank[j]];
-    lam[j] = (s > alpha) ? alpha / s : 1.0;
+  __syncthreads();
+  // 4^k <= largest diagonal entry < 4^(k+1)
+  const int k4 = s_emax == 0 ? 0 : (s_emax - 1023) >> 1;
+  const double down = __hiloint2double((1023 - 2 * k4) << 20, 0);
+#pragma unroll
+  for (int u = 0; u < kHold; ++u) {
+    const int e = tid + u * nt;
+    if (e >= nE) continue;
+    int a, b;
+    entry(e, a, b);
+    const double g = g64[u] * down;
+    ff x = ff_of(g);
+    if (!(fabsf(x.h) < 3e38f)) x = {__int_as_float(0x7fffffff), 0.f};
+    G[a * Ls + b] = G[b * Ls + a] = make_float2(x.h, x.l);
+    if (weights_mode) G64[a * L + b] = G64[b * L + a] = g;
   }
-  __syncwarp();
-  // M_q^T, rows padded to Lp = L rounded up to 4 (zeros), so that a row is read as float4
+  __syncthreads();
+  // ---- one sweep = Le - 1 rounds of the round-robin tournament over Le indices; a round
+  // rotates H disjoint pairs at once
+  const int nB = H * (H - 1) / 2, wt = tid - 32, nw = nt - 32;     // worker threads: warps 1 and up
+  int bi = 0, bj = 0;                            // the worker's block: (pair bi) x (pair bj), bi < bj;
+  const bool has_block = wt >= 0 && wt < 2 * nB; // lane parity: the row of pair bi it writes
+  const unsigned block_lanes = __ballot_sync(0xffffffffu, has_block);
+  const int half = wt & 1;
+  if (has_block) {
+    const int t = wt >> 1;
+    bj = (int)((sqrtf(8.f * t + 1.f) + 1.f) * 0.5f);
+    while (bj * (bj - 1) / 2 > t) --bj;
+    while ((bj + 1) * bj / 2 <= t) ++bj;
+    bi = t - bj * (bj - 1) / 2;
+  }
+  int vi[kEigRows], vk[kEigRows];                // its eigenvector rows: (pair, component)
+#pragma unroll
+  for (int m = 0; m < kEigRows; ++m) {
+    const int k = wt + m * nw;
+    vi[m] = wt >= 0 && k < H * L ? k / L : -1;
+    vk[m] = vi[m] >= 0 ? k - vi[m] * L : 0;
+  }
+  auto ldp = [](const float2* m, int k) {
+    const float2 x = m[k];
+    return ff{x.x, x.y};
+  };
+  auto stg = [&](int a, int b, ff x) { G[a * Ls + b] = G[b * Ls + a] = make_float2(x.h, x.l); };
+  // eigenvector rows of the round in buffer `buf` (an identity rotation leaves its pairs as
+  // they are)
+  auto rotate_rows = [&](int buf) {
+    int o[kEigRows], o2[kEigRows];
+    ff vp[kEigRows], vr[kEigRows];
+    float4 r[kEigRows];
+#pragma unroll
+    for (int m = 0; m < kEigRows; ++m) {
+      const int i = max(vi[m], 0);
+      const int2 pi = pr[buf * H + i];
+      r[m] = rot[buf * H + i];
+      o[m] = pi.x * Ls + vk[m];
+      o2[m] = pi.y * Ls + vk[m];
+      vp[m] = ldp(V, o[m]);
+      vr[m] = ldp(V, o2[m]);
+    }
+    bool turn = false;
+#pragma unroll
+    for (int m = 0; m < kEigRows; ++m) turn = turn || r[m].z != 0.f;
+    if (!turn) return;
+#pragma unroll
+    for (int m = 0; m < kEigRows; ++m) {
+      const ff c = {r[m].x, r[m].y}, s = {r[m].z, r[m].w};
+      const ff x = ff_lin(c, vp[m], {-s.h, -s.l}, vr[m]), y = ff_lin(s, vp[m], c, vr[m]);
+      if (vi[m] >= 0) {
+        V[o[m]] = make_float2(x.h, x.l);
+        V[o2[m]] = make_float2(y.h, y.l);
+      }
+    }
+  };
+  int buf = 0, rows_due = 0;
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+    int rotated = 0;
+    for (int rnd = 0; rnd < Le - 1; ++rnd) {
+      int mine = 0, p = 0, r = 0;
+      ff gpp, gpr, grr, c, s;
+      if (tid < 32) {
+        if (tid < H) {
+          auto player = [&](int k) {
+            int x = k - 1 + rnd;
+            x = x >= Le - 1 ? x - (Le - 1) : x;
+            return k == 0 ? 0 : x + 1;
+          };
+          p = player(tid);
+          r = player(Le - 1 - tid);
+          if (p > r) { const int x = p; p = r; r = x; }
+          gpp = ldp(G, p * Ls + p);
+          gpr = ldp(G, p * Ls + r);
+          grr = ldp(G, r * Ls + r);
+          mine = ff_rotation(gpp, gpr, grr, c, s) ? 1 : 0;
+          rot[buf * H + tid] = make_float4(c.h, c.l, s.h, s.l);
+          pr[buf * H + tid] = make_int2(p, r);
+        }
+      } else if (rows_due) {
+        rotate_rows(buf ^ 1);
+      }
+      const int any = __syncthreads_or(mine);
+      if (any) {
+        rotated = 1;
+        if (tid < 32) {
+          if (mine) {                                        // diagonal block, from registers
+            const ff ns = {-s.h, -s.l};
+            const ff a1 = ff_lin(c, gpp, ns, gpr), b1 = ff_lin(c, gpr, ns, grr);
+            const ff c1 = ff_lin(s, gpp, c, gpr), d1 = ff_lin(s, gpr, c, grr);
+            stg(p, p, ff_lin(c, a1, ns, b1));
+            stg(p, r, ff_lin(s, a1, c, b1));
+            stg(r, r, ff_lin(s, c1, c, d1));
+          }
+        } else if (has_block) {
+          // the two threads of a block read all of it, then write a row each
+          const float4 ri = rot[buf * H + bi], rj = rot[buf * H + bj];
+          const int2 pi = pr[buf * H + bi], pj = pr[buf * H + bj];
+          const int row = half ? pi.y : pi.x, other = half ? pi.x : pi.y;
+          const ff ci = {ri.x, ri.y}, si = half ? ff{ri.z, ri.w} : ff{-ri.z, -ri.w};
+          const ff cj = {rj.x, rj.y}, sj = {rj.z, rj.w};
+          const ff a = ldp(G, row * Ls + pj.x), b = ldp(G, row * Ls + pj.y);
+          const ff d = ldp(G, other * Ls + pj.x), e = ldp(G, other * Ls + pj.y);
+          const ff a1 = ff_lin(ci, a, si, d), b1 = ff_lin(ci, b, si, e);
+          const ff a2 = ff_lin(cj, a1, {-sj.h, -sj.l}, b1), b2 = ff_lin(sj, a1, cj, b1);
+          __syncwarp(block_lanes);
+          stg(row, pj.x, a2);
+          stg(row, pj.y, b2);
+        }
+        __syncthreads();
+      }
+      rows_due = any;
+      buf ^= 1;
+    }
+    if (!rotated) break;
+  }
+  if (rows_due && wt >= 0) rotate_rows(buf ^ 1);
+  __syncthreads();
+  if (weights_mode) {
+    // ---- Rayleigh quotients v^T G v / v^T v in FP64
+    double* V64 = G64 + L * L;                                     // [L][L]
+    double* W64 = V64 + L * L;
+    for (int k = tid; k < L * L; k += nt) {
+      const int j = k / L, a = k - j * L;
+      V64[k] = ff_val(ldp(V, j * Ls + a));
+    }
+    __syncthreads();
+    for (int k = tid; k < L * L; k += nt) {
+      const int j = k / L, a = k - j * L;
+      double y = 0.0;
+      for (int b = 0; b < L; ++b) y = fma(G64[b * L + a], V64[j * L + b], y);
+      W64[k] = V64[k] * y;
+    }
+    __syncthreads();
+    for (int j = tid; j < L; j += nt) {
+      double n = 0.0, s = 0.0;
+      for (int a = 0; a < L; ++a) {
+        s += W64[j * L + a];
+        n = fma(V64[j * L + a], V64[j * L + a], n);
+      }
+      const double r = s / n;
+      const ff x = ff_of(r);
+      lam[j] = make_float2(x.h, x.l);
+      G64[j] = r;                                // G64 was last read before the barrier above
+    }
+  } else {
+    for (int j = tid; j < L; j += nt) lam[j] = G[j * Ls + j];
+  }
+  __syncthreads();
+  for (int j = tid; j < L; j += nt) {
+    const float2 x = lam[j];
+    int rk = 0;
+#pragma unroll 4
+    for (int k = 0; k < L; ++k) {
+      const float2 y = lam[k];
+      rk += (y.x > x.x) || (y.x == x.x && (y.y > x.y || (y.y == x.y && k < j)));
+    }
+    rank[j] = rk;
+    if (weights_mode) {
+      const double sv = sqrt(fmax(G64[j], 0.0)) * __hiloint2double((1023 + k4) << 20, 0);
+      tb_out[(size_t)q * L + rk] = (float)((double)mb / (sv + (double)mb));
+      continue;
+    }
+    // m = min(1, alpha lambda^-1/2) in the scaled units, 1 where lambda is not positive
+    const ff al = ff_of((double)mb * (double)inv_zeta * (double)tbq[rk] * __hiloint2double((1023 - k4) << 20, 0));
+    ff m = {1.f, 0.f};
+    if (x.x > 0.f) {
+      const ff t = ff_mul(al, ff_rsqrt({x.x, x.y}));
+      if (t.h < 1.f || (t.h == 1.f && t.l < 0.f)) m = t;
+    }
+    tm[j] = make_float2(m.h, m.l);
+  }
+  if (weights_mode) return;
+  __syncthreads();
+  for (int k = tid; k < L * L; k += nt) {        // diag(m) V^T, over G
+    const int j = k / L, o = j * Ls + k - j * L;
+    const ff w = ff_mul(ldp(tm, j), ldp(V, o));
+    G[o] = make_float2(w.h, w.l);
+  }
+  __syncthreads();
+  // M_q^T, rows padded to Lp = L rounded up to 4 (zeros), so that a row is read as float4;
+  // each entry (symmetric) is summed in float pairs and rounded once
   const int Lp = (L + 3) & ~3;
-  for (int idx = lane; idx < L * Lp; idx += 32) {
-    int b = idx / Lp, a = idx % Lp;
-    double m = 0.0;
-    if (a < L)
-      for (int j = 0; j < L; ++j) m += V[a * Ls + j] * lam[j] * V[b * Ls + j];
-    Mout[(size_t)q * L * Lp + idx] = (float)m;
+  float* Mq = Mout + (size_t)q * L * Lp;
+  for (int e = tid; e < nE; e += nt) {
+    int a, b;
+    entry(e, a, b);
+    ff m0 = {0.f, 0.f}, m1 = {0.f, 0.f};
+    const ff one = {1.f, 0.f};
+    int j = 0;
+#pragma unroll 2
+    for (; j + 2 <= L; j += 2) {
+      m0 = ff_lin(ldp(G, j * Ls + b), ldp(V, j * Ls + a), one, m0);
+      m1 = ff_lin(ldp(G, (j + 1) * Ls + b), ldp(V, (j + 1) * Ls + a), one, m1);
+    }
+    if (j < L) m0 = ff_lin(ldp(G, j * Ls + b), ldp(V, j * Ls + a), one, m0);
+    m0 = ff_lin(one, m0, one, m1);
+    Mq[b * Lp + a] = Mq[a * Lp + b] = m0.h + m0.l;
   }
+  for (int k = tid; k < L * (Lp - L); k += nt) Mq[(k / (Lp - L)) * Lp + L + k % (Lp - L)] = 0.f;
 }
 
 // Pixel-driven update: each thread owns one pixel; for every facet covering it,
@@ -506,18 +759,25 @@ void launch_nuclear(fhs_ctx* ctx, const Cube& cb, const float* xcheck, float* P,
   if (!weights_mode) launch_nuclear_apply(ctx, cb, xcheck, P, A, st);
 }
 
+template <bool W64>
+static void gram_cuda_core(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, cudaStream_t st) {
+  const int L = cb.L, nch = nchunk_max(cb), use_P = P != nullptr ? 1 : 0;
+  dim3 gg(nch, cb.Qy * cb.Qx);
+  auto go = [&](auto kernel) {
+    kernel<<<gg, 256, 0, st>>>(xcheck, P, cb.d_facets, cb.d_win, cb.d_win64, cb.n1, cb.n2, L, use_P, ctx->s.gram, nch);
+  };
+  if (L <= 4) go(k_gram<1, W64>);
+  else if (L <= 16) go(k_gram<2, W64>);
+  else go(k_gram<4, W64>);
+  note_launches(1);
+}
+
 // Per-chunk partial Grams of Z_q = D_q S~_q xcheck (+ P_q) into ctx->s.gram: the tcgen05
 // kernel when tc and L <= 32, else the CUDA-core float-float kernel.
 void launch_gram(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, bool tc, cudaStream_t st) {
-  const int L = cb.L;
   const int nch = nchunk_max(cb);
-  dim3 gg(nch, cb.Qy * cb.Qx);
-  const int use_P = P != nullptr ? 1 : 0;
   if (tc && launch_gram_tc(cb, xcheck, P, ctx->s.gram, nch, st)) return;   // counts its launch
-  if (L <= 4) k_gram<1><<<gg, 256, 0, st>>>(xcheck, P, cb.d_facets, cb.d_win, cb.n1, cb.n2, L, use_P, ctx->s.gram, nch);
-  else if (L <= 16) k_gram<2><<<gg, 256, 0, st>>>(xcheck, P, cb.d_facets, cb.d_win, cb.n1, cb.n2, L, use_P, ctx->s.gram, nch);
-  else k_gram<4><<<gg, 256, 0, st>>>(xcheck, P, cb.d_facets, cb.d_win, cb.n1, cb.n2, L, use_P, ctx->s.gram, nch);
-  note_launches(1);
+  gram_cuda_core<false>(ctx, cb, xcheck, P, st);
 }
 
 void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P,
@@ -525,19 +785,21 @@ void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, 
   const int L = cb.L;
   const int Q = cb.Qy * cb.Qx;
   const int nch = nchunk_max(cb);
-  dim3 gg(nch, Q);
-  if (weights_mode) {
-    k_gram_f64<<<gg, 256, 0, st>>>(xcheck, cb.d_facets, cb.d_win64, cb.n1, cb.n2, L, ctx->s.gram, nch);
+  if (weights_mode) gram_cuda_core<true>(ctx, cb, xcheck, nullptr, st);
+  else launch_gram(ctx, cb, xcheck, P, ctx->path == FHS_PATH_FAST && cb.gram_tc, st);
+  const bool sum = nch > kEigDirect;
+  if (sum) {
+    k_gram_sum<<<dim3(kEigParts, Q), 256, 0, st>>>(ctx->s.gram, nch, cb.d_facets, L);
     note_launches(1);
-  } else {
-    launch_gram(ctx, cb, xcheck, P, ctx->path == FHS_PATH_FAST && cb.gram_tc, st);
   }
-  size_t sm = (size_t)2 * L * (L + 1) * sizeof(double) + L * sizeof(double) + 2 * (L / 2 + 1) * sizeof(double) +
-              (L + 2 * (L / 2 + 1)) * sizeof(int);
   static bool attr = false;
-  if (!attr) { cudaFuncSetAttribute(k_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024); attr = true; }
-  k_eig<<<Q, 32, sm, st>>>(ctx->s.gram, nch, cb.d_facets, L, theta_bar, cb.d_mubar, (float)(1.0 / cb.zeta),
-                           ctx->s.nucM, theta_bar_out, weights_mode ? 1 : 0, 40);
+  if (!attr) {
+    cudaFuncSetAttribute(k_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_smem(kMaxL, true));
+    attr = true;
+  }
+  k_eig<<<Q, eig_threads(L), eig_smem(L, weights_mode), st>>>(
+      ctx->s.gram, nch, sum ? kEigParts : nch, cb.d_facets, L, theta_bar, cb.d_mubar, (float)(1.0 / cb.zeta),
+      ctx->s.nucM, theta_bar_out, weights_mode ? 1 : 0, 40);
   note_launches(1);
 }
 
