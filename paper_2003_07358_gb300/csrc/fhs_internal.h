@@ -130,7 +130,7 @@ struct Scratch {
   float* img = nullptr;      size_t img_elems = 0;      // [L][n1][n2]
   float* img2 = nullptr;
   float2* vis = nullptr;     size_t vis_elems = 0;      // [n_vis]
-  float2* vis2 = nullptr;                               // [n_vis] forward-backward iterate (preconditioning)
+  float2* vis2 = nullptr;                               // [n_vis] two floats per visibility (preconditioning)
   double* red = nullptr;     size_t red_elems = 0;      // reduction partials
   double* red_host = nullptr;                           // pinned host copy
   double* gram = nullptr;    size_t gram_elems = 0;     // nuclear Gram partials (FP64)
@@ -239,7 +239,8 @@ void launch_grid_dde_count(const Cube& cb, cudaStream_t st);
 void launch_l2ball_partials(const Cube& cb, const float2* z, const float2* y, float2* d,
                             double* partials, int nparts, cudaStream_t st);
 void launch_l2ball_scale(const Cube& cb, const float2* d, const float* scale, float2* v, cudaStream_t st);
-void launch_precond_duals(const Cube& cb, float2* d, float2* t, float* blk_scale, double* partials, cudaStream_t st);
+void launch_precond_duals(const Cube& cb, float2* d, float2* t, const float* blk_scale, const double* dnorm,
+                          double* partials, cudaStream_t st);
 void launch_vis_scale(float2* v, const float* f, int64_t n, bool divide, cudaStream_t st);
 void launch_vis_gather(const int64_t* perm, int64_t n, const float2* in, float2* out, cudaStream_t st);
 void launch_vis_scatter(const int64_t* perm, int64_t n, const float2* in, float2* out, cudaStream_t st);

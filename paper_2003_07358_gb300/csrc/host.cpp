@@ -876,7 +876,7 @@ void pdfb_iteration_cube(fhs_ctx* ctx, int c, const fhs_iterate& a) {
     const float* gscale = ctx->s.blk_scale;
     if (cb.n_sub > 0) {
       // U-metric projections by forward-backward sub-iterations; s.vis <- v = U (d - w)
-      launch_precond_duals(cb, ctx->s.vis, ctx->s.vis2, ctx->s.blk_scale, ctx->s.red, st);
+      launch_precond_duals(cb, ctx->s.vis, ctx->s.vis2, ctx->s.blk_scale, stat + 2 * pp, ctx->s.red, st);
       check_launch("preconditioned duals");
       gscale = nullptr;
     }

@@ -15,6 +15,7 @@
 
 #include <algorithm>
 
+#include "ffloat.cuh"
 #include "fhs_internal.h"
 
 namespace fhs {
@@ -24,13 +25,6 @@ constexpr int kGramSub = 64;       // pixels staged in shared memory at a time
 
 __device__ __forceinline__ float facet_weight(const NucFacet& f, const float* __restrict__ win, int rr, int cc) {
   return win[f.wy_off + rr] * win[f.wx_off + cc];
-}
-
-// Error-free transformation a + b = s + e (Knuth TwoSum), no contraction.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
 // Partial Gram of chunk blockIdx.x of facet blockIdx.y, accumulated in
@@ -210,49 +204,6 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
 // would lose: the sums of the chunk partials, m_j, and, for the weights, the
 // eigenvalues themselves (Rayleigh quotients, whose error is second order in the
 // eigenvectors').
-struct ff {
-  float h, l;
-};
-
-__device__ __forceinline__ ff ff_of(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
-}
-__device__ __forceinline__ double ff_val(ff a) { return (double)a.h + (double)a.l; }
-
-// c a + s b.
-__device__ __forceinline__ ff ff_lin(ff c, ff a, ff s, ff b) {
-  const float p = __fmul_rn(c.h, a.h), q = __fmul_rn(s.h, b.h);
-  float pe = __fmaf_rn(c.h, a.h, -p), qe = __fmaf_rn(s.h, b.h, -q);
-  pe = __fmaf_rn(c.l, a.h, __fmaf_rn(c.h, a.l, pe));
-  qe = __fmaf_rn(s.l, b.h, __fmaf_rn(s.h, b.l, qe));
-  float t, e;
-  two_sum(p, q, t, e);
-  e = __fadd_rn(e, __fadd_rn(pe, qe));
-  const float h = __fadd_rn(t, e);
-  return {h, __fsub_rn(e, __fsub_rn(h, t))};
-}
-
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-  const float p = __fmul_rn(a.h, b.h);
-  const float e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
-  const float h = __fadd_rn(p, e);
-  return {h, __fsub_rn(e, __fsub_rn(h, p))};
-}
-
-// u^-1/2 (u > 0): one Newton step from the FP32 value with the residual 1 - u y^2 formed
-// as a pair.
-__device__ __forceinline__ ff ff_rsqrt(ff u) {
-  const float y = rsqrtf(u.h);
-  const float q = __fmul_rn(y, y), qe = __fmaf_rn(y, y, -q);
-  const float w = __fmul_rn(u.h, q);
-  const float we = __fmaf_rn(u.l, q, __fmaf_rn(u.h, qe, __fmaf_rn(u.h, q, -w)));
-  const float r = __fsub_rn(__fsub_rn(1.f, w), we);
-  const float cor = y * fmaf(0.375f * r, r, 0.5f * r);
-  const float h = __fadd_rn(y, cor);
-  return {h, __fsub_rn(cor, __fsub_rn(h, y))};
-}
-
 // Plane rotation (c, s) that annihilates gpr of [[gpp, gpr], [gpr, grr]] up to the FP32
 // accuracy of its tangent (the remainder is annihilated in the next sweep); c and s are
 // float pairs with c^2 + s^2 = 1 to about 2^-46.  False (identity) when gpr is below the
