@@ -14,56 +14,6 @@
 // for 64-bit accesses).  Forward rows read only the n2 image columns (the others
 // are zero); inverse rows store only those columns.
 
-// exp(-2 pi i j / 32), j < 16
-__constant__ float2 c_w32[16] = {
-    {1.f, 0.f},                          {9.807852804e-01f, -1.950903220e-01f},
-    {9.238795325e-01f, -3.826834324e-01f}, {8.314696123e-01f, -5.555702330e-01f},
-    {7.071067812e-01f, -7.071067812e-01f}, {5.555702330e-01f, -8.314696123e-01f},
-    {3.826834324e-01f, -9.238795325e-01f}, {1.950903220e-01f, -9.807852804e-01f},
-    {0.f, -1.f},                           {-1.950903220e-01f, -9.807852804e-01f},
-    {-3.826834324e-01f, -9.238795325e-01f}, {-5.555702330e-01f, -8.314696123e-01f},
-    {-7.071067812e-01f, -7.071067812e-01f}, {-8.314696123e-01f, -5.555702330e-01f},
-    {-9.238795325e-01f, -3.826834324e-01f}, {-9.807852804e-01f, -1.950903220e-01f},
-};
-
-// In-place R-point DFT of v (natural order in and out), radix-2 decimation in time
-// down to the 8-, 4- and 2-point kernels; sign exp(-2 pi i / R), INV flips it.
-template <int R, bool INV>
-__device__ __forceinline__ void rdft(float2* v) {
-  if constexpr (R == 2) {
-    dft2(v[0], v[1]);
-  } else if constexpr (R == 4) {
-    dft4(v[0], v[1], v[2], v[3], INV);
-  } else if constexpr (R == 8) {
-    dft8(v, INV);
-  } else {
-    constexpr int H = R / 2;
-    float2 e[H], o[H];
-#pragma unroll
-    for (int k = 0; k < H; ++k) {
-      e[k] = v[2 * k];
-      o[k] = v[2 * k + 1];
-    }
-    rdft<H, INV>(e);
-    rdft<H, INV>(o);
-#pragma unroll
-    for (int k = 0; k < H; ++k) {
-      float2 t;
-      if (k == 0) {
-        t = o[0];
-      } else if (2 * k == H) {               // w = -i (forward), +i (inverse)
-        t = INV ? make_float2(-o[k].y, o[k].x) : make_float2(o[k].y, -o[k].x);
-      } else {
-        float2 w = c_w32[k * (32 / R)];
-        if (INV) w.y = -w.y;
-        t = cmul(o[k], w);
-      }
-      v[k] = cadd(e[k], t);
-      v[k + H] = csub(e[k], t);
-    }
-  }
-}
-
 template <int N> struct RegRowCfg;
 template <> struct RegRowCfg<2048> { static constexpr int R1 = 16, R2 = 16, R3 = 8; };
 template <> struct RegRowCfg<4096> { static constexpr int R1 = 16, R2 = 16, R3 = 16; };

@@ -209,6 +209,11 @@ void launch_fft_adjoint(fhs_ctx* ctx, const Cube& cb, float2* grid, float* out, 
                         bool accumulate, cudaStream_t st);
 void launch_fft_forward_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float2* grid, cudaStream_t st);
 bool fft_forward_packed(const Cube& cb);
+// two-for-one transforms of grid sides 2^a and 3 2^a with one-pass columns (fft_mid.cu)
+bool fft_mid_supported(const Cube& cb);
+void launch_fft_forward_mid(fhs_ctx* ctx, const Cube& cb, const float* x, float2* grid, cudaStream_t st);
+void launch_fft_adjoint_mid(fhs_ctx* ctx, const Cube& cb, const float2* grid, float* out, const float* eta,
+                            bool accumulate, cudaStream_t st);
 void launch_fft_adjoint_fast(fhs_ctx* ctx, const Cube& cb, float2* grid, float* out, const float* eta,
                              bool accumulate, cudaStream_t st);
 void launch_degrid(const Cube& cb, const float2* grid, float2* out, bool tiled, cudaStream_t st);

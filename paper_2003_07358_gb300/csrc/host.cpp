@@ -597,7 +597,7 @@ void alloc_scratch(fhs_ctx* ctx) {
   s.grid = dalloc<float2>(grid); s.grid_elems = grid;
   size_t pack = 0;
   for (const Cube& cb : ctx->cubes)
-    if (fft_forward_packed(cb)) pack = std::max(pack, (size_t)cb.L * cb.K1 * (cb.n2 / 2));
+    if (fft_forward_packed(cb) || fft_mid_supported(cb)) pack = std::max(pack, (size_t)cb.L * cb.K1 * (cb.n2 / 2));
   if (pack) s.pack = dalloc<float2>(pack);
   s.coef_elems = coef;          // allocated on first use of the plain path (ensure_coef)
   s.ll1 = dalloc<float>(ll1);
@@ -691,7 +691,7 @@ bool make_lane(fhs_ctx* ctx) {
   }
   size_t pack = 0;
   for (const Cube& cb : ctx->cubes)
-    if (fft_forward_packed(cb)) pack = std::max(pack, (size_t)cb.L * cb.K1 * (cb.n2 / 2));
+    if (fft_forward_packed(cb) || fft_mid_supported(cb)) pack = std::max(pack, (size_t)cb.L * cb.K1 * (cb.n2 / 2));
   get(b.grid, a.grid_elems, sizeof(float2));
   get(b.pack, pack, sizeof(float2));
   get(b.coef, a.coef_elems, sizeof(float));

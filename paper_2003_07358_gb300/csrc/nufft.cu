@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "ffloat.cuh"
+#include "fft_core.cuh"
 #include "fhs_internal.h"
 
 namespace fhs {
@@ -37,50 +38,7 @@ __constant__ KbPoly c_kb;
 
 cudaError_t upload_kb_poly(const KbPoly& p) { return cudaMemcpyToSymbol(c_kb, &p, sizeof(p)); }
 
-// ------------------------------------------------------------------ complex
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }
-
-// ----------------------------------------------------------- R-point DFTs
-// Forward sign exp(-2 pi i / R); `inv` flips the sign (unnormalised).
-__device__ __forceinline__ void dft2(float2& a, float2& b) {
-  float2 t = a;
-  a = cadd(t, b);
-  b = csub(t, b);
-}
-
-__device__ __forceinline__ void dft4(float2& x0, float2& x1, float2& x2, float2& x3, bool inv) {
-  float2 a0 = cadd(x0, x2), a1 = csub(x0, x2), a2 = cadd(x1, x3), a3 = csub(x1, x3);
-  // -i * a3 = (a3.y, -a3.x)
-  float2 mia3 = inv ? make_float2(-a3.y, a3.x) : make_float2(a3.y, -a3.x);
-  x0 = cadd(a0, a2);
-  x2 = csub(a0, a2);
-  x1 = cadd(a1, mia3);
-  x3 = csub(a1, mia3);
-}
-
-__device__ __forceinline__ void dft8(float2* v, bool inv) {
-  float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
-  float2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-  dft4(e0, e1, e2, e3, inv);
-  dft4(o0, o1, o2, o3, inv);
-  const float c = 0.70710678118654752440f;
-  float sg = inv ? 1.f : -1.f;
-  // w^1 = (c, sg c), w^2 = (0, sg), w^3 = (-c, sg c)
-  float2 t1 = cmul(o1, make_float2(c, sg * c));
-  float2 t2 = cmul(o2, make_float2(0.f, sg));
-  float2 t3 = cmul(o3, make_float2(-c, sg * c));
-  v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
-  v[1] = cadd(e1, t1); v[5] = csub(e1, t1);
-  v[2] = cadd(e2, t2); v[6] = csub(e2, t2);
-  v[3] = cadd(e3, t3); v[7] = csub(e3, t3);
-}
 
 template <int R>
 __device__ __forceinline__ void dftR(float2* v, bool inv) {
@@ -374,17 +332,6 @@ static void col_n(const Cube& cb, float2* grid, int ngroups, int gmul, int istri
 // context's table (Kmax is a multiple of every grid side).  Rows: one CTA per image
 // row; columns: one CTA per W adjacent grid columns, the whole column in one pass, so
 // the grid rows stay in natural order (N1c = K1, N2c = 1).
-__device__ __forceinline__ void dft3(float2& x0, float2& x1, float2& x2, bool inv) {
-  const float h = 0.866025403784438646764f;                  // sqrt(3) / 2
-  const float2 t = cadd(x1, x2), d = csub(x1, x2);
-  const float2 m = make_float2(fmaf(-0.5f, t.x, x0.x), fmaf(-0.5f, t.y, x0.y));
-  const float2 ihd = make_float2(-h * d.y, h * d.x);         // i (sqrt(3) / 2) (x1 - x2)
-  x0 = cadd(x0, t);
-  // forward: y1 = m - i h d, y2 = m + i h d; the inverse flips the sign of i
-  x1 = inv ? cadd(m, ihd) : csub(m, ihd);
-  x2 = inv ? csub(m, ihd) : cadd(m, ihd);
-}
-
 template <int R>
 __device__ __forceinline__ void gen_pass(const float2* __restrict__ src, float2* __restrict__ dst, int N, int W,
                                          int Ns, const float2* __restrict__ tw, int Kmax, bool inv) {
@@ -526,6 +473,10 @@ static void launch_fft_adjoint_gen(fhs_ctx* ctx, const Cube& cb, float2* grid, f
 }
 
 void launch_fft_forward(fhs_ctx* ctx, const Cube& cb, const float* x, float2* grid, cudaStream_t st) {
+  if (ctx->path == FHS_PATH_FAST && ctx->s.pack && fft_mid_supported(cb)) {
+    launch_fft_forward_mid(ctx, cb, x, grid, st);
+    return;
+  }
   if (!cb.pow2) {
     launch_fft_forward_gen(ctx, cb, x, grid, st);
     return;
@@ -545,6 +496,10 @@ void launch_fft_forward(fhs_ctx* ctx, const Cube& cb, const float* x, float2* gr
 
 void launch_fft_adjoint(fhs_ctx* ctx, const Cube& cb, float2* grid, float* out, const float* eta, bool accumulate,
                         cudaStream_t st) {
+  if (ctx->path == FHS_PATH_FAST && ctx->s.pack && fft_mid_supported(cb)) {
+    launch_fft_adjoint_mid(ctx, cb, grid, out, eta, accumulate, st);
+    return;
+  }
   if (!cb.pow2) {
     launch_fft_adjoint_gen(ctx, cb, grid, out, eta, accumulate, st);
     return;
