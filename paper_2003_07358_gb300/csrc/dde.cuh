@@ -10,10 +10,19 @@
 // (row r, column c; kernel index j1, j2 in [0, 2R]; taps a = r - j1, b = c - j2):
 //   de-gridding  u_m = sum_{j1,j2} K[j1][j2] sum_a w_r[a] sum_b w_c[b] x[j1 + a][j2 + b]
 //   gridding     x[r][c] += sum_b w_c[b] sum_a w_r[a] conj(K[r - a][c - b]) v_m
-// Both are separable passes through per-warp shared-memory scratch: one warp works on
-// one visibility at a time (its lanes split the footprint cells, the row and column
-// passes and the kernel coefficients), so the kernel coefficients and the grid window
-// are read coalesced once per visibility.
+// Both are separable passes of which each lane of a half-warp runs one row or column in
+// registers (a polynomial product: F x 7 or SD x 7 complex FMAs with no shared-memory
+// operand), with one transposition through shared memory in between; a warp works on two
+// visibilities at a time.  De-gridding: lane c takes column c of the window (its loads
+// coalesce along the row), then lane j1 row j1 of the intermediate and of the kernel.
+// Gridding: lane j1 takes row j1 of the kernel, then lane c column c of the footprint, so a
+// row's atomics fall on consecutive cells.  Lanes 0..13 of a half hold the polynomial of
+// one Kaiser-Bessel tap each and exchange the 14 weights by shuffles.
+// (One visibility per warp with every pass reading its operands from shared memory took
+// 2.04 ms to de-grid and 4.03 to 4.13 ms to grid 2.1 M visibilities of 16 channels of 1024^2
+// with 9 x 9 kernels, about 700 instructions a visibility; this form takes 0.83 and
+// 1.64 ms, bound by issue: 126 FMAs a pass and lane, and for the gridder 30 conversions and
+// atomics.)
 //
 // Gridding keeps the scheme of k_grid: one CTA per (grid tile, channel) owns the tile's
 // cells in shared memory and adds, in 32-bit fixed point with integer atomics (order-
@@ -21,88 +30,96 @@
 // Visibilities are bucketed by the tile of their first tap, and a footprint (F <= 15 <
 // tile side) reaches only the 3 x 3 neighbouring tiles, so a CTA scans those buckets,
 // keeps (by warp ballot) the visibilities whose footprint meets its tile, and processes
-// them one by one.  The scale S = 2^e of a tile satisfies n_c m S < 2^30 with n_c the
-// largest number of extended footprints covering one of its cells (counted once per
-// kernel set, MODE 1) and m = max over the contributing visibilities of
-// max(|Re v|, |Im v|) * sum_j (|Re K_j| + |Im K_j|), a bound of every tap value
-// |Re|, |Im| of conj(g_m[k]) v_m (Kaiser-Bessel weights are at most 1).
+// them two by two.  The scale S = 2^e of a tile satisfies C m S < 2^30 with C the largest sum
+// over one of its cells of the extended weights covering it, sum_j (|Re K_j| + |Im K_j|)
+// phi phi (summed once per kernel set, MODE 1), and m = max over the contributing
+// visibilities of max(|Re v|, |Im v|).
 
 namespace fhs {
 
 constexpr int kDdeThreads = 256;
 constexpr int kDdeWarps = kDdeThreads / 32;
 
-// Per-warp scratch; WIN: with the grid window (de-gridding only).
-template <int R, bool WIN>
-struct DdeScratch {
-  static constexpr int SD = 2 * R + 1;
-  static constexpr int F = kTaps + 2 * R;
-  float2 win[WIN ? F * F : 1];   // de-gridding: the grid window of the footprint
-  float2 mid[F * SD];            // de-gridding: column pass; gridding: H[r][j2]
-  float2 ker[SD * SD];           // de-gridding: K; gridding: conj(K) v S
-  float w[2 * kTaps];            // row weights, then column weights
-};
+constexpr int kDdeLd = 17;            // row pitch of the transposition (float2): odd, over 15 columns
 
-// Row and column Kaiser-Bessel weights of (xr, xc) into s.w (lanes 0..13).
-template <class Scr>
-__device__ __forceinline__ void dde_weights(Scr& s, float xr, float xc, int lane) {
-  if (lane < kTaps) s.w[lane] = kb_tap(lane, xr);
-  else if (lane < 2 * kTaps) s.w[lane] = kb_tap(lane - kTaps, xc);
+// The polynomial of the lane's tap (row taps on lanes 0..6 of a half, column taps on 7..13).
+struct DdeTap {
+  float c[kPolyDeg + 1];
+};
+__device__ __forceinline__ DdeTap dde_tap_poly(int lane) {
+  const int j = lane & 15, t = j < kTaps ? j : (j < 2 * kTaps ? j - kTaps : 0);
+  DdeTap p;
+#pragma unroll
+  for (int d = 0; d <= kPolyDeg; ++d) p.c[d] = c_kb.c[t][d];
+  return p;
 }
 
-// u_m of one visibility by the whole warp (same value returned on every lane).
-template <int R>
-__device__ __forceinline__ float2 dde_degrid_one(const float2* __restrict__ gl, float2 uvm,
-                                                 const float2* __restrict__ Km, const VisGeom& vg,
-                                                 DdeScratch<R, true>& s, int lane) {
-  constexpr int SD = 2 * R + 1, F = kTaps + 2 * R;
-  float xr, xc;
-  const int kr = kb_first(uvm.y, vg.tc.hi_r, vg.tc.lo_r, xr);
-  const int kc = kb_first(uvm.x, vg.tc.hi_c, vg.tc.lo_c, xc);
-  dde_weights(s, xr, xc, lane);
-  for (int k = lane; k < SD * SD; k += 32) s.ker[k] = Km[k];
-  for (int k = lane; k < F * F; k += 32) {
-    const int r = k / F, c = k - r * F;
-    const int row = phys_row2(wrap1(kr - R + r, vg), vg);
-    s.win[k] = gl[(size_t)row * vg.K2 + wrap2(kc - R + c, vg)];
-  }
-  __syncwarp();
-  float wc[kTaps], wr[kTaps];
+// Row and column Kaiser-Bessel weights of the half-warp's visibility on each of its lanes.
+__device__ __forceinline__ void dde_weights(const DdeTap& p, float xr, float xc, int lane, float* wr, float* wc) {
+  const float x = (lane & 15) < kTaps ? xr : xc;
+  float w = p.c[kPolyDeg];
+#pragma unroll
+  for (int d = kPolyDeg - 1; d >= 0; --d) w = fmaf(w, x, p.c[d]);
+  const int h = lane & 16;
 #pragma unroll
   for (int b = 0; b < kTaps; ++b) {
-    wr[b] = s.w[b];
-    wc[b] = s.w[kTaps + b];
+    wr[b] = __shfl_sync(0xffffffffu, w, h + b);
+    wc[b] = __shfl_sync(0xffffffffu, w, h + kTaps + b);
   }
-  // column pass: mid[r][j2] = sum_b w_c[b] win[r][j2 + b]
-  for (int k = lane; k < F * SD; k += 32) {
-    const int r = k / SD, j2 = k - r * SD;
-    const float2* p = s.win + r * F + j2;
-    float2 a = make_float2(0.f, 0.f);
+}
+
+// u_m of the visibility of each half-warp (the value is returned on the half's lanes); tr:
+// the half's [SD][kDdeLd] scratch.
+template <int R>
+__device__ __forceinline__ float2 dde_degrid_half(const float2* __restrict__ gl, float2 uvm,
+                                                  const float2* __restrict__ Km, const VisGeom& vg, const DdeTap& tap,
+                                                  float2* tr, int lane) {
+  constexpr int SD = 2 * R + 1, F = kTaps + 2 * R;
+  const int j = lane & 15;
+  float xr, xc, wr[kTaps], wc[kTaps];
+  const int kr = kb_first(uvm.y, vg.tc.hi_r, vg.tc.lo_r, xr);
+  const int kc = kb_first(uvm.x, vg.tc.hi_c, vg.tc.lo_c, xc);
+  // the lane's column of the window and its row of the kernel, all loads in flight
+  const float2* col = gl + wrap2(kc - R + min(j, F - 1), vg);
+  float2 x[F], K[SD];
 #pragma unroll
-    for (int b = 0; b < kTaps; ++b) {
-      a.x = fmaf(wc[b], p[b].x, a.x);
-      a.y = fmaf(wc[b], p[b].y, a.y);
-    }
-    s.mid[k] = a;
-  }
-  __syncwarp();
-  // row pass and the kernel: u = sum_j K[j] sum_a w_r[a] mid[j1 + a][j2]
-  float2 u = make_float2(0.f, 0.f);
-  for (int k = lane; k < SD * SD; k += 32) {
-    const int j1 = k / SD, j2 = k - j1 * SD;
-    const float2* p = s.mid + j1 * SD + j2;
-    float2 I = make_float2(0.f, 0.f);
+  for (int r = 0; r < F; ++r) x[r] = __ldg(col + (size_t)phys_row2(wrap1(kr - R + r, vg), vg) * vg.K2);
+  const float2* Kr = Km + min(j, SD - 1) * SD;
+#pragma unroll
+  for (int j2 = 0; j2 < SD; ++j2) K[j2] = __ldg(Kr + j2);
+  dde_weights(tap, xr, xc, lane, wr, wc);
+  // row pass: mid[j1][c] = sum_a w_r[a] x[j1 + a][c]
+#pragma unroll
+  for (int j1 = 0; j1 < SD; ++j1) {
+    float2 m = make_float2(0.f, 0.f);
 #pragma unroll
     for (int a = 0; a < kTaps; ++a) {
-      I.x = fmaf(wr[a], p[a * SD].x, I.x);
-      I.y = fmaf(wr[a], p[a * SD].y, I.y);
+      m.x = fmaf(wr[a], x[j1 + a].x, m.x);
+      m.y = fmaf(wr[a], x[j1 + a].y, m.y);
     }
-    const float2 K = s.ker[k];
-    u.x = fmaf(K.x, I.x, fmaf(-K.y, I.y, u.x));
-    u.y = fmaf(K.x, I.y, fmaf(K.y, I.x, u.y));
+    if (j < F) tr[j1 * kDdeLd + j] = m;
+  }
+  __syncwarp();
+  // column pass and the kernel row: u = sum_j2 K[j1][j2] sum_b w_c[b] mid[j1][j2 + b]
+  float2 u = make_float2(0.f, 0.f);
+  if (j < SD) {
+    float2 m[F];
+#pragma unroll
+    for (int c = 0; c < F; ++c) m[c] = tr[j * kDdeLd + c];
+#pragma unroll
+    for (int j2 = 0; j2 < SD; ++j2) {
+      float2 I = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int b = 0; b < kTaps; ++b) {
+        I.x = fmaf(wc[b], m[j2 + b].x, I.x);
+        I.y = fmaf(wc[b], m[j2 + b].y, I.y);
+      }
+      u.x = fmaf(K[j2].x, I.x, fmaf(-K[j2].y, I.y, u.x));
+      u.y = fmaf(K[j2].x, I.y, fmaf(K[j2].y, I.x, u.y));
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = 8; o > 0; o >>= 1) {
     u.x += __shfl_xor_sync(0xffffffffu, u.x, o);
     u.y += __shfl_xor_sync(0xffffffffu, u.y, o);
   }
@@ -112,8 +129,8 @@ __device__ __forceinline__ float2 dde_degrid_one(const float2* __restrict__ gl, 
 
 // MODE 0: out[i] = u_i.  MODE 1: the PDFB data step of k_degrid_pdfb (z = v + 2u - u_prev,
 // d = z - y, u_prev <- u, per-block FP64 partial sums).  CTA = 256 consecutive
-// visibilities of channel blockIdx.y; warp w computes those of lanes 32 w .. 32 w + 31
-// one by one, and lane t keeps the t-th result for the per-visibility epilogue.
+// visibilities of channel blockIdx.y; half h of warp w computes those of lanes
+// 32 w + 16 h .. + 15 one by one, and each lane keeps its own for the per-visibility epilogue.
 template <int R, int MODE>
 __global__ void __launch_bounds__(kDdeThreads) k_degrid_dde(const float2* __restrict__ grid,
                                                             const float2* __restrict__ uv,
@@ -125,18 +142,21 @@ __global__ void __launch_bounds__(kDdeThreads) k_degrid_dde(const float2* __rest
                                                             const uint8_t* __restrict__ blk, int B,
                                                             double* __restrict__ partials, int nparts) {
   constexpr int SD = 2 * R + 1;
-  __shared__ DdeScratch<R, true> scr[kDdeWarps];
+  __shared__ float2 scr[2 * kDdeWarps][SD * kDdeLd];
   __shared__ double sred[kDdeWarps * 2 * kMaxB];
   const int l = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t end = vis_off[l + 1];
   const int64_t wbase = vis_off[l] + (int64_t)blockIdx.x * kDdeThreads + wid * 32;
   const float2* gl = grid + (size_t)l * vg.K1 * vg.K2;
   float2 mine = make_float2(0.f, 0.f);
-  for (int t = 0; t < 32; ++t) {
-    const int64_t i = wbase + t;
-    if (i >= end) break;                               // warp-uniform
-    const float2 u = dde_degrid_one<R>(gl, uv[i], kern + (size_t)kidx[i] * SD * SD, vg, scr[wid], lane);
-    if (lane == t) mine = u;
+  const DdeTap tap = dde_tap_poly(lane);
+#pragma unroll 1
+  for (int t = 0; t < 16; ++t) {
+    if (wbase + t >= end) break;                       // warp-uniform
+    const int64_t i = min(wbase + (lane & 16) + t, end - 1);   // past the end: repeated, not kept
+    const float2 u = dde_degrid_half<R>(gl, uv[i], kern + (size_t)kidx[i] * SD * SD, vg, tap,
+                                        scr[2 * wid + (lane >> 4)], lane);
+    if ((lane & 15) == t) mine = u;
   }
   const int64_t i = wbase + lane;
   const bool valid = i < end;
@@ -144,20 +164,18 @@ __global__ void __launch_bounds__(kDdeThreads) k_degrid_dde(const float2* __rest
     if (valid) out[i] = mine;
     return;
   }
-  double v0 = 0.0, v1 = 0.0;
+  float2 d = make_float2(0.f, 0.f), yy = d;
   int b = 0;
   if (valid) {
-    const float2 yy = y[i], vv = v[i], up = u_prev[i];
+    const float2 vv = v[i], up = u_prev[i];
+    yy = y[i];
     const float2 z = make_float2(vv.x + 2.f * mine.x - up.x, vv.y + 2.f * mine.y - up.y);
-    const float2 d = make_float2(z.x - yy.x, z.y - yy.y);
+    d = make_float2(z.x - yy.x, z.y - yy.y);
     out[i] = d;
     u_prev[i] = mine;
     b = blk[i];
-    v0 = (double)d.x * d.x + (double)d.y * d.y;
-    const double rx = (double)yy.x - mine.x, ry = (double)yy.y - mine.y;
-    v1 = rx * rx + ry * ry;
   }
-  block_partials<kDdeWarps>(v0, v1, b, valid, B, sred, partials + ((size_t)l * nparts + blockIdx.x) * 2 * B);
+  block_partials<kDdeWarps>(d, yy, mine, b, valid, B, sred, partials + ((size_t)l * nparts + blockIdx.x) * 2 * B);
 }
 
 // Local start (mod K) of a footprint that starts at absolute cell k, relative to tile
@@ -170,66 +188,75 @@ __device__ __forceinline__ int dde_local(int k, int t0, int K, int pw) {
 // Whether a footprint of F cells starting at local offset d (mod K) meets [0, T).
 __device__ __forceinline__ bool dde_meets(int d, int F, int T, int K) { return d < T || d + F - 1 >= K; }
 
-// Adds the footprint cells of one visibility that lie in the tile (MODE 0: fixed-point
-// values of conj(g) v S, with vS = v S; MODE 1: one count per cell), by the whole warp.
+// Adds the footprint cells of each half-warp's visibility that lie in the tile: fixed-point
+// values of conj(g) v S, with vS = v S (`on` false: nothing is added); tr: the half's
+// [SD][kDdeLd] scratch.  MODE 1: the weights' bound (|Re K| + |Im K|) phi phi vS.x instead,
+// rounded up.
 template <int R, int MODE>
-__device__ __forceinline__ void dde_grid_one(int* are, int* aim, int TP, int T, int dr, int dc, float xr, float xc,
-                                             float2 vS, const float2* __restrict__ Km, const VisGeom& vg,
-                                             DdeScratch<R, false>& s, int lane) {
+__device__ __forceinline__ void dde_grid_half(int* are, int* aim, int TP, int T, int dr, int dc, float xr, float xc,
+                                              float2 vS, const float2* __restrict__ Km, bool on, const VisGeom& vg,
+                                              const DdeTap& tap, float2* tr, int lane) {
   constexpr int SD = 2 * R + 1, F = kTaps + 2 * R;
+  const int j = lane & 15;
+  float wr[kTaps], wc[kTaps];
+  const float2* Kr = Km + min(j, SD - 1) * SD;
+  float2 Z[SD];
+#pragma unroll
+  for (int j2 = 0; j2 < SD; ++j2) {
+    const float2 K = __ldg(Kr + j2);
+    Z[j2] = MODE == 1 ? make_float2((fabsf(K.x) + fabsf(K.y)) * vS.x, 0.f)
+                      : make_float2(fmaf(K.x, vS.x, K.y * vS.y), fmaf(K.x, vS.y, -K.y * vS.x));   // conj(K) v S
+  }
+  dde_weights(tap, xr, xc, lane, wr, wc);
   if (MODE == 1) {
-    for (int k = lane; k < F * F; k += 32) {
-      const int r = k / F, c = k - r * F;
-      const int lr = wrap1(dr + r, vg), lc = wrap2(dc + c, vg);
-      if (lr < T && lc < T) atomicAdd(are + lr * TP + lc, 1);
-    }
-    return;
-  }
-  dde_weights(s, xr, xc, lane);
-  for (int k = lane; k < SD * SD; k += 32) {
-    const float2 K = Km[k];
-    s.ker[k] = make_float2(fmaf(K.x, vS.x, K.y * vS.y), fmaf(K.x, vS.y, -K.y * vS.x));   // conj(K) v S
-  }
-  __syncwarp();
-  float wc[kTaps], wr[kTaps];
 #pragma unroll
-  for (int b = 0; b < kTaps; ++b) {
-    wr[b] = s.w[b];
-    wc[b] = s.w[kTaps + b];
+    for (int b = 0; b < kTaps; ++b) {
+      wr[b] = fabsf(wr[b]);
+      wc[b] = fabsf(wc[b]);
+    }
   }
-  // row pass: H[r][j2] = sum_a w_r[a] Z[r - a][j2]
-  for (int k = lane; k < F * SD; k += 32) {
-    const int r = k / SD, j2 = k - r * SD;
+  // column pass: H[j1][c] = sum_b w_c[b] Z[j1][c - b]
+#pragma unroll
+  for (int c = 0; c < F; ++c) {
     float2 h = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int a = 0; a < kTaps; ++a) {
-      const int j1 = r - a;
-      if (j1 >= 0 && j1 < SD) {
-        const float2 z = s.ker[j1 * SD + j2];
-        h.x = fmaf(wr[a], z.x, h.x);
-        h.y = fmaf(wr[a], z.y, h.y);
-      }
-    }
-    s.mid[k] = h;
-  }
-  __syncwarp();
-  // column pass and the tile's cells: x[r][c] = sum_b w_c[b] H[r][c - b]
-  for (int k = lane; k < F * F; k += 32) {
-    const int r = k / F, c = k - r * F;
-    const int lr = wrap1(dr + r, vg), lc = wrap2(dc + c, vg);
-    if (lr >= T || lc >= T) continue;
-    float2 x = make_float2(0.f, 0.f);
 #pragma unroll
     for (int b = 0; b < kTaps; ++b) {
       const int j2 = c - b;
       if (j2 >= 0 && j2 < SD) {
-        const float2 h = s.mid[r * SD + j2];
-        x.x = fmaf(wc[b], h.x, x.x);
-        x.y = fmaf(wc[b], h.y, x.y);
+        h.x = fmaf(wc[b], Z[j2].x, h.x);
+        h.y = fmaf(wc[b], Z[j2].y, h.y);
       }
     }
-    atomicAdd(are + lr * TP + lc, __float2int_rn(x.x));
-    atomicAdd(aim + lr * TP + lc, __float2int_rn(x.y));
+    if (j < SD) tr[j * kDdeLd + c] = h;
+  }
+  __syncwarp();
+  // row pass and the tile's cells of column c: x[r][c] = sum_a w_r[a] H[r - a][c]
+  const int lc = wrap2(dc + j, vg);
+  if (on && j < F && lc < T) {
+    float2 H[SD];
+#pragma unroll
+    for (int j1 = 0; j1 < SD; ++j1) H[j1] = tr[j1 * kDdeLd + j];
+#pragma unroll
+    for (int r = 0; r < F; ++r) {
+      float2 x = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int a = 0; a < kTaps; ++a) {
+        const int j1 = r - a;
+        if (j1 >= 0 && j1 < SD) {
+          x.x = fmaf(wr[a], H[j1].x, x.x);
+          x.y = fmaf(wr[a], H[j1].y, x.y);
+        }
+      }
+      const int lr = wrap1(dr + r, vg);
+      if (lr < T) {
+        if (MODE == 1) {
+          atomicAdd(are + lr * TP + lc, __float2int_ru(x.x));
+        } else {
+          atomicAdd(are + lr * TP + lc, __float2int_rn(x.x));
+          atomicAdd(aim + lr * TP + lc, __float2int_rn(x.y));
+        }
+      }
+    }
   }
   __syncwarp();
 }
@@ -247,8 +274,7 @@ __device__ __forceinline__ int dde_source(int s, int tr, int tc, int ntr, int nt
 
 // MODE 0: grid the (block-scaled) values into tile blockIdx.x of channel blockIdx.y and
 // store it (v_write, when set, receives the scaled values of the tile's own
-// visibilities); MODE 1: store the tile's largest footprint count of a cell in
-// ncmax[l][tile].
+// visibilities); MODE 1: store the tile's largest weight sum of a cell in cover[l][tile].
 template <int R, int MODE>
 __global__ void __launch_bounds__(kDdeThreads) k_grid_dde(const float2* __restrict__ vals,
                                                           const float* __restrict__ blk_scale,
@@ -259,11 +285,11 @@ __global__ void __launch_bounds__(kDdeThreads) k_grid_dde(const float2* __restri
                                                           const float* __restrict__ kl1,
                                                           const int32_t* __restrict__ tile_off,
                                                           const int64_t* __restrict__ vis_off,
-                                                          float2* __restrict__ grid, int* __restrict__ ncmax,
+                                                          float2* __restrict__ grid, float* __restrict__ cover,
                                                           VisGeom vg, int T, int ntr, int ntc, int B) {
   constexpr int SD = 2 * R + 1, F = kTaps + 2 * R;
   extern __shared__ __align__(16) int dde_acc[];
-  __shared__ DdeScratch<R, false> scr[kDdeWarps];
+  __shared__ float2 scr[2 * kDdeWarps][SD * kDdeLd];
   __shared__ float sred[kDdeWarps];
   __shared__ int sredi[kDdeWarps];
   const int TP = grid_row_stride(T);
@@ -280,51 +306,61 @@ __global__ void __launch_bounds__(kDdeThreads) k_grid_dde(const float2* __restri
   const int32_t* toff = tile_off + (size_t)l * (ntr * ntc * 4 + 1);
   const int t0r = tr * T, t0c = tc * T;
   float S = 1.f;
-  if (MODE == 0) {
-    // sweep 0: bound m of the tap values of the visibilities meeting the tile; the
-    // tile's own visibilities also get their scaled value written once
-    float m = 0.f;
-    for (int s = 0; s < 9; ++s) {
-      const int src = dde_source(s, tr, tc, ntr, ntc);
-      if (src < 0) continue;
-      const bool own = src == tau;
-      const int beg = toff[src * 4], end = toff[src * 4 + 4];
-      for (int k = beg + (int)threadIdx.x; k < end; k += kDdeThreads) {
-        const int64_t i = vbase + k;
-        float2 val = vals[i];
+  // sweep 0: the largest |v| component of the visibilities meeting the tile (MODE 1: the sum
+  // of their kernels' magnitudes); the tile's own visibilities also get their scaled value
+  // written once
+  float m = 0.f;
+  for (int s = 0; s < 9; ++s) {
+    const int src = dde_source(s, tr, tc, ntr, ntc);
+    if (src < 0) continue;
+    const bool own = src == tau;
+    const int beg = toff[src * 4], end = toff[src * 4 + 4];
+    for (int k = beg + (int)threadIdx.x; k < end; k += kDdeThreads) {
+      const int64_t i = vbase + k;
+      float2 val = make_float2(0.f, 0.f);
+      if (MODE == 0) {
+        val = vals[i];
         if (blk_scale) {
           const float sc = blk_scale[l * B + blk[i]];
           val.x *= sc;
           val.y *= sc;
         }
         if (own && v_write) v_write[i] = val;
-        const float2 w = uv[i];
-        float xr, xc;
-        const int kr = kb_first(w.y, vg.tc.hi_r, vg.tc.lo_r, xr);
-        const int kc = kb_first(w.x, vg.tc.hi_c, vg.tc.lo_c, xc);
-        if (dde_meets(dde_local(kr - R, t0r, vg.K1, vg.pw), F, T, vg.K1) &&
-            dde_meets(dde_local(kc - R, t0c, vg.K2, vg.pw), F, T, vg.K2))
-          m = fmaxf(m, fmaxf(fabsf(val.x), fabsf(val.y)) * kl1[kidx[i]]);
+      }
+      const float2 w = uv[i];
+      float xr, xc;
+      const int kr = kb_first(w.y, vg.tc.hi_r, vg.tc.lo_r, xr);
+      const int kc = kb_first(w.x, vg.tc.hi_c, vg.tc.lo_c, xc);
+      if (dde_meets(dde_local(kr - R, t0r, vg.K1, vg.pw), F, T, vg.K1) &&
+          dde_meets(dde_local(kc - R, t0c, vg.K2, vg.pw), F, T, vg.K2)) {
+        if (MODE == 1) m += kl1[kidx[i]];
+        else m = fmaxf(m, fmaxf(fabsf(val.x), fabsf(val.y)));
       }
     }
+  }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) sred[wid] = m;
-    __syncthreads();
-    m = 0.f;
+  for (int o = 16; o > 0; o >>= 1) {
+    const float e = __shfl_xor_sync(0xffffffffu, m, o);
+    m = MODE == 1 ? m + e : fmaxf(m, e);
+  }
+  if (lane == 0) sred[wid] = m;
+  __syncthreads();
+  m = 0.f;
 #pragma unroll
-    for (int w = 0; w < kDdeWarps; ++w) m = fmaxf(m, sred[w]);
-    const int nc = ncmax[l * ntr * ntc + tau];
-    if (m > 1e-30f && nc > 0) {
-      const float t = 1073741824.f / ((float)nc * (m * 1.0009765625f));
+  for (int w = 0; w < kDdeWarps; ++w) m = MODE == 1 ? m + sred[w] : fmaxf(m, sred[w]);
+  if (MODE == 1) {
+    S = cover_unit(m);
+  } else {
+    const float C = cover[l * ntr * ntc + tau];
+    if (m > 1e-30f && C > 0.f) {
+      const float t = 1073741824.f / (C * (m * 1.0009765625f));
       const int e = (int)((__float_as_uint(t) >> 23) & 0xffu) - 127;   // 2^e <= t
       S = pow2f(max(-120, min(e, 120)));
     }
-  } else {
-    __syncthreads();
   }
   // sweep 1: each warp takes 32 candidates at a time and processes the ones that meet
-  // the tile, one by one
+  // the tile, two by two (one per half-warp)
+  const DdeTap tap = dde_tap_poly(lane);
   for (int s = 0; s < 9; ++s) {
     const int src = dde_source(s, tr, tc, ntr, ntc);
     if (src < 0) continue;
@@ -344,20 +380,23 @@ __global__ void __launch_bounds__(kDdeThreads) k_grid_dde(const float2* __restri
       }
       unsigned mask = __ballot_sync(0xffffffffu, hit);
       while (mask) {
-        const int src_lane = __ffs(mask) - 1;
+        const int first = __ffs(mask) - 1;
         mask &= mask - 1;
-        const int64_t i = vbase + k0 + src_lane;
-        const int drs = __shfl_sync(0xffffffffu, dr, src_lane), dcs = __shfl_sync(0xffffffffu, dc, src_lane);
-        const float xrs = __shfl_sync(0xffffffffu, xr, src_lane), xcs = __shfl_sync(0xffffffffu, xc, src_lane);
-        float2 vS = make_float2(0.f, 0.f);
-        const float2* Km = nullptr;
+        const int second = mask ? __ffs(mask) - 1 : -1;
+        mask &= mask - 1;                                  // (0 stays 0)
+        const bool on = lane < 16 || second >= 0;
+        const int from = lane < 16 || second < 0 ? first : second;
+        const int drs = __shfl_sync(0xffffffffu, dr, from), dcs = __shfl_sync(0xffffffffu, dc, from);
+        const float xrs = __shfl_sync(0xffffffffu, xr, from), xcs = __shfl_sync(0xffffffffu, xc, from);
+        const int64_t i = vbase + k0 + from;
+        float2 vS = make_float2(S, 0.f);
         if (MODE == 0) {
-          float2 val = vals[i];
+          const float2 val = vals[i];
           const float sc = (blk_scale ? blk_scale[l * B + blk[i]] : 1.f) * S;
           vS = make_float2(val.x * sc, val.y * sc);
-          Km = kern + (size_t)kidx[i] * SD * SD;
         }
-        dde_grid_one<R, MODE>(are, aim, TP, T, drs, dcs, xrs, xcs, vS, Km, vg, scr[wid], lane);
+        dde_grid_half<R, MODE>(are, aim, TP, T, drs, dcs, xrs, xcs, vS, kern + (size_t)kidx[i] * SD * SD, on,
+                               vg, tap, scr[2 * wid + (lane >> 4)], lane);
       }
     }
   }
@@ -371,7 +410,7 @@ __global__ void __launch_bounds__(kDdeThreads) k_grid_dde(const float2* __restri
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w = 0; w < kDdeWarps; ++w) mx = max(mx, sredi[w]);
-      ncmax[l * ntr * ntc + tau] = mx;
+      cover[l * ntr * ntc + tau] = __int2float_ru(mx) / S;                 // S: a power of two
     }
     return;
   }
@@ -434,7 +473,7 @@ void launch_grid_dde(const Cube& cb, const float2* vals, const float* blk_scale,
   }                                                                                                               \
   k_grid_dde<RR, 0><<<grd, kDdeThreads, sm, st>>>(vals, blk_scale, v_write, cb.d_uv, cb.d_blk, cb.d_dde_kern,      \
                                                   cb.d_dde_idx, cb.d_dde_l1, cb.d_tile_off, cb.d_vis_off, grid,   \
-                                                  cb.d_dde_ncmax, vg, cb.tile, cb.ntile_r, cb.ntile_c, cb.B)
+                                                  cb.d_dde_cover, vg, cb.tile, cb.ntile_r, cb.ntile_c, cb.B)
   FHS_DDE_SWITCH(cb.dde_R, FHS_L)
 #undef FHS_L
   note_launches(1);
@@ -450,9 +489,9 @@ void launch_grid_dde_count(const Cube& cb, cudaStream_t st) {
     cudaFuncSetAttribute(k_grid_dde<RR, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);               \
     attr[RR] = true;                                                                                              \
   }                                                                                                               \
-  k_grid_dde<RR, 1><<<grd, kDdeThreads, sm, st>>>(nullptr, nullptr, nullptr, cb.d_uv, cb.d_blk, nullptr,           \
-                                                  nullptr, nullptr, cb.d_tile_off, cb.d_vis_off, nullptr,         \
-                                                  cb.d_dde_ncmax, vg, cb.tile, cb.ntile_r, cb.ntile_c, cb.B)
+  k_grid_dde<RR, 1><<<grd, kDdeThreads, sm, st>>>(nullptr, nullptr, nullptr, cb.d_uv, cb.d_blk, cb.d_dde_kern,     \
+                                                  cb.d_dde_idx, cb.d_dde_l1, cb.d_tile_off, cb.d_vis_off, nullptr,         \
+                                                  cb.d_dde_cover, vg, cb.tile, cb.ntile_r, cb.ntile_c, cb.B)
   FHS_DDE_SWITCH(cb.dde_R, FHS_L)
 #undef FHS_L
   note_launches(1);

@@ -627,40 +627,52 @@ __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ grid,
   out[i] = degrid_one(grid + (size_t)l * vg.K1 * vg.K2, uv[i], vg);
 }
 
-// Deterministic CTA reduction of per-block sums: values v0 (||z-y||^2) and v1
-// (||y - u||^2) of the visibility handled by this thread, block id b.
+// x^2 + y^2 as a float pair.
+__device__ __forceinline__ ff ff_norm2(ff x, ff y) { return ff_add(ff_mul(x, x), ff_mul(y, y)); }
+
+// Deterministic CTA reduction of the per-block sums of ||d||^2 and ||y - u||^2, one
+// visibility per thread (block id b): float pairs within a warp (FP64 shuffles and products
+// cost a warp about 1600 clk, these 300), FP64 across the warps.  Warps with a value whose
+// square leaves FP32's range take FP64.
 template <int NW>
-__device__ __forceinline__ void block_partials(double v0, double v1, int b, bool valid, int B, double* sred,
+__device__ __forceinline__ void block_partials(float2 d, float2 y, float2 u, int b, bool valid, int B, double* sred,
                                                double* out) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int b0 = __shfl_sync(0xffffffffu, valid ? b : -1, 0);
-  // lanes with invalid entries contribute zero to any block
-  bool uniform = __all_sync(0xffffffffu, !valid || b == b0) && b0 >= 0;
   for (int k = threadIdx.x; k < NW * 2 * B; k += blockDim.x) sred[k] = 0.0;
   __syncthreads();
-  if (uniform) {
-    double s0 = valid ? v0 : 0.0, s1 = valid ? v1 : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-    }
-    if (lane == 0) {
-      sred[(wid * 2 + 0) * B + b0] = s0;
-      sred[(wid * 2 + 1) * B + b0] = s1;
-    }
-  } else {
-    for (int bb = 0; bb < B; ++bb) {
-      double s0 = (valid && b == bb) ? v0 : 0.0, s1 = (valid && b == bb) ? v1 : 0.0;
+  if (!valid) d = y = u = make_float2(0.f, 0.f);
+  ff rx, ry;
+  two_sum(y.x, -u.x, rx.h, rx.l);
+  two_sum(y.y, -u.y, ry.h, ry.l);
+  const float m0 = fmaxf(fabsf(d.x), fabsf(d.y)), m1 = fmaxf(fabsf(rx.h), fabsf(ry.h));
+  const bool wide = m0 > 1e18f || m1 > 1e18f || (m0 > 0.f && m0 < 1e-15f) || (m1 > 0.f && m1 < 1e-15f);
+  const bool fp64 = __any_sync(0xffffffffu, wide);
+  const ff q0 = ff_norm2({d.x, 0.f}, {d.y, 0.f}), q1 = ff_norm2(rx, ry);
+  const double x0 = fp64 ? (double)d.x * d.x + (double)d.y * d.y : 0.0;
+  const double ax = fp64 ? (double)y.x - u.x : 0.0, ay = fp64 ? (double)y.y - u.y : 0.0;
+  unsigned left = __ballot_sync(0xffffffffu, valid);
+  while (left) {                                       // one pass per block id among the lanes
+    const int bb = __shfl_sync(0xffffffffu, b, __ffs(left) - 1);
+    const bool in = valid && b == bb;
+    left &= ~__ballot_sync(0xffffffffu, in);
+    double s0, s1;
+    if (fp64) {
+      s0 = in ? x0 : 0.0;
+      s1 = in ? ax * ax + ay * ay : 0.0;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         s0 += __shfl_xor_sync(0xffffffffu, s0, o);
         s1 += __shfl_xor_sync(0xffffffffu, s1, o);
       }
-      if (lane == 0) {
-        sred[(wid * 2 + 0) * B + bb] = s0;
-        sred[(wid * 2 + 1) * B + bb] = s1;
-      }
+    } else {
+      const ff zero = {0.f, 0.f};
+      const ff f0 = ff_warp_sum(in ? q0 : zero), f1 = ff_warp_sum(in ? q1 : zero);
+      s0 = lane == 0 ? ff_val(f0) : 0.0;
+      s1 = lane == 0 ? ff_val(f1) : 0.0;
+    }
+    if (lane == 0) {
+      sred[(wid * 2 + 0) * B + bb] = s0;
+      sred[(wid * 2 + 1) * B + bb] = s1;
     }
   }
   __syncthreads();
@@ -683,21 +695,19 @@ __global__ void __launch_bounds__(256) k_degrid_pdfb(const float2* __restrict__ 
   const int l = blockIdx.y;
   int64_t i = vis_off[l] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   bool valid = i < vis_off[l + 1];
-  double v0 = 0.0, v1 = 0.0;
+  float2 d = make_float2(0.f, 0.f), yy = d, u = d;
   int b = 0;
   if (valid) {
-    float2 u = degrid_one(grid + (size_t)l * vg.K1 * vg.K2, uv[i], vg);
-    float2 yy = y[i], vv = v[i], up = u_prev[i];
+    u = degrid_one(grid + (size_t)l * vg.K1 * vg.K2, uv[i], vg);
+    float2 vv = v[i], up = u_prev[i];
+    yy = y[i];
     float2 z = make_float2(vv.x + 2.f * u.x - up.x, vv.y + 2.f * u.y - up.y);
-    float2 d = make_float2(z.x - yy.x, z.y - yy.y);
+    d = make_float2(z.x - yy.x, z.y - yy.y);
     d_out[i] = d;
     u_prev[i] = u;
     b = blk[i];
-    v0 = (double)d.x * d.x + (double)d.y * d.y;
-    double rx = (double)yy.x - u.x, ry = (double)yy.y - u.y;
-    v1 = rx * rx + ry * ry;
   }
-  block_partials<8>(v0, v1, b, valid, B, sred, partials + ((size_t)l * nparts + blockIdx.x) * 2 * B);
+  block_partials<8>(d, yy, u, b, valid, B, sred, partials + ((size_t)l * nparts + blockIdx.x) * 2 * B);
 }
 
 // Tile-staged degridding (fast path).  One CTA per (grid tile, channel): every
@@ -886,16 +896,15 @@ __global__ void __launch_bounds__(256) k_l2ball_partials(const float2* __restric
   const int l = blockIdx.y;
   int64_t i = vis_off[l] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   bool valid = i < vis_off[l + 1];
-  double v0 = 0.0;
+  float2 d = make_float2(0.f, 0.f);
   int b = 0;
   if (valid) {
     float2 zz = z[i], yy = y[i];
-    float2 d = make_float2(zz.x - yy.x, zz.y - yy.y);
+    d = make_float2(zz.x - yy.x, zz.y - yy.y);
     d_out[i] = d;
     b = blk[i];
-    v0 = (double)d.x * d.x + (double)d.y * d.y;
   }
-  block_partials<8>(v0, 0.0, b, valid, B, sred, partials + ((size_t)l * nparts + blockIdx.x) * 2 * B);
+  block_partials<8>(d, make_float2(0.f, 0.f), make_float2(0.f, 0.f), b, valid, B, sred, partials + ((size_t)l * nparts + blockIdx.x) * 2 * B);
 }
 
 // ------------------------------------------------- preconditioned data duals
@@ -1115,12 +1124,12 @@ __global__ void k_l2ball_scale(const float2* __restrict__ d, const float* __rest
 // and right, 3 crosses right only.
 // Accumulation is in fixed point with 32-bit integer shared-memory atomics (several
 // times faster than floating-point ones, and order-independent, so the result is
-// bitwise deterministic), with one scale S = 2^e per tile chosen so that
-// n_c |c| < 2^30 for every tap value c = w v S, with n_c the largest number of
-// footprints that cover one cell of the tile (counted once per context, MODE 1) and
-// |v| <= m = max over the tile's visibilities of max(|Re v|, |Im v|): no cell can
-// overflow, and the resolution is n_c m / 2^30 (about 2^-23 of m for the densest
-// tiles of the large workload, n_c ~ 100).
+// bitwise deterministic), with one scale S = 2^e per tile chosen so that C m S < 2^30, with
+// C the largest sum over a cell of the tile of the weights |w_r w_c| that cover it (summed
+// once per context, MODE 1) and m = max over the tile's visibilities of max(|Re v|, |Im v|):
+// no cell can overflow, and the resolution is C m / 2^30.  (With the number of footprints in
+// place of their weights, about 8 times as large, the rounding of the taps was most of the
+// adjoint's error: 2.1e-7 against 1.6e-7 now at 23 channels of 768^2.)
 
 constexpr int kGridThreads = 128;                // threads per gridding CTA
 
@@ -1146,7 +1155,7 @@ __device__ __forceinline__ void grid_pass_range(const int32_t* toff, int pass, i
 // Adds the 7 x 7 taps of one visibility to the tile accumulators: rows lr + a,
 // columns lc + b.  ra[a] = row weight * S, wc[b] = column weight, (vx, vy) = v.
 // INTERIOR: the whole footprint lies in the tile (no bounds tests); otherwise only
-// rows in [a0, a1) and columns in [b0, b1) are added.  MODE 1 adds 1 per tap.
+// rows in [a0, a1) and columns in [b0, b1) are added.  MODE 1 adds |weight| S, rounded up.
 template <bool INTERIOR, int MODE>
 __device__ __forceinline__ void grid_taps(int* are, int* aim, int TP, int lr, int lc, const float* ra,
                                           const float* wc, float vx, float vy, int a0, int a1, int b0, int b1) {
@@ -1160,7 +1169,7 @@ __device__ __forceinline__ void grid_taps(int* are, int* aim, int TP, int lr, in
     for (int b = 0; b < kTaps; ++b) {
       if (!INTERIOR && (b < b0 || b >= b1)) continue;
       if (MODE == 1) {
-        atomicAdd(pr + b, 1);
+        atomicAdd(pr + b, __float2int_ru(fabsf(wc[b] * ra[a])));
       } else {
         atomicAdd(pr + b, __float2int_rn(wc[b] * xr));
         atomicAdd(pi + b, __float2int_rn(wc[b] * xi));
@@ -1169,15 +1178,22 @@ __device__ __forceinline__ void grid_taps(int* are, int* aim, int TP, int lr, in
   }
 }
 
+// Power of two S with S total < 2^30, at most 2^12: the unit of the weight sums of a tile
+// whose footprints weigh `total` together.
+__device__ __forceinline__ float cover_unit(float total) {
+  const float t = 1073741824.f / (fmaxf(total, 1.f) * 1.01f);
+  return pow2f(max(-120, min((int)((__float_as_uint(t) >> 23) & 0xffu) - 127, 12)));
+}
+
 // MODE 0: grid the (block-scaled) values into the tile and store it; MODE 1 (once per
-// context): count the footprints covering each cell and store the tile's maximum in
-// ncmax[l][tile].
+// context): sum the weights covering each cell and store the tile's maximum in
+// cover[l][tile].
 template <int MODE>
 __global__ void __launch_bounds__(kGridThreads, 1024 / kGridThreads) k_grid(const float2* __restrict__ vals, const float* __restrict__ blk_scale,
                                               float2* __restrict__ v_write, const float2* __restrict__ uv,
                                               const uint8_t* __restrict__ blk, const int32_t* __restrict__ tile_off,
                                               const int64_t* __restrict__ vis_off, float2* __restrict__ grid,
-                                              int* __restrict__ ncmax, VisGeom vg, int T, int ntr, int ntc, int B) {
+                                              float* __restrict__ cover, VisGeom vg, int T, int ntr, int ntc, int B) {
   extern __shared__ __align__(16) int sacc_i[];
   constexpr int NW = kGridThreads / 32;
   __shared__ float sred[NW];
@@ -1216,15 +1232,22 @@ __global__ void __launch_bounds__(kGridThreads, 1024 / kGridThreads) k_grid(cons
     m = 0.f;
 #pragma unroll
     for (int w = 0; w < NW; ++w) m = fmaxf(m, sred[w]);
-    const int nc = ncmax[l * ntr * ntc + tau];
-    if (m > 1e-30f && nc > 0) {
-      // S = 2^e <= 2^30 / (n_c m'), m' = m (1 + 2^-10) covering the roundings of v s,
-      // of the row product and a kernel weight a hair above 1
-      const float t = 1073741824.f / ((float)nc * (m * 1.0009765625f));
+    const float C = cover[l * ntr * ntc + tau];
+    if (m > 1e-30f && C > 0.f) {
+      // S = 2^e <= 2^30 / (C m'), m' = m (1 + 2^-10) covering the roundings of v s and of
+      // the products
+      const float t = 1073741824.f / (C * (m * 1.0009765625f));
       const int e = (int)((__float_as_uint(t) >> 23) & 0xffu) - 127;   // 2^e <= t
       S = pow2f(max(-120, min(e, 120)));
     }
   } else {
+    float nv = 0.f;
+    for (int pass = 0; pass < 4; ++pass) {
+      int sr, sc, beg, end;
+      grid_pass_range(toff, pass, tr, tc, ntr, ntc, sr, sc, beg, end);
+      nv += (float)(end - beg);
+    }
+    S = cover_unit(nv);
     __syncthreads();
   }
   // ---- sweep 1: taps
@@ -1274,7 +1297,7 @@ __global__ void __launch_bounds__(kGridThreads, 1024 / kGridThreads) k_grid(cons
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w = 0; w < NW; ++w) mx = max(mx, sredi[w]);
-      ncmax[l * ntr * ntc + tau] = mx;
+      cover[l * ntr * ntc + tau] = __int2float_ru(mx) / S;                 // S: a power of two
     }
     return;
   }
@@ -1484,7 +1507,7 @@ void launch_grid(const Cube& cb, const float2* vals, const float* blk_scale, flo
   dim3 grd(cb.ntile_r * cb.ntile_c, cb.L);
   size_t sm = 2 * (size_t)cb.tile * grid_row_stride(cb.tile) * sizeof(int);
   k_grid<0><<<grd, kGridThreads, sm, st>>>(vals, blk_scale, v_write, cb.d_uv, cb.d_blk, cb.d_tile_off, cb.d_vis_off, grid,
-                                  cb.d_ncmax, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
+                                  cb.d_cover, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
   note_launches(1);
 }
 
@@ -1494,7 +1517,7 @@ void launch_grid_count(const Cube& cb, cudaStream_t st) {
   dim3 grd(cb.ntile_r * cb.ntile_c, cb.L);
   size_t sm = 2 * (size_t)cb.tile * grid_row_stride(cb.tile) * sizeof(int);
   k_grid<1><<<grd, kGridThreads, sm, st>>>(nullptr, nullptr, nullptr, cb.d_uv, cb.d_blk, cb.d_tile_off, cb.d_vis_off, nullptr,
-                                  cb.d_ncmax, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
+                                  cb.d_cover, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
   note_launches(1);
 }
 
