@@ -15,11 +15,11 @@
 //                 W <- z min(1, alpha_i / ||z_i||), z = W + Psi^dagger x
 //                 (weights mode: theta_i = mu / (||Psi^dagger x||_i + mu)).
 //   k_syn2_all  : one synthesis level (4 -> 3, 3 -> 2, 2 -> 1) of every basis in
-//                 one launch (k_syn2_one: one basis, as above), a 32x32 output
-//                 tile of one channel per CTA,
+//                 one launch (k_syn2_one: one basis, as above), a 64x64 or 32x32
+//                 output tile of one channel per CTA,
 //                 polyphase (even outputs take the odd taps and vice versa),
 //                 register-blocked.
-//   k_synfin    : level 1 of all eight bases and the Dirac block for a 32x32
+//   k_synfin    : level 1 of all eight bases and the Dirac block for a 64x64 or 32x32
 //                 output tile, accumulated in registers; A += kappa * result.
 // Same conventions as the plain kernels (zero-padded full convolution, odd
 // phase, coefficients scaled by 1/3).
@@ -28,7 +28,6 @@ namespace fhs {
 
 constexpr int kT2 = 32;                              // tile side (coefficients or outputs)
 constexpr int kIn2 = 2 * kT2 + kMaxFilt - 2;         // 78: input rows/cols of an analysis tile
-constexpr int kKn2 = kT2 / 2 + kMaxFilt / 2;         // 24: coefficient rows/cols of a synthesis tile
 
 // Filter taps of basis F/2 - 1, read straight from the constant bank: with the tap
 // index known at compile time (unrolled loops) every FMA takes the tap as a
@@ -284,141 +283,132 @@ struct Syn2 {
   int mo1, mo2, m1, m2;
 };
 
-// Staging of the four coefficient bands (LL, d0, d1, d2; raw values, zero outside the
-// level) of the synthesis tile (r0, c0) of channel l: window rows [r0/2, r0/2 + KN),
-// columns [c0/2, c0/2 + KN), KN = 16 + F/2, by 4-byte asynchronous copies (lane =
-// column, warp = row), band b at b kTS2e, rows at stride kKn2 + 1.
-constexpr int kTS2e = kKn2 * (kKn2 + 1);             // 600
+// Synthesis of one (basis, level) tile of T x T outputs.  Pass y: a thread takes one
+// coefficient column and STEPS coefficient rows of it (2 STEPS output rows), its
+// STEPS + F/2 - 1 coefficients of two bands at a time straight from global memory into
+// registers (coalesced along the row, all in flight), and leaves the low and high rows in
+// shared memory; pass x: a thread takes OUT consecutive outputs of a row, its windows read
+// as float4 (the row pitches spread a quarter-warp over all banks).  Per pixel and basis
+// of length F this is about 2.3 F FMAs at T = 64 beside F/4 loads and stores; the form with
+// 32 x 32 tiles that staged the bands in shared memory and read every operand of both passes
+// from there spent 735 instructions a pixel at level 1 of all bases for 180 FMAs (6.70 ms at
+// 16 channels of 4096^2; now 3.10 ms, 1.6 of them the bytes).
+//
+// 32 x 32 tiles (images too small for two waves of the others) are bound by latency: half the
+// rows and outputs per thread, and all four bands' loads in flight at once.
+template <int T> struct SynCfg {
+  static constexpr int STEPS = T == 64 ? 4 : 2;      // coefficient rows per task of pass y
+  static constexpr int OUT = T == 64 ? 16 : 8;       // outputs per thread of pass x
+  static constexpr int KN = T / 2 + kMaxFilt / 2;    // coefficient columns, longest filter
+  static constexpr int LD = T == 64 ? 44 : 28;       // pitch of the low / high rows
+  static constexpr int SEGS = T / 2 / STEPS;
+  static constexpr int NT = (KN * SEGS + 31) / 32 * 32;      // 320 or 192: one task of pass y each
+  static constexpr int XT = T * T / OUT;                     // 256 or 128 threads of pass x
+  static constexpr int BUF = 2 * T * LD;                     // floats: low rows, then high rows
+  static_assert(LD >= KN && LD % 4 == 0 && XT <= NT, "synthesis tile");
+};
 
-template <int F>
-__device__ __forceinline__ void syn2_stage_e(const Syn2& s, int l, int r0, int c0, float* tc) {
-  constexpr int KN = kT2 / 2 + F / 2;
-  static_assert(KN <= 32, "one warp spans a staged row");
-  const int kc = threadIdx.x & 31, kr0 = threadIdx.x >> 5;   // lane = column, warp = row (step 8)
-  if (kc < KN) {
-    const int klo = r0 / 2, gc = c0 / 2 + kc;
-    // rows kr0, kr0 + 8, ... of this thread that lie inside the band (none if the column is out)
-    const int nrows = gc < s.mo2 ? min((KN - kr0 + 7) / 8, max(0, (s.mo1 - klo - kr0 + 7) / 8)) : 0;
-    const float* Wl = s.W + (size_t)l * s.I;
-    const float* b0 = s.ll ? s.ll + (size_t)l * s.mo1 * s.mo2 : Wl + s.off[3];
-    const int64_t start = (int64_t)(klo + kr0) * s.mo2 + gc, step = 8 * (int64_t)s.mo2;
-    const float* bp[4] = {b0 + start, Wl + s.off[0] + start, Wl + s.off[1] + start, Wl + s.off[2] + start};
-    float* dst = tc + kr0 * (kKn2 + 1) + kc;
-#pragma unroll
-    for (int band = 0; band < 4; ++band) {
-      const float* src = bp[band];
-#pragma unroll
-      for (int j = 0; j < (KN + 7) / 8; ++j) {
-        if (kr0 + 8 * j < KN) {
-          const bool v = j < nrows;
-          cp_async4(dst + band * kTS2e + 8 * j * (kKn2 + 1), v ? src : b0, v);
-        }
-        src += step;
-      }
-    }
-  }
-  cp_async_commit();
-}
-
-// Synthesis of one staged (basis, level) tile, added to acc[4]: outputs at row
-// il = threadIdx.x >> 3, columns 4 * (threadIdx.x & 7) + q.  tl, t0, t1, t2: window
-// element (0, 0) of the LL, d0, d1, d2 bands, rows at stride R.  Coefficients carry the
-// 1/3 of the dictionary except a synthesised LL band (ll_scale = 1).
-template <int F, int R>
-__device__ __forceinline__ void syn2_compute(const float* tl, const float* t0, const float* t1, const float* t2,
-                                             float* lx, float* hx, float ll_scale, float acc[4]) {
-  constexpr int KN = kT2 / 2 + F / 2;
-  constexpr int WIN = F / 2 + 1;
-  FTaps<F> f;
-  f.load();
+template <int T, int F, bool INSIDE>
+__device__ __forceinline__ void syn_pass_y(const Syn2& s, int l, int r0, int c0, float* lx, float ll_scale) {
+  using C = SynCfg<T>;
+  constexpr int KN = T / 2 + F / 2, ROWS = C::STEPS + F / 2 - 1;
+  const int seg = threadIdx.x / KN, kc = threadIdx.x - seg * KN;
+  if (seg >= C::SEGS) return;
+  const int m0 = seg * C::STEPS, k = r0 / 2 + m0, gc = c0 / 2 + kc;
+  const int nrow = INSIDE ? ROWS : (gc < s.mo2 ? s.mo1 - k : 0);       // rows of this column inside the band
+  const float* Wl = s.W + (size_t)l * s.I;
+  const int64_t start = (int64_t)k * s.mo2 + gc;
   const float third = 1.f / 3.f;
-  for (int item = threadIdx.x; item < KN * 8; item += 256) {
-    const int kc = item % KN, mg = (item / KN) * 2;
-    float vl[WIN + 1], v1[WIN + 1], v0[WIN + 1], v2[WIN + 1];
+  FTaps<F> f;
+  float* o = lx + 2 * m0 * C::LD + kc;
+  // low rows (half 0) from LL and d1, high rows (half 1) from d0 and d2
+  constexpr int NH = T == 64 ? 1 : 2;                // halves loaded together
+  float va[NH][ROWS], vb[NH][ROWS];
+  auto fetch = [&](int half, float* a, float* b) {
+    const float* pa = half ? Wl + s.off[0] + start
+                           : (s.ll ? s.ll + (size_t)l * s.mo1 * s.mo2 : Wl + s.off[3]) + start;
+    const float* pb = Wl + s.off[half ? 2 : 1] + start;
 #pragma unroll
-    for (int u = 0; u <= WIN; ++u) {
-      const int o = (mg + u) * R + kc;
-      vl[u] = tl[o];
-      v0[u] = t0[o];
-      v1[u] = t1[o];
-      v2[u] = t2[o];
+    for (int u = 0; u < ROWS; ++u) {
+      a[u] = INSIDE || u < nrow ? pa[(size_t)u * s.mo2] : 0.f;
+      b[u] = INSIDE || u < nrow ? pb[(size_t)u * s.mo2] : 0.f;
     }
-    // raw coefficients; the dictionary's 1/3 (and ll_scale) applied once per output
+  };
 #pragma unroll
-    for (int mm = 0; mm < 2; ++mm) {
+  for (int h = 0; h < NH; ++h) fetch(h, va[h], vb[h]);
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    if (half >= NH) fetch(half, va[0], vb[0]);
+    const float* a = va[half < NH ? half : 0];
+    const float* b = vb[half < NH ? half : 0];
+#pragma unroll
+    for (int m = 0; m < C::STEPS; ++m) {
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
-        float slh = 0.f, slg = 0.f, sxh = 0.f, sxg = 0.f;
+        float sh = 0.f, sg = 0.f;
 #pragma unroll
         for (int q = 0; q < F / 2; ++q) {
-          const float hh = f.h[2 * q + 1 - p], gg = f.g[2 * q + 1 - p];
-          slh = fmaf(hh, vl[mm + q], slh);
-          slg = fmaf(gg, v1[mm + q], slg);
-          sxh = fmaf(hh, v0[mm + q], sxh);
-          sxg = fmaf(gg, v2[mm + q], sxg);
+          sh = fmaf(f.h[2 * q + 1 - p], a[m + q], sh);
+          sg = fmaf(f.g[2 * q + 1 - p], b[m + q], sg);
         }
-        const int il = 2 * (mg + mm) + p;
-        lx[il * (kKn2 + 1) + kc] = fmaf(ll_scale, slh, third * slg);
-        hx[il * (kKn2 + 1) + kc] = third * (sxh + sxg);
+        // the dictionary's 1/3 (ll_scale: 1 for a synthesised LL band) once per value
+        o[(half * T + 2 * m + p) * C::LD] = half ? third * (sh + sg) : fmaf(ll_scale, sh, third * sg);
       }
     }
   }
-  __syncthreads();
-  {
-    const int il = threadIdx.x >> 3, g4 = threadIdx.x & 7;
-    const int mg = 2 * g4;
-    float a[WIN + 1], b[WIN + 1];
+}
+
+// acc += outputs OUT (tid % (T/OUT)) .. of row tid / (T/OUT).
+template <int T, int F>
+__device__ __forceinline__ void syn_pass_x(const float* lx, float (&acc)[SynCfg<T>::OUT]) {
+  using C = SynCfg<T>;
+  constexpr int NW = SynCfg<T>::OUT / 2 + F / 2 - 1, N4 = (NW + 3) / 4;
+  if ((int)threadIdx.x >= C::XT) return;
+  const int il = threadIdx.x / (T / SynCfg<T>::OUT), mg = threadIdx.x % (T / SynCfg<T>::OUT) * (SynCfg<T>::OUT / 2);
+  FTaps<F> f;
+  float a[4 * N4], b[4 * N4];
 #pragma unroll
-    for (int u = 0; u <= WIN; ++u) {
-      a[u] = lx[il * (kKn2 + 1) + mg + u];
-      b[u] = hx[il * (kKn2 + 1) + mg + u];
+  for (int u = 0; u < N4; ++u) {
+    const float4 x = *reinterpret_cast<const float4*>(lx + il * C::LD + mg + 4 * u);
+    const float4 y = *reinterpret_cast<const float4*>(lx + (T + il) * C::LD + mg + 4 * u);
+    a[4 * u] = x.x; a[4 * u + 1] = x.y; a[4 * u + 2] = x.z; a[4 * u + 3] = x.w;
+    b[4 * u] = y.x; b[4 * u + 1] = y.y; b[4 * u + 2] = y.z; b[4 * u + 3] = y.w;
+  }
+#pragma unroll
+  for (int m = 0; m < SynCfg<T>::OUT / 2; ++m) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      float v = 0.f;
+#pragma unroll
+      for (int q = 0; q < F / 2; ++q)
+        v = fmaf(f.h[2 * q + 1 - p], a[m + q], fmaf(f.g[2 * q + 1 - p], b[m + q], v));
+      acc[2 * m + p] += v;
     }
+  }
+}
+
+// Pass y, a barrier, pass x of filter length F on the buffer sh (2 T LD floats).
+template <int T, int F>
+__device__ __forceinline__ void syn_tile(const Syn2& s, int l, int r0, int c0, float* sh, float ll_scale,
+                                         float (&acc)[SynCfg<T>::OUT]) {
+  const bool inside = r0 / 2 + T / 2 + F / 2 <= s.mo1 && c0 / 2 + T / 2 + F / 2 <= s.mo2;
+  if (inside) syn_pass_y<T, F, true>(s, l, r0, c0, sh, ll_scale);
+  else syn_pass_y<T, F, false>(s, l, r0, c0, sh, ll_scale);
+  __syncthreads();
+  syn_pass_x<T, F>(sh, acc);
+}
+
+// The accumulators as a [T][T + 4] tile in sh (after a barrier), for coalesced stores.
+template <int T>
+__device__ __forceinline__ void syn_to_tile(float* sh, const float (&acc)[SynCfg<T>::OUT]) {
+  __syncthreads();
+  if ((int)threadIdx.x < SynCfg<T>::XT) {
+    float* o = sh + threadIdx.x / (T / SynCfg<T>::OUT) * (T + 4) + threadIdx.x % (T / SynCfg<T>::OUT) * SynCfg<T>::OUT;
 #pragma unroll
-    for (int mm = 0; mm < 2; ++mm) {
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        float v = 0.f;
-#pragma unroll
-        for (int q = 0; q < F / 2; ++q)
-          v = fmaf(f.h[2 * q + 1 - p], a[mm + q], fmaf(f.g[2 * q + 1 - p], b[mm + q], v));
-        acc[2 * mm + p] += v;
-      }
-    }
+    for (int u = 0; u < SynCfg<T>::OUT / 4; ++u)
+      *reinterpret_cast<float4*>(o + 4 * u) = make_float4(acc[4 * u], acc[4 * u + 1], acc[4 * u + 2], acc[4 * u + 3]);
   }
   __syncthreads();
-}
-
-// Staging and compute of basis b = F/2 - 1 (runtime b, compile-time F).
-__device__ __forceinline__ void syn2_stage_any(int b, const Syn2& s, int l, int r0, int c0, float* tc) {
-  switch (b) {
-    case 0: syn2_stage_e<2>(s, l, r0, c0, tc); break;
-    case 1: syn2_stage_e<4>(s, l, r0, c0, tc); break;
-    case 2: syn2_stage_e<6>(s, l, r0, c0, tc); break;
-    case 3: syn2_stage_e<8>(s, l, r0, c0, tc); break;
-    case 4: syn2_stage_e<10>(s, l, r0, c0, tc); break;
-    case 5: syn2_stage_e<12>(s, l, r0, c0, tc); break;
-    case 6: syn2_stage_e<14>(s, l, r0, c0, tc); break;
-    default: syn2_stage_e<16>(s, l, r0, c0, tc); break;
-  }
-}
-
-template <int F>
-__device__ __forceinline__ void syn2_compute_e(const float* tc, float* lx, float* hx, float lls, float acc[4]) {
-  syn2_compute<F, kKn2 + 1>(tc, tc + kTS2e, tc + 2 * kTS2e, tc + 3 * kTS2e, lx, hx, lls, acc);
-}
-
-__device__ __forceinline__ void syn2_compute_any(int b, const float* tc, float* lx, float* hx, float lls,
-                                                 float acc[4]) {
-  switch (b) {
-    case 0: syn2_compute_e<2>(tc, lx, hx, lls, acc); break;
-    case 1: syn2_compute_e<4>(tc, lx, hx, lls, acc); break;
-    case 2: syn2_compute_e<6>(tc, lx, hx, lls, acc); break;
-    case 3: syn2_compute_e<8>(tc, lx, hx, lls, acc); break;
-    case 4: syn2_compute_e<10>(tc, lx, hx, lls, acc); break;
-    case 5: syn2_compute_e<12>(tc, lx, hx, lls, acc); break;
-    case 6: syn2_compute_e<14>(tc, lx, hx, lls, acc); break;
-    default: syn2_compute_e<16>(tc, lx, hx, lls, acc); break;
-  }
 }
 
 // One synthesis level (4 -> 3, 3 -> 2 or 2 -> 1) of every basis in one launch, tiles of
@@ -430,28 +420,26 @@ struct Syn2All {
   int nb;
 };
 
-template <int F>
+template <int T, int F>
 __device__ __forceinline__ void syn2_body(const Syn2& s, float* __restrict__ out, int tiles_x, int tile, int l,
                                           float* sh) {
   const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
-  const int r0 = ty * kT2, c0 = tx * kT2;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  syn2_stage_e<F>(s, l, r0, c0, sh);
-  cp_async_wait<0>();
-  __syncthreads();
-  syn2_compute<F, kKn2 + 1>(sh, sh + kTS2e, sh + 2 * kTS2e, sh + 3 * kTS2e, sh + 4 * kTS2e,
-                            sh + 4 * kTS2e + kT2 * (kKn2 + 1), s.ll ? 1.f : 1.f / 3.f, acc);
-  const int il = threadIdx.x >> 3, jc0 = 4 * (threadIdx.x & 7);
-  const int r = r0 + il;
-  if (r >= s.m1) return;
-  float* ol = out + (size_t)l * s.m1 * s.m2 + (size_t)r * s.m2;
+  const int r0 = ty * T, c0 = tx * T;
+  float acc[SynCfg<T>::OUT];
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (c0 + jc0 + q < s.m2) ol[c0 + jc0 + q] = acc[q];
+  for (int u = 0; u < SynCfg<T>::OUT; ++u) acc[u] = 0.f;
+  syn_tile<T, F>(s, l, r0, c0, sh, s.ll ? 1.f : 1.f / 3.f, acc);
+  syn_to_tile<T>(sh, acc);
+  float* ol = out + (size_t)l * s.m1 * s.m2;
+  for (int k = threadIdx.x; k < T * T; k += SynCfg<T>::NT) {
+    const int r = k / T, c = k % T;
+    if (r0 + r < s.m1 && c0 + c < s.m2) ol[(size_t)(r0 + r) * s.m2 + c0 + c] = sh[r * (T + 4) + c];
+  }
 }
 
-__global__ void __launch_bounds__(256) k_syn2_all(const Syn2All a) {
-  __shared__ float sh[4 * kTS2e + 2 * kT2 * (kKn2 + 1)];
+template <int T>
+__global__ void __launch_bounds__(SynCfg<T>::NT) k_syn2_all(const Syn2All a) {
+  __shared__ __align__(16) float sh[SynCfg<T>::BUF];
   const int t = blockIdx.x, l = blockIdx.y;
   int bi = 0;
 #pragma unroll 1
@@ -459,21 +447,21 @@ __global__ void __launch_bounds__(256) k_syn2_all(const Syn2All a) {
     if (t >= a.tile0[k]) bi = k;
   const int tile = t - a.tile0[bi];
   switch (a.F[bi]) {
-    case 2: syn2_body<2>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
-    case 4: syn2_body<4>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
-    case 6: syn2_body<6>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
-    case 8: syn2_body<8>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
-    case 10: syn2_body<10>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
-    case 12: syn2_body<12>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
-    case 14: syn2_body<14>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
-    default: syn2_body<16>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    case 2: syn2_body<T, 2>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    case 4: syn2_body<T, 4>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    case 6: syn2_body<T, 6>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    case 8: syn2_body<T, 8>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    case 10: syn2_body<T, 10>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    case 12: syn2_body<T, 12>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    case 14: syn2_body<T, 14>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
+    default: syn2_body<T, 16>(a.s[bi], a.out[bi], a.tiles_x[bi], tile, l, sh); break;
   }
 }
 
 template <int F>
-__global__ void __launch_bounds__(256) k_syn2_one(const Syn2 s, float* __restrict__ out, int tiles_x) {
-  __shared__ float sh[4 * kTS2e + 2 * kT2 * (kKn2 + 1)];
-  syn2_body<F>(s, out, tiles_x, blockIdx.x, blockIdx.y, sh);
+__global__ void __launch_bounds__(SynCfg<64>::NT) k_syn2_one(const Syn2 s, float* __restrict__ out, int tiles_x) {
+  __shared__ __align__(16) float sh[SynCfg<64>::BUF];
+  syn2_body<64, F>(s, out, tiles_x, blockIdx.x, blockIdx.y, sh);
 }
 
 // A level runs as one launch per basis when the smallest basis alone has at least two
@@ -484,16 +472,16 @@ static bool sara_level_per_basis(const int* tiles, int L) {
   return mn >= 2LL * 4 * num_sms();
 }
 
-#define FHS_F_SWITCH(F, KERNEL, GRID, ...)                               \
+#define FHS_F_SWITCH(F, KERNEL, GRID, NT, ...)                           \
   switch (F) {                                                           \
-    case 2: KERNEL<2><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;         \
-    case 4: KERNEL<4><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;         \
-    case 6: KERNEL<6><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;         \
-    case 8: KERNEL<8><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;         \
-    case 10: KERNEL<10><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;       \
-    case 12: KERNEL<12><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;       \
-    case 14: KERNEL<14><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;       \
-    default: KERNEL<16><<<GRID, 256, 0, st>>>(__VA_ARGS__); break;       \
+    case 2: KERNEL<2><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;          \
+    case 4: KERNEL<4><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;          \
+    case 6: KERNEL<6><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;          \
+    case 8: KERNEL<8><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;          \
+    case 10: KERNEL<10><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;        \
+    case 12: KERNEL<12><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;        \
+    case 14: KERNEL<14><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;        \
+    default: KERNEL<16><<<GRID, NT, 0, st>>>(__VA_ARGS__); break;        \
   }
 
 struct SynFin2 {
@@ -504,51 +492,56 @@ struct SynFin2 {
   int vec4;            // A, W, the Dirac block and n2 allow 16-byte accesses
 };
 
-// Level 1 of all bases: the tiles of basis b + 1 are staged (cp.async) while basis b
-// is computed.
-__global__ void __launch_bounds__(256, 3) k_synfin(SynFin2 s, float* __restrict__ A) {
-  __shared__ float sh[2 * 4 * kTS2e + 2 * kT2 * (kKn2 + 1)];
-  float* lx = sh + 8 * kTS2e;
-  float* hx = lx + kT2 * (kKn2 + 1);
-  const int l = blockIdx.z;
-  const int r0 = blockIdx.y * kT2, c0 = blockIdx.x * kT2;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  syn2_stage_any(0, s.lv[0], l, r0, c0, sh);
-#pragma unroll 1
-  for (int b = 0; b < 8; ++b) {
-    if (b + 1 < 8) {
-      syn2_stage_any(b + 1, s.lv[b + 1], l, r0, c0, sh + ((b + 1) & 1) * 4 * kTS2e);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    syn2_compute_any(b, sh + (b & 1) * 4 * kTS2e, lx, hx, 1.f, acc);
-  }
-  const int il = threadIdx.x >> 3, jc0 = 4 * (threadIdx.x & 7);
-  const int r = r0 + il;
-  if (r >= s.n1) return;
-  const size_t N = (size_t)s.n1 * s.n2;
-  const size_t drow = (size_t)l * s.lv[0].I + s.dirac_off + (size_t)r * s.n2;
-  const float* Wd = s.lv[0].W + drow;
-  float* Al = A + (size_t)l * N + (size_t)r * s.n2;
-  const int c = c0 + jc0;
-  // four consecutive outputs: one 16-byte read-modify-write of A when the row and the
-  // Dirac block allow it
-  if (s.vec4 && c + 3 < s.n2) {
-    const float4 wd = *reinterpret_cast<const float4*>(Wd + c);
-    float4 a = *reinterpret_cast<const float4*>(Al + c);
-    a.x = fmaf(s.kappa, acc[0] + wd.x * (1.f / 3.f), a.x);
-    a.y = fmaf(s.kappa, acc[1] + wd.y * (1.f / 3.f), a.y);
-    a.z = fmaf(s.kappa, acc[2] + wd.z * (1.f / 3.f), a.z);
-    a.w = fmaf(s.kappa, acc[3] + wd.w * (1.f / 3.f), a.w);
-    *reinterpret_cast<float4*>(Al + c) = a;
-    return;
-  }
+// Level 1 of all bases and the Dirac block for a T x T output tile, accumulated in
+// registers; A += kappa * result.  The low / high rows of consecutive bases alternate between
+// two buffers, so a basis costs one barrier.
+template <int T>
+__global__ void __launch_bounds__(SynCfg<T>::NT, T == 64 ? 3 : 2) k_synfin(const SynFin2 s, float* __restrict__ A) {
+  extern __shared__ __align__(16) float synfin_sh[];             // 2 BUF floats
+  constexpr int BUF = SynCfg<T>::BUF;
+  const int l = blockIdx.z, r0 = blockIdx.y * T, c0 = blockIdx.x * T;
+  float acc[SynCfg<T>::OUT];
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (c + q < s.n2) Al[c + q] = fmaf(s.kappa, acc[q] + Wd[c + q] * (1.f / 3.f), Al[c + q]);
+  for (int u = 0; u < SynCfg<T>::OUT; ++u) acc[u] = 0.f;
+  syn_tile<T, 2>(s.lv[0], l, r0, c0, synfin_sh, 1.f, acc);
+  syn_tile<T, 4>(s.lv[1], l, r0, c0, synfin_sh + BUF, 1.f, acc);
+  syn_tile<T, 6>(s.lv[2], l, r0, c0, synfin_sh, 1.f, acc);
+  syn_tile<T, 8>(s.lv[3], l, r0, c0, synfin_sh + BUF, 1.f, acc);
+  syn_tile<T, 10>(s.lv[4], l, r0, c0, synfin_sh, 1.f, acc);
+  syn_tile<T, 12>(s.lv[5], l, r0, c0, synfin_sh + BUF, 1.f, acc);
+  syn_tile<T, 14>(s.lv[6], l, r0, c0, synfin_sh, 1.f, acc);
+  syn_tile<T, 16>(s.lv[7], l, r0, c0, synfin_sh + BUF, 1.f, acc);
+  syn_to_tile<T>(synfin_sh, acc);
+  const size_t N = (size_t)s.n1 * s.n2;
+  const float* Wd = s.lv[0].W + (size_t)l * s.lv[0].I + s.dirac_off;
+  float* Al = A + (size_t)l * N;
+  // four consecutive outputs: one 16-byte read-modify-write of A where the rows and the
+  // Dirac block allow it
+  for (int k = threadIdx.x; k < T * T / 4; k += SynCfg<T>::NT) {
+    const int rr = k / (T / 4), cc = k % (T / 4) * 4, r = r0 + rr, c = c0 + cc;
+    if (r >= s.n1 || c >= s.n2) continue;
+    const float4 v = *reinterpret_cast<const float4*>(synfin_sh + rr * (T + 4) + cc);
+    const size_t o = (size_t)r * s.n2 + c;
+    if (s.vec4 && c + 3 < s.n2) {
+      const float4 wd = *reinterpret_cast<const float4*>(Wd + o);
+      float4 a = *reinterpret_cast<const float4*>(Al + o);
+      a.x = fmaf(s.kappa, v.x + wd.x * (1.f / 3.f), a.x);
+      a.y = fmaf(s.kappa, v.y + wd.y * (1.f / 3.f), a.y);
+      a.z = fmaf(s.kappa, v.z + wd.z * (1.f / 3.f), a.z);
+      a.w = fmaf(s.kappa, v.w + wd.w * (1.f / 3.f), a.w);
+      *reinterpret_cast<float4*>(Al + o) = a;
+    } else {
+      const float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (c + q < s.n2) Al[o + q] = fmaf(s.kappa, e[q] + Wd[o + q] * (1.f / 3.f), Al[o + q]);
+    }
+  }
 }
+
+// Synthesis tiles: 64 x 64 where they make at least two waves of CTAs (three per SM; halo
+// 1.56 coefficients per output pair against 2.25 at 32), else 32 x 32.
+static bool syn_large_tiles(int64_t ctas64) { return ctas64 >= 2LL * 3 * num_sms(); }
 
 // ------------------------------------------------------------- launchers
 // Analysis of every basis and level into the coefficient buffer, the l2,1 dual (or
@@ -610,7 +603,7 @@ void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, co
     for (int k = 0; k < 8; ++k) tiles[k] = (k + 1 < 8 ? a.b[k + 1].tile0 : t0) - a.b[k].tile0;
     if (sara_level_per_basis(tiles, L)) {
       for (int k = 0; k < 8; ++k) {
-        FHS_F_SWITCH(a.b[k].F, k_ana2_one, dim3(tiles[k], L), a.b[k], coef, S.I);
+        FHS_F_SWITCH(a.b[k].F, k_ana2_one, dim3(tiles[k], L), 256, a.b[k], coef, S.I);
       }
       note_launches(8);
     } else {
@@ -640,7 +633,13 @@ void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, co
   for (int j = kLevels; j >= 2; --j) {
     Syn2All a;
     a.nb = 8;
-    int t0 = 0;
+    auto tiles_of = [&](int b, int T) {
+      return ((S.cols[b][j - 1] + T - 1) / T) * ((S.rows[b][j - 1] + T - 1) / T);
+    };
+    int64_t n64 = 0;
+    for (int b = 0; b < 8; ++b) n64 += tiles_of(b, 64);
+    const int T = syn_large_tiles(n64 * L) ? 64 : 32;
+    int t0 = 0, tiles[8];
     for (int k = 0; k < 8; ++k) {
       const int b = 7 - k;
       Syn2& s = a.s[k];
@@ -653,20 +652,20 @@ void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, co
       s.m1 = S.rows[b][j - 1]; s.m2 = S.cols[b][j - 1];
       a.out[k] = (j == 2) ? slots + ctx->s.ll1_off[b] : (j == 3) ? ctx->s.ll2 + ctx->s.ll2_off[b]
                                                                  : ctx->s.ll3 + ctx->s.ll3_off[b];
-      a.tiles_x[k] = (s.m2 + kT2 - 1) / kT2;
+      a.tiles_x[k] = (s.m2 + T - 1) / T;
       a.tile0[k] = t0;
       a.F[k] = 2 * (b + 1);
-      t0 += a.tiles_x[k] * ((s.m1 + kT2 - 1) / kT2);
+      tiles[k] = tiles_of(b, T);
+      t0 += tiles[k];
     }
-    int tiles[8];
-    for (int k = 0; k < 8; ++k) tiles[k] = (k + 1 < 8 ? a.tile0[k + 1] : t0) - a.tile0[k];
-    if (sara_level_per_basis(tiles, L)) {
+    if (T == 64 && sara_level_per_basis(tiles, L)) {
       for (int k = 0; k < 8; ++k) {
-        FHS_F_SWITCH(a.F[k], k_syn2_one, dim3(tiles[k], L), a.s[k], a.out[k], a.tiles_x[k]);
+        FHS_F_SWITCH(a.F[k], k_syn2_one, dim3(tiles[k], L), SynCfg<64>::NT, a.s[k], a.out[k], a.tiles_x[k]);
       }
       note_launches(8);
     } else {
-      k_syn2_all<<<dim3(t0, L), 256, 0, st>>>(a);
+      if (T == 64) k_syn2_all<64><<<dim3(t0, L), SynCfg<64>::NT, 0, st>>>(a);
+      else k_syn2_all<32><<<dim3(t0, L), SynCfg<32>::NT, 0, st>>>(a);
       note_launches(1);
     }
   }
@@ -686,8 +685,13 @@ void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, co
   fin.kappa = (float)cb.kappa;
   fin.vec4 = (cb.n2 % 4 == 0 && S.dirac_off % 4 == 0 && S.I % 4 == 0 && ((uintptr_t)A % 16) == 0 &&
               ((uintptr_t)W % 16) == 0) ? 1 : 0;
-  dim3 g((cb.n2 + kT2 - 1) / kT2, (cb.n1 + kT2 - 1) / kT2, L);
-  k_synfin<<<g, 256, 0, st>>>(fin, A);
+  auto launch_fin = [&](auto kernel, int T, int nt, int buf) {
+    const size_t sm = 2 * (size_t)buf * sizeof(float);
+    kernel<<<dim3((cb.n2 + T - 1) / T, (cb.n1 + T - 1) / T, L), nt, sm, st>>>(fin, A);
+  };
+  const int64_t n64 = (int64_t)((cb.n2 + 63) / 64) * ((cb.n1 + 63) / 64) * L;
+  if (syn_large_tiles(n64)) launch_fin(k_synfin<64>, 64, SynCfg<64>::NT, SynCfg<64>::BUF);
+  else launch_fin(k_synfin<32>, 32, SynCfg<32>::NT, SynCfg<32>::BUF);
   note_launches(1);
 }
 
