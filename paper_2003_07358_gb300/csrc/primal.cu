@@ -4,6 +4,7 @@
 // variation xi; float4 streaming, fixed grid, fixed-order reductions.
 #include <cuda_runtime.h>
 
+#include "ffloat.cuh"
 #include "fhs_internal.h"
 
 namespace fhs {
@@ -29,6 +30,26 @@ __device__ __forceinline__ void cta_sum2(double a, double b, double* out) {
   }
 }
 
+// CTA sums of two float pairs per thread (fixed order), written in FP64: FP64 shuffles would
+// cost every warp 640 clk of the FP64 pipe, 5 us over the 64 warps of an SM.
+template <int NT>
+__device__ __forceinline__ void cta_sum2(ff a, ff b, double* out) {
+  __shared__ float2 s[2][NT / 32];
+  a = ff_warp_sum(a);
+  b = ff_warp_sum(b);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane == 0) { s[0][wid] = make_float2(a.h, a.l); s[1][wid] = make_float2(b.h, b.l); }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    ff x = {0.f, 0.f};
+    for (int w = 0; w < NT / 32; ++w) {
+      const float2 v = s[threadIdx.x][w];
+      x = ff_add(x, {v.x, v.y});
+    }
+    out[threadIdx.x] = ff_val(x);
+  }
+}
+
 // Compensated (Kahan) FP32 running sum; the FP64 pipe of the SM is kept for the
 // final per-thread totals only.
 struct KahanF {
@@ -44,6 +65,10 @@ struct KahanF {
 __global__ void __launch_bounds__(256) k_primal(float4* __restrict__ X, float4* __restrict__ Xc,
                                                 const float4* __restrict__ A, float tau, int64_t n4,
                                                 double* __restrict__ partials) {
+  if ((int64_t)blockIdx.x * blockDim.x >= n4) {          // small images: nothing for this CTA
+    if (threadIdx.x < 2) partials[2 * (size_t)blockIdx.x + threadIdx.x] = 0.0;
+    return;
+  }
   KahanF dx2, x2;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
     float4 x = X[i], a = A[i];
@@ -63,7 +88,7 @@ __global__ void __launch_bounds__(256) k_primal(float4* __restrict__ X, float4* 
     dx2.add(fmaf(d0, d0, fmaf(d1, d1, fmaf(d2, d2, d3 * d3))));
     x2.add(fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w))));
   }
-  cta_sum2<256>((double)dx2.s - (double)dx2.c, (double)x2.s - (double)x2.c, partials + 2 * blockIdx.x);
+  cta_sum2<256>(ff{dx2.s, -dx2.c}, ff{x2.s, -x2.c}, partials + 2 * blockIdx.x);
 }
 
 int primal_parts(const Cube&) { return kPrimalCTAs; }
