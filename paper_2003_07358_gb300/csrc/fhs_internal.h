@@ -151,8 +151,9 @@ struct Scratch {
 // Streams, events and scratch of one further lane of an iteration.
 struct Lane {
   Scratch s;
-  cudaStream_t stream = nullptr, aux = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;   // this lane's fork to / join from its aux stream
+  cudaStream_t stream = nullptr, aux = nullptr, aux2 = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;   // this lane's fork to its aux streams, join from aux
+  cudaEvent_t ev_join2 = nullptr;                     // join from aux2
   cudaEvent_t ev_done = nullptr;                      // the lane's last work (joined by the first lane)
 };
 
@@ -174,6 +175,10 @@ struct fhs_ctx {
   // run beside the data term (they read Xcheck and P only) and join before the update of A
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // third stream: the sparsity duals down to the last synthesis level (they read Xcheck and
+  // W only), where the iteration's launches do not fill the GPU one by one
+  cudaStream_t aux2 = nullptr;
+  cudaEvent_t ev_join2 = nullptr;
   // further lanes of an iteration (fast path, two or more cubes): cube c runs on lane
   // lane_of[c]; lane k > 0 has its own streams, events and scratch in xl[k - 1]
   int lanes = 1;                   // requested lanes (fhs_set_lanes)
@@ -260,6 +265,10 @@ void launch_l21_weights(const Cube& cb, const float* coef, float* theta, cudaStr
 // fused analysis + l2,1 dual (+ synthesis into A), or weights mode (theta_out)
 void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, const float* theta, float* A,
                       float* theta_out, bool weights, cudaStream_t st);
+// its two halves: everything that reads x (Xcheck) and W only, then A += kappa Psi W
+void launch_sara_dual(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, const float* theta, float* theta_out,
+                      bool weights, cudaStream_t st);
+void launch_sara_fin(fhs_ctx* ctx, const Cube& cb, const float* W, float* A, cudaStream_t st);
 bool sara_fast_supported(const Cube& cb);
 
 // nuclear (nuclear.cu)

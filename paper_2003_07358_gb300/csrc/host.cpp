@@ -634,6 +634,7 @@ void free_scratch(Scratch& s) {
 void free_lane(fhs_ctx* ctx, Lane& x, int slot) {
   if (x.stream) cudaStreamSynchronize(x.stream);
   if (x.aux) cudaStreamSynchronize(x.aux);
+  if (x.aux2) cudaStreamSynchronize(x.aux2);
   Scratch& s = x.s;
   void* ps[] = {s.grid, s.pack, s.coef, s.t0, s.t1, s.t2, s.t3, s.img, s.vis, s.vis2, s.red, s.gram, s.nucM,
                 s.blk_scale, s.blk_out, s.ll1, s.ll2, s.ll3};
@@ -642,7 +643,8 @@ void free_lane(fhs_ctx* ctx, Lane& x, int slot) {
   s = Scratch();
   if (x.stream) cudaStreamDestroy(x.stream);
   if (x.aux) cudaStreamDestroy(x.aux);
-  for (cudaEvent_t e : {x.ev_fork, x.ev_join, x.ev_done})
+  if (x.aux2) cudaStreamDestroy(x.aux2);
+  for (cudaEvent_t e : {x.ev_fork, x.ev_join, x.ev_join2, x.ev_done})
     if (e) cudaEventDestroy(e);
   x = Lane();
   for (Cube& cb : ctx->cubes) cb.tm_grid[slot] = nullptr;
@@ -724,6 +726,8 @@ bool make_lane(fhs_ctx* ctx) {
   if (ok) {
     ok = cudaStreamCreateWithFlags(&x.stream, cudaStreamNonBlocking) == cudaSuccess &&
          cudaStreamCreateWithFlags(&x.aux, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaStreamCreateWithFlags(&x.aux2, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&x.ev_join2, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&x.ev_fork, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&x.ev_join, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&x.ev_done, cudaEventDisableTiming) == cudaSuccess;
@@ -800,6 +804,18 @@ void ensure_coef(fhs_ctx* ctx) {
 
 bool use_fast(fhs_ctx* ctx, const Cube& cb) { return ctx->path == FHS_PATH_FAST && sara_fast_supported(cb); }
 
+// Whether the sparsity duals of an iteration run on a stream of their own beside the data
+// term: with one lane, up to 2^25 pixel-channels, where launches of either do not fill the
+// GPU for long (64^2 x 4 113 -> 71 us per iteration, 256^2 x 20 429 -> 400, 512^2 x 16 with
+// DDEs 2.99 -> 2.92 ms, 1024^2 x 32 6.77 -> 6.63 ms alone and no change among others).  At
+// 4096^2 x 4 it cost 1.3 % and, with the GPU already shared by four lanes, 1.2 %.
+constexpr int64_t kSidePixels = (int64_t)1 << 25;
+
+bool sara_beside_data(fhs_ctx* ctx, const Cube& cb) {
+  return use_fast(ctx, cb) && cb.sara_fast && lanes_in_use(ctx) == 1 &&
+         (int64_t)cb.L * cb.n1 * cb.n2 <= kSidePixels;
+}
+
 void sara_dual(fhs_ctx* ctx, const Cube& cb, const float* xcheck, float* W, const float* theta, float* A) {
   cudaStream_t st = ctx->stream;
   if (use_fast(ctx, cb) && cb.sara_fast) {
@@ -850,6 +866,13 @@ void pdfb_iteration_cube(fhs_ctx* ctx, int c, const fhs_iterate& a) {
     launch_nuclear_gram_eig(ctx, cb, a.Xcheck, a.state.P, a.state.theta_bar, false, nullptr, ctx->aux);
     check_launch("nuclear Gram");
     FHS_CUDA(cudaEventRecord(ctx->ev_join, ctx->aux));
+    const bool side = sara_beside_data(ctx, cb);
+    if (side) {
+      FHS_CUDA(cudaStreamWaitEvent(ctx->aux2, ctx->ev_fork, 0));
+      launch_sara_dual(ctx, cb, a.Xcheck, a.state.W, a.state.theta, nullptr, false, ctx->aux2);
+      check_launch("sara dual");
+      FHS_CUDA(cudaEventRecord(ctx->ev_join2, ctx->aux2));
+    }
     launch_fft_forward(ctx, cb, a.X, ctx->s.grid, st);
     // preconditioned duals (Section 3.2): the degridder forms d = U^-1 v + Phi x_check - y
     if (cb.n_sub > 0) launch_vis_scale((float2*)a.state.v, cb.d_U, cb.n_vis, true, st);
@@ -888,7 +911,13 @@ void pdfb_iteration_cube(fhs_ctx* ctx, int c, const fhs_iterate& a) {
     FHS_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));          // join
     launch_nuclear_apply(ctx, cb, a.Xcheck, a.state.P, A, st);
     check_launch("nuclear dual");
-    sara_dual(ctx, cb, a.Xcheck, a.state.W, a.state.theta, A);
+    if (side) {
+      FHS_CUDA(cudaStreamWaitEvent(st, ctx->ev_join2, 0));
+      launch_sara_fin(ctx, cb, a.state.W, A, st);
+      check_launch("sara synthesis");
+    } else {
+      sara_dual(ctx, cb, a.Xcheck, a.state.W, a.state.theta, A);
+    }
     launch_primal(cb, a.X, a.Xcheck, A, stat, pp, st);
     check_launch("primal");
   }
@@ -901,6 +930,8 @@ void swap_lane(fhs_ctx* ctx, Lane& x) {
   std::swap(ctx->s, x.s);
   std::swap(ctx->stream, x.stream);
   std::swap(ctx->aux, x.aux);
+  std::swap(ctx->aux2, x.aux2);
+  std::swap(ctx->ev_join2, x.ev_join2);
   std::swap(ctx->ev_fork, x.ev_fork);
   std::swap(ctx->ev_join, x.ev_join);
 }
@@ -939,13 +970,18 @@ void pdfb_iteration(fhs_ctx* ctx, const fhs_iterate* it) {
 void reweight_cube(fhs_ctx* ctx, const Cube& cb, const float* x, float* theta, float* theta_bar) {
   cudaStream_t st = ctx->stream;
   ensure_coef(ctx);
+  // the facet Grams and eigen-solves (theta_bar) beside the wavelet weights (theta)
+  FHS_CUDA(cudaEventRecord(ctx->ev_fork, st));
+  FHS_CUDA(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
+  launch_nuclear(ctx, cb, x, nullptr, nullptr, nullptr, true, theta_bar, ctx->aux);
+  FHS_CUDA(cudaEventRecord(ctx->ev_join, ctx->aux));
   if (use_fast(ctx, cb) && cb.sara_fast) {
     launch_sara_fast(ctx, cb, x, nullptr, nullptr, nullptr, theta, true, st);
   } else {
     launch_sara_analysis(ctx, cb, x, ctx->s.coef, st);
     launch_l21_weights(cb, ctx->s.coef, theta, st);
   }
-  launch_nuclear(ctx, cb, x, nullptr, nullptr, nullptr, true, theta_bar, st);
+  FHS_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
   check_launch("reweight");
 }
 
@@ -1487,6 +1523,8 @@ fhs_status fhs_create(const fhs_cube_desc* cubes, int32_t ncubes, void* stream, 
     FHS_CUDA(cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking));
     FHS_CUDA(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
     FHS_CUDA(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
+    FHS_CUDA(cudaStreamCreateWithFlags(&ctx->aux2, cudaStreamNonBlocking));
+    FHS_CUDA(cudaEventCreateWithFlags(&ctx->ev_join2, cudaEventDisableTiming));
     if (tune)
       for (int c = 0; c < ncubes; ++c) tune_after_build(ctx, c, choice[c], keys[c]);
     FHS_CUDA(cudaStreamSynchronize(ctx->stream));
@@ -1497,7 +1535,8 @@ fhs_status fhs_create(const fhs_cube_desc* cubes, int32_t ncubes, void* stream, 
     if (ctx->d_tw) cudaFree(ctx->d_tw);
     if (ctx->gstream) cudaStreamDestroy(ctx->gstream);
     if (ctx->aux) cudaStreamDestroy(ctx->aux);
-    for (cudaEvent_t e2 : {ctx->ev_in, ctx->ev_out, ctx->ev_fork, ctx->ev_join})
+    if (ctx->aux2) cudaStreamDestroy(ctx->aux2);
+    for (cudaEvent_t e2 : {ctx->ev_in, ctx->ev_out, ctx->ev_fork, ctx->ev_join, ctx->ev_join2})
       if (e2) cudaEventDestroy(e2);
     delete ctx;
     return e.st;
@@ -1518,8 +1557,13 @@ fhs_status fhs_destroy(fhs_ctx* ctx) {
     cudaStreamSynchronize(ctx->aux);
     cudaStreamDestroy(ctx->aux);
   }
+  if (ctx->aux2) {
+    cudaStreamSynchronize(ctx->aux2);
+    cudaStreamDestroy(ctx->aux2);
+  }
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+  if (ctx->ev_join2) cudaEventDestroy(ctx->ev_join2);
   free_lanes(ctx, 1);
   if (ctx->ev_lanes_fork) cudaEventDestroy(ctx->ev_lanes_fork);
   for (cudaEvent_t e : ctx->tev) cudaEventDestroy(e);

@@ -544,10 +544,17 @@ __global__ void __launch_bounds__(SynCfg<T>::NT, T == 64 ? 3 : 2) k_synfin(const
 static bool syn_large_tiles(int64_t ctas64) { return ctas64 >= 2LL * 3 * num_sms(); }
 
 // ------------------------------------------------------------- launchers
-// Analysis of every basis and level into the coefficient buffer, the l2,1 dual (or
-// weights), then (dual mode) the synthesis accumulated into A.
+// launch_sara_dual: analysis of every basis and level into the coefficient buffer, the l2,1
+// dual (or weights), then (dual mode) the synthesis down to the LL1 bands; launch_sara_fin:
+// level 1 of the synthesis and the Dirac block, accumulated into A.
 void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, const float* theta, float* A,
                       float* theta_out, bool weights, cudaStream_t st) {
+  launch_sara_dual(ctx, cb, x, W, theta, theta_out, weights, st);
+  if (!weights) launch_sara_fin(ctx, cb, W, A, st);
+}
+
+void launch_sara_dual(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, const float* theta, float* theta_out,
+                      bool weights, cudaStream_t st) {
   const SaraLayout& S = cb.sara;
   const int L = cb.L;
   float* coef = ctx->s.coef;
@@ -626,7 +633,6 @@ void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, co
     note_launches(1);
   }
   if (weights) return;
-  SynFin2 fin;
   float* slots = ctx->s.ll1;
   // levels 4 -> 2: one launch per level over the tiles of every basis; the synthesised
   // LL3, LL2 and LL1 bands reuse the analysis slots (s.ll3, s.ll2, s.ll1)
@@ -669,9 +675,17 @@ void launch_sara_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float* W, co
       note_launches(1);
     }
   }
+}
+
+void launch_sara_fin(fhs_ctx* ctx, const Cube& cb, const float* W, float* A, cudaStream_t st) {
+  const SaraLayout& S = cb.sara;
+  const int L = cb.L;
+  SynFin2 fin;
+  int64_t o1 = 0;                                    // the LL1 slots of launch_sara_dual
   for (int b = 0; b < 8; ++b) {
     Syn2& f = fin.lv[b];
-    f.ll = slots + ctx->s.ll1_off[b];
+    f.ll = ctx->s.ll1 + o1;
+    o1 += (int64_t)L * S.rows[b][1] * S.cols[b][1];
     f.W = W;
     f.I = S.I;
     f.off[0] = S.off[b][1][0]; f.off[1] = S.off[b][1][1]; f.off[2] = S.off[b][1][2];
