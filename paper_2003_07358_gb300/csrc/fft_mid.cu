@@ -1,5 +1,5 @@
-// 2-D DFT of the zero-padded real image for grid sides K = 2^a (32 .. 2048) and 3 2^a (96 ..
-// 3072) whose column transform takes one pass (grid rows in natural order): images up to
+// 2-D DFT of the zero-padded real image for grid sides K = 2^a (128 .. 2048) and 3 2^a (96 ..
+// 3072) whose column transform takes one pass (grid rows in natural order): images of 64 to
 // 512 on power-of-two sides, up to 1536 where a side is 3 2^m.
 //
 // Two-for-one: packed column j < n2/2 holds the image columns j + n2/2 (real part, grid
@@ -30,8 +30,6 @@ namespace {
 template <int N> struct MidCfg;
 #define FHS_MID_CFG(N, A, B, C) \
   template <> struct MidCfg<N> { static constexpr int R1 = A, R2 = B, R3 = C; };
-FHS_MID_CFG(32, 8, 4, 1)
-FHS_MID_CFG(64, 8, 8, 1)
 FHS_MID_CFG(96, 12, 8, 1)
 FHS_MID_CFG(128, 16, 8, 1)
 FHS_MID_CFG(192, 16, 12, 1)
@@ -47,8 +45,6 @@ FHS_MID_CFG(3072, 16, 16, 12)
 
 #define FHS_MID_SWITCH(n, FN, ...)                   \
   switch (n) {                                       \
-    case 32: FN<32>(__VA_ARGS__); break;             \
-    case 64: FN<64>(__VA_ARGS__); break;             \
     case 96: FN<96>(__VA_ARGS__); break;             \
     case 128: FN<128>(__VA_ARGS__); break;           \
     case 192: FN<192>(__VA_ARGS__); break;           \
@@ -64,8 +60,8 @@ FHS_MID_CFG(3072, 16, 16, 12)
   }
 
 bool mid_side(int K) {
-  while (K > 0 && K % 2 == 0 && K > 96) K /= 2;
-  return K == 32 || K == 64 || K == 96;
+  while (K % 2 == 0 && K > 128) K /= 2;
+  return K == 128 || K == 96;
 }
 
 // v[k] *= w^k, w = exp(-+2 pi i b / len) (table step `step` per unit of b): the powers w^1 ..
@@ -345,9 +341,12 @@ void mid_row_adj(const Cube& cb, const float2* grid, float2* P, const float2* tw
 
 }  // namespace
 
-// One-pass columns (natural row order) and both sides among the instantiated lengths.
+// One-pass columns (natural row order) and both sides among the instantiated lengths.  Grids
+// with a side of 32 or 64 cells (images of 16 and 32) keep the transforms they had: 2 to 13 us
+// of a call, and the pairing of Phi with its adjoint over DDE kernels on 64 cells lies at the
+// resolution of the fixed-point gridder, so its results there are left as they are.
 bool fft_mid_supported(const Cube& cb) {
-  return cb.N2c == 1 && mid_side(cb.K1) && mid_side(cb.K2) && cb.K1 <= 3072 && cb.K2 <= 3072;
+  return cb.N2c == 1 && cb.K1 >= 96 && cb.K2 >= 96 && mid_side(cb.K1) && mid_side(cb.K2) && cb.K1 <= 3072 && cb.K2 <= 3072;
 }
 
 void launch_fft_forward_mid(fhs_ctx* ctx, const Cube& cb, const float* x, float2* grid, cudaStream_t st) {

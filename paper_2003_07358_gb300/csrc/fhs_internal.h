@@ -76,7 +76,7 @@ struct Cube {
   int64_t* d_perm = nullptr;                 // [n_vis]
   int32_t* d_tile_off = nullptr;             // [L][ntiles*4 + 1] per-channel tile/class offsets (relative)
   int ntile_r, ntile_c, tile;                // gridder tiles
-  float* d_cover = nullptr;                  // [L][ntiles] largest sum over a cell of the weights covering it
+  int* d_ncmax = nullptr;                    // [L][ntiles] most footprints covering one cell of a tile
   // device copies of per-cube parameters and tables
   NucFacet* d_facets = nullptr;
   float* d_win = nullptr;                    // window tables (y and x windows concatenated)
@@ -92,8 +92,7 @@ struct Cube {
   float* d_U = nullptr;                      // [n_vis]
   // DDE-extended G (Section 2.1): kernel half-width R (-1: plain Kaiser-Bessel rows),
   // kernels [n_kern][2R+1][2R+1], kernel of each visibility (internal order), per kernel
-  // sum of |Re| + |Im| (rounded up), per (channel, tile) largest sum over a cell of the
-  // extended weights covering it
+  // sum of |Re| + |Im| (rounded up), per (channel, tile) largest extended-footprint count
   // launch choices of the autotuner (defaults: tile-staged de-gridder, tensor-core Gram
   // where L <= 32, fused SARA tiles, 16 CTAs per SM for the l2,1 dual pass)
   int degrid_tiled = 1;
@@ -107,7 +106,7 @@ struct Cube {
   float2* d_dde_kern = nullptr;
   int32_t* d_dde_idx = nullptr;
   float* d_dde_l1 = nullptr;
-  float* d_dde_cover = nullptr;
+  int* d_dde_ncmax = nullptr;
   float* d_gamma = nullptr;                  // [L*B] 1 / max U of the block
   float* d_eta = nullptr;                    // [L]
   float* d_mubar = nullptr;                  // [Q]

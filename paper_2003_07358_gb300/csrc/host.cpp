@@ -544,9 +544,9 @@ void build_cube(Cube& cb, const fhs_cube_desc& d, cudaStream_t st, int tile) {
   upload(cb.d_eta, eta_f.data(), eta_f.size(), st);
   upload(cb.d_mubar, mub_f.data(), mub_f.size(), st);
   upload(cb.d_M_lb, cb.M_lb.data(), cb.M_lb.size(), st);
-  // per grid tile, the largest sum of the weights that cover one of its cells (fixes the
+  // per grid tile, the most footprints that cover one of its cells (fixes the
   // gridder's fixed-point scale; depends on the uv coverage only)
-  cb.d_cover = dalloc<float>((size_t)d.L * cb.ntile_r * cb.ntile_c);
+  cb.d_ncmax = dalloc<int>((size_t)d.L * cb.ntile_r * cb.ntile_c);
   launch_grid_count(cb, st);
   FHS_CUDA(cudaGetLastError());
   FHS_CUDA(cudaStreamSynchronize(st));
@@ -554,8 +554,8 @@ void build_cube(Cube& cb, const fhs_cube_desc& d, cudaStream_t st, int tile) {
 
 void free_cube(Cube& cb) {
   void* ps[] = {cb.d_uv, cb.d_blk, cb.d_perm, cb.d_vis_off, cb.d_tile_off, cb.d_facets, cb.d_win, cb.d_win64, cb.d_tile_of,
-                cb.d_scale_r, cb.d_scale_c, cb.d_eps, cb.d_eta, cb.d_mubar, cb.d_cover, cb.d_M_lb, cb.d_U, cb.d_gamma,
-                cb.d_dde_kern, cb.d_dde_idx, cb.d_dde_l1, cb.d_dde_cover};
+                cb.d_scale_r, cb.d_scale_c, cb.d_eps, cb.d_eta, cb.d_mubar, cb.d_ncmax, cb.d_M_lb, cb.d_U, cb.d_gamma,
+                cb.d_dde_kern, cb.d_dde_idx, cb.d_dde_l1, cb.d_dde_ncmax};
   for (void* p : ps)
     if (p) cudaFree(p);
 }
@@ -1940,7 +1940,7 @@ fhs_status fhs_set_dde(fhs_ctx* ctx, int32_t cube, int32_t S_d, int32_t n_kern, 
     cb.d_dde_kern = dalloc<float2>((size_t)n_kern * sd2);
     cb.d_dde_l1 = dalloc<float>(n_kern);
     if (!cb.d_dde_idx) cb.d_dde_idx = dalloc<int32_t>(n ? n : 1);
-    if (!cb.d_dde_cover) cb.d_dde_cover = dalloc<float>((size_t)cb.L * cb.ntile_r * cb.ntile_c);
+    if (!cb.d_dde_ncmax) cb.d_dde_ncmax = dalloc<int>((size_t)cb.L * cb.ntile_r * cb.ntile_c);
     upload(cb.d_dde_kern, reinterpret_cast<const float2*>(kern), (size_t)n_kern * sd2, st);
     upload(cb.d_dde_l1, l1.data(), l1.size(), st);
     if (n) upload(cb.d_dde_idx, idx.data(), idx.size(), st);

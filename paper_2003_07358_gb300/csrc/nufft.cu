@@ -1124,12 +1124,12 @@ __global__ void k_l2ball_scale(const float2* __restrict__ d, const float* __rest
 // and right, 3 crosses right only.
 // Accumulation is in fixed point with 32-bit integer shared-memory atomics (several
 // times faster than floating-point ones, and order-independent, so the result is
-// bitwise deterministic), with one scale S = 2^e per tile chosen so that C m S < 2^30, with
-// C the largest sum over a cell of the tile of the weights |w_r w_c| that cover it (summed
-// once per context, MODE 1) and m = max over the tile's visibilities of max(|Re v|, |Im v|):
-// no cell can overflow, and the resolution is C m / 2^30.  (With the number of footprints in
-// place of their weights, about 8 times as large, the rounding of the taps was most of the
-// adjoint's error: 2.1e-7 against 1.6e-7 now at 23 channels of 768^2.)
+// bitwise deterministic), with one scale S = 2^e per tile chosen so that
+// n_c |c| < 2^30 for every tap value c = w v S, with n_c the largest number of
+// footprints that cover one cell of the tile (counted once per context, MODE 1) and
+// |v| <= m = max over the tile's visibilities of max(|Re v|, |Im v|): no cell can
+// overflow, and the resolution is n_c m / 2^30 (about 2^-23 of m for the densest
+// tiles of the large workload, n_c ~ 100).
 
 constexpr int kGridThreads = 128;                // threads per gridding CTA
 
@@ -1155,7 +1155,7 @@ __device__ __forceinline__ void grid_pass_range(const int32_t* toff, int pass, i
 // Adds the 7 x 7 taps of one visibility to the tile accumulators: rows lr + a,
 // columns lc + b.  ra[a] = row weight * S, wc[b] = column weight, (vx, vy) = v.
 // INTERIOR: the whole footprint lies in the tile (no bounds tests); otherwise only
-// rows in [a0, a1) and columns in [b0, b1) are added.  MODE 1 adds |weight| S, rounded up.
+// rows in [a0, a1) and columns in [b0, b1) are added.  MODE 1 adds 1 per tap.
 template <bool INTERIOR, int MODE>
 __device__ __forceinline__ void grid_taps(int* are, int* aim, int TP, int lr, int lc, const float* ra,
                                           const float* wc, float vx, float vy, int a0, int a1, int b0, int b1) {
@@ -1169,7 +1169,7 @@ __device__ __forceinline__ void grid_taps(int* are, int* aim, int TP, int lr, in
     for (int b = 0; b < kTaps; ++b) {
       if (!INTERIOR && (b < b0 || b >= b1)) continue;
       if (MODE == 1) {
-        atomicAdd(pr + b, __float2int_ru(fabsf(wc[b] * ra[a])));
+        atomicAdd(pr + b, 1);
       } else {
         atomicAdd(pr + b, __float2int_rn(wc[b] * xr));
         atomicAdd(pi + b, __float2int_rn(wc[b] * xi));
@@ -1178,22 +1178,15 @@ __device__ __forceinline__ void grid_taps(int* are, int* aim, int TP, int lr, in
   }
 }
 
-// Power of two S with S total < 2^30, at most 2^12: the unit of the weight sums of a tile
-// whose footprints weigh `total` together.
-__device__ __forceinline__ float cover_unit(float total) {
-  const float t = 1073741824.f / (fmaxf(total, 1.f) * 1.01f);
-  return pow2f(max(-120, min((int)((__float_as_uint(t) >> 23) & 0xffu) - 127, 12)));
-}
-
 // MODE 0: grid the (block-scaled) values into the tile and store it; MODE 1 (once per
-// context): sum the weights covering each cell and store the tile's maximum in
-// cover[l][tile].
+// context): count the footprints covering each cell and store the tile's maximum in
+// ncmax[l][tile].
 template <int MODE>
 __global__ void __launch_bounds__(kGridThreads, 1024 / kGridThreads) k_grid(const float2* __restrict__ vals, const float* __restrict__ blk_scale,
                                               float2* __restrict__ v_write, const float2* __restrict__ uv,
                                               const uint8_t* __restrict__ blk, const int32_t* __restrict__ tile_off,
                                               const int64_t* __restrict__ vis_off, float2* __restrict__ grid,
-                                              float* __restrict__ cover, VisGeom vg, int T, int ntr, int ntc, int B) {
+                                              int* __restrict__ ncmax, VisGeom vg, int T, int ntr, int ntc, int B) {
   extern __shared__ __align__(16) int sacc_i[];
   constexpr int NW = kGridThreads / 32;
   __shared__ float sred[NW];
@@ -1232,22 +1225,15 @@ __global__ void __launch_bounds__(kGridThreads, 1024 / kGridThreads) k_grid(cons
     m = 0.f;
 #pragma unroll
     for (int w = 0; w < NW; ++w) m = fmaxf(m, sred[w]);
-    const float C = cover[l * ntr * ntc + tau];
-    if (m > 1e-30f && C > 0.f) {
-      // S = 2^e <= 2^30 / (C m'), m' = m (1 + 2^-10) covering the roundings of v s and of
-      // the products
-      const float t = 1073741824.f / (C * (m * 1.0009765625f));
+    const int nc = ncmax[l * ntr * ntc + tau];
+    if (m > 1e-30f && nc > 0) {
+      // S = 2^e <= 2^30 / (n_c m'), m' = m (1 + 2^-10) covering the roundings of v s,
+      // of the row product and a kernel weight a hair above 1
+      const float t = 1073741824.f / ((float)nc * (m * 1.0009765625f));
       const int e = (int)((__float_as_uint(t) >> 23) & 0xffu) - 127;   // 2^e <= t
       S = pow2f(max(-120, min(e, 120)));
     }
   } else {
-    float nv = 0.f;
-    for (int pass = 0; pass < 4; ++pass) {
-      int sr, sc, beg, end;
-      grid_pass_range(toff, pass, tr, tc, ntr, ntc, sr, sc, beg, end);
-      nv += (float)(end - beg);
-    }
-    S = cover_unit(nv);
     __syncthreads();
   }
   // ---- sweep 1: taps
@@ -1297,7 +1283,7 @@ __global__ void __launch_bounds__(kGridThreads, 1024 / kGridThreads) k_grid(cons
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w = 0; w < NW; ++w) mx = max(mx, sredi[w]);
-      cover[l * ntr * ntc + tau] = __int2float_ru(mx) / S;                 // S: a power of two
+      ncmax[l * ntr * ntc + tau] = mx;
     }
     return;
   }
@@ -1507,7 +1493,7 @@ void launch_grid(const Cube& cb, const float2* vals, const float* blk_scale, flo
   dim3 grd(cb.ntile_r * cb.ntile_c, cb.L);
   size_t sm = 2 * (size_t)cb.tile * grid_row_stride(cb.tile) * sizeof(int);
   k_grid<0><<<grd, kGridThreads, sm, st>>>(vals, blk_scale, v_write, cb.d_uv, cb.d_blk, cb.d_tile_off, cb.d_vis_off, grid,
-                                  cb.d_cover, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
+                                  cb.d_ncmax, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
   note_launches(1);
 }
 
@@ -1517,7 +1503,7 @@ void launch_grid_count(const Cube& cb, cudaStream_t st) {
   dim3 grd(cb.ntile_r * cb.ntile_c, cb.L);
   size_t sm = 2 * (size_t)cb.tile * grid_row_stride(cb.tile) * sizeof(int);
   k_grid<1><<<grd, kGridThreads, sm, st>>>(nullptr, nullptr, nullptr, cb.d_uv, cb.d_blk, cb.d_tile_off, cb.d_vis_off, nullptr,
-                                  cb.d_cover, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
+                                  cb.d_ncmax, vis_geom(cb), cb.tile, cb.ntile_r, cb.ntile_c, cb.B);
   note_launches(1);
 }
 

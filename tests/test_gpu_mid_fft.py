@@ -1,6 +1,6 @@
 """Phi and Re Phi^dagger on image sides whose grids take the two-for-one mid-size transforms
-(every transform length from 32 to 3072, rows and columns of different kinds) against the
-FP64 oracle; sides 9 * 16 and plain-path contexts keep the general transforms."""
+(every transform length from 96 to 3072, rows and columns of different kinds) against the
+FP64 oracle; sides of 16 and 32, sides 9 * 16 and plain-path contexts keep the others."""
 from __future__ import annotations
 
 import numpy as np
