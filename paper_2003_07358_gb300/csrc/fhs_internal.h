@@ -225,7 +225,7 @@ void launch_degrid(const Cube& cb, const float2* grid, float2* out, bool tiled, 
 void encode_degrid_maps(fhs_ctx* ctx);
 void encode_cube_maps(Cube& cb, const float2* grid, int slot);
 void launch_fill_pattern(float* p, int64_t n, uint32_t seed, cudaStream_t st);
-void launch_gram(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, bool tc, cudaStream_t st);
+int launch_gram(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, bool tc, cudaStream_t st);
 int num_sms();   // streaming multiprocessors of the current device
 unsigned read_device_status(bool clear);
 int degrid_tiled_parts(const Cube& cb);

@@ -23,6 +23,10 @@
 // 32 channels (L <= 32), or 2 half-chunks of 512 pixels x 4 slices x 16 channels
 // (L <= 16; the two diagonal 64 x 64 blocks of C are used).
 //
+// Bound by latency, two CTAs per SM: of about 23 us a chunk of 16 channels 10 are its loads,
+// 8 the slicing stages, 3 the epilogue (1.50 ms at 4096^2 x 16 with 256 facets; 2.23 ms when
+// the loads waited for one another and the epilogue's exchange had 32-way bank conflicts).
+//
 // Layout of an operand stage in shared memory (K-major, no swizzle, bf16): 4 MMA
 // K-steps of 16; within a step, core matrices of 8 rows x 16 bytes, adjacent in K at
 // 128 B (leading byte offset) and in rows at 256 B (stride byte offset).  A = B (the
@@ -131,12 +135,26 @@ __device__ __forceinline__ void tc_slices2(float z0, float z1, float scale, uint
   }
 }
 
-// Value of facet pixel (rr, cc) (linear index p < Nq), channel l: D_q Xcheck + P_q.
-__device__ __forceinline__ float tc_z(const float* __restrict__ xc, const float* __restrict__ P, const NucFacet& f,
-                                      float d, size_t xo, size_t N, int Nq, int use_P, int p, int l) {
-  float v = d * xc[(size_t)l * N + xo];
-  if (use_P) v += P[f.p_off + (size_t)l * Nq + p];
-  return v;
+// z = d Xcheck + P of one facet pixel (linear index p, image offset xo), channels l0 ..
+// l0 + 15 (zero from L on): the 32 loads are in flight together (a test of l < L around each
+// pair made them wait for one another: 17 us of a chunk's 29).
+__device__ __forceinline__ void tc_z16(const float* __restrict__ xc, const float* __restrict__ P, const NucFacet& f,
+                                       float d, size_t xo, size_t N, int Nq, int use_P, int p, int l0, int L,
+                                       float (&z)[16]) {
+  const float* xp = xc + (size_t)l0 * N + xo;
+  float q[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) z[l] = l0 + l < L ? xp[(size_t)l * N] : 0.f;
+  if (use_P) {
+    const float* pp = P + f.p_off + (size_t)l0 * Nq + p;
+#pragma unroll
+    for (int l = 0; l < 16; ++l) q[l] = l0 + l < L ? pp[(size_t)l * Nq] : 0.f;
+  } else {
+#pragma unroll
+    for (int l = 0; l < 16; ++l) q[l] = 0.f;
+  }
+#pragma unroll
+  for (int l = 0; l < 16; ++l) z[l] = d * z[l] + q[l];
 }
 
 // LP = 16 (two half-chunks side by side) or 32 (one chunk).  Grid (chunks, facets).
@@ -206,8 +224,10 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(const float* __restri
         const int rr = p / w, cc = p - rr * w;
         const float d = win[f.wy_off + rr] * win[f.wx_off + cc];
         const size_t xo = (size_t)(f.r0 + rr) * n2 + (f.c0 + cc);
+        float z[16];
+        tc_z16(xc, P, f, d, xo, N, Nq, use_P, p, 0, L, z);
 #pragma unroll
-        for (int l = 0; l < LP; ++l) zs[l * kTcChunk + qq] = l < L ? tc_z(xc, P, f, d, xo, N, Nq, use_P, p, l) : 0.f;
+        for (int l = 0; l < LP; ++l) zs[l * kTcChunk + qq] = z[l];
       } else {
 #pragma unroll
         for (int l = 0; l < LP; ++l) zs[l * kTcChunk + qq] = 0.f;
@@ -249,8 +269,12 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(const float* __restri
         const int xo = (f.r0 + rr) * n2 + (f.c0 + cc);     // < 2^24 (n1, n2 <= 4096)
         px = make_int2(__float_as_int(d), xo);
 #pragma unroll
-        for (int l = 0; l < LP; ++l)
-          if (l < L) mx[h][l] = fmaxf(mx[h][l], fabsf(tc_z(xc, P, f, d, (size_t)xo, N, Nq, use_P, p, l)));
+        for (int l0 = 0; l0 < LP; l0 += 16) {
+          float z[16];
+          tc_z16(xc, P, f, d, (size_t)xo, N, Nq, use_P, p, l0, L, z);
+#pragma unroll
+          for (int l = 0; l < 16; ++l) mx[h][l0 + l] = fmaxf(mx[h][l0 + l], fabsf(z[l]));
+        }
       }
       s_px[tid + j * kTcThreads] = px;
     }
@@ -418,16 +442,18 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(const float* __restri
     }
   }
   // integer sums: exact in any order; the first column half writes, the second adds
+  // (entry [h][k][b][a]: the lanes of a warp hold consecutive a, so every access is free of
+  // bank conflicts; with [a][b] each was 32-way)
   long long* ired = reinterpret_cast<long long*>(red);
-  long long* r = ired + (((size_t)h * 4 + k) * LP + a) * LP;
+  long long* r = ired + (((size_t)h * 4 + k) * LP) * LP + a;
   if (half == 0) {
 #pragma unroll
-    for (int b = 0; b < LP; ++b) r[b] = T[b];
+    for (int b = 0; b < LP; ++b) r[b * LP] = T[b];
   }
   __syncthreads();
   if (half == 1) {
 #pragma unroll
-    for (int b = 0; b < LP; ++b) r[b] += T[b];
+    for (int b = 0; b < LP; ++b) r[b * LP] += T[b];
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
   __syncthreads();
@@ -435,11 +461,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(const float* __restri
   // sum over slices k (exact), then per half-chunk the scales 2^(e_a + 1) 2^(e_b + 1) 2^-42
   double* out = part + ((size_t)q * nchunk_max + chunk) * L * L;
   for (int ab = tid; ab < L * L; ab += kTcThreads) {
-    const int a2 = ab / L, b2 = ab % L;
+    const int b2 = ab / L, a2 = ab % L;
     double g = 0.0;
     for (int hh = 0; hh < NH; ++hh) {
       long long gh = 0;
-      for (int kk = 0; kk < 4; ++kk) gh += ired[(((size_t)hh * 4 + kk) * LP + a2) * LP + b2];
+      for (int kk = 0; kk < 4; ++kk) gh += ired[(((size_t)hh * 4 + kk) * LP + b2) * LP + a2];
       g += (double)gh * (s_pow[hh][a2] * s_pow[hh][b2] * 0x1p-42);
     }
     out[ab] = g;

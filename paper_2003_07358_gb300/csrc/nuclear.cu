@@ -196,6 +196,85 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
   }
 }
 
+// Partial Grams of up to LM <= 8 channels: a thread streams pixels (chunks blockIdx.x,
+// blockIdx.x + parts, ... of the facet) and keeps every entry of the upper triangle as a
+// float pair in registers (the products and sums of k_gram), so a pixel is read once and
+// nothing is staged; the CTA adds its threads' pairs in a fixed order.  Output slot
+// blockIdx.x, as k_gram_sum leaves it.  The tensor-core kernel pads such facets to 16
+// channels and pays a chunk's slicing and epilogue all the same: 1.61 ms at 4 channels of
+// 4096^2 (256 facets), here 0.25 ms.
+template <int LM>
+__global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc, const float* __restrict__ P,
+                                                    const NucFacet* __restrict__ facets,
+                                                    const float* __restrict__ win, int n1, int n2, int L, int use_P,
+                                                    double* __restrict__ part, int nchunk_max, int parts) {
+  constexpr int NP = LM * (LM + 1) / 2, LD = NP | 1, SH = 128 / NP;   // shares of the final sum
+  __shared__ float2 red[128 * LD];
+  __shared__ float2 red2[SH * NP];
+  const int q = blockIdx.y, tid = threadIdx.x;
+  const NucFacet f = facets[q];
+  const int w = f.c1 - f.c0, Nq = (f.r1 - f.r0) * w, nch = (Nq + kGramChunk - 1) / kGramChunk;
+  if ((int)blockIdx.x >= nch) return;
+  const size_t N = (size_t)n1 * n2;
+  float hi[NP], lo[NP];
+#pragma unroll
+  for (int e = 0; e < NP; ++e) hi[e] = lo[e] = 0.f;
+  for (int c = blockIdx.x; c < nch; c += parts) {
+#pragma unroll 2
+    for (int k = 0; k < kGramChunk / 128; ++k) {
+      const int p = c * kGramChunk + k * 128 + tid;
+      const bool in = p < Nq;
+      const int rr = in ? p / w : 0, cc = in ? p - rr * w : 0;
+      const float d = facet_weight(f, win, rr, cc);
+      const float* xp = xc + (size_t)(f.r0 + rr) * n2 + (f.c0 + cc);
+      const float* pp = P + f.p_off + p;
+      float z[LM], u[LM];
+#pragma unroll
+      for (int l = 0; l < LM; ++l) {
+        z[l] = in && l < L ? xp[(size_t)l * N] : 0.f;
+        u[l] = in && use_P && l < L ? pp[(size_t)l * Nq] : 0.f;
+      }
+#pragma unroll
+      for (int l = 0; l < LM; ++l) z[l] = fmaf(d, z[l], u[l]);
+      int e = 0;
+#pragma unroll
+      for (int b = 0; b < LM; ++b)
+#pragma unroll
+        for (int a = 0; a <= b; ++a, ++e) {
+          const float pr = __fmul_rn(z[a], z[b]), pe = __fmaf_rn(z[a], z[b], -pr);
+          float t, er;
+          two_sum(hi[e], pr, t, er);
+          hi[e] = t;
+          lo[e] = __fadd_rn(lo[e], __fadd_rn(er, pe));
+        }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < NP; ++e) {
+    const float h = __fadd_rn(hi[e], lo[e]);
+    red[tid * LD + e] = make_float2(h, __fsub_rn(lo[e], __fsub_rn(h, hi[e])));
+  }
+  __syncthreads();
+  if (tid < SH * NP) {
+    const int e = tid % NP;
+    ff s = {0.f, 0.f};
+    for (int t = tid / NP; t < 128; t += SH) s = ff_add(s, {red[t * LD + e].x, red[t * LD + e].y});
+    red2[tid] = make_float2(s.h, s.l);
+  }
+  __syncthreads();
+  if (tid < NP) {
+    ff s = {0.f, 0.f};
+    for (int t = 0; t < SH; ++t) s = ff_add(s, {red2[t * NP + tid].x, red2[t * NP + tid].y});
+    int b = 0;
+    while ((b + 1) * (b + 2) / 2 <= tid) ++b;
+    const int a = tid - b * (b + 1) / 2;
+    if (b < L) {
+      double* out = part + ((size_t)q * nchunk_max + blockIdx.x) * L * L;
+      out[a * L + b] = out[b * L + a] = ff_val(s);
+    }
+  }
+}
+
 // ------------------------------------------------------------ eigen-solve
 // A GB300 SM issues one FP64 warp instruction per 64 clocks and sub-partition, whatever
 // the number of active lanes (measured: 64 clk per dependent or independent DFMA, 431 for
@@ -592,17 +671,20 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
 }
 
 // Pixel-driven update: each thread owns one pixel; for every facet covering it,
-// z = P_q + D_q x, P_q <- z M_q, A += zeta D_q P_q.  Row b of M_q^T is read as
-// float4 (one load per four FMAs, the same address across the warp).  Up to 16
-// channels the A contributions of all covering facets are summed in shared memory
-// (one slot per thread and channel) and A is read and written once per pixel with all
-// of its loads in flight; above that, A is updated per facet.
+// z = P_q + D_q x, P_q <- z M_q, A += zeta D_q P_q.  BB outputs at a time: their rows of
+// M_q^T are read as float4 (the same address across the warp, L1) against 4 FMAs a row and
+// load, and the BB accesses to A and to P are in flight together.  One output at a time, with
+// A read and written between the outputs above 16 channels, took 0.744 ms at 1024^2 x 32 (64
+// facets) and 1.50 ms at 4096^2 x 16 (256 facets); now 0.378 and 1.33 ms (4.4 TB/s).  BB = 8
+// and the register limits by measurement: at 16 channels BB = 8 spills (1.74 ms at 64
+// registers) or loses occupancy (2.89 ms at 154), BB = 2 1.45 ms; at 32 channels BB = 4 0.419.
 template <int LMAX>
-__global__ void __launch_bounds__(256) k_apply(const float* __restrict__ xc, float* __restrict__ P,
+__global__ void __launch_bounds__(256, LMAX == 16 ? 4 : (LMAX == 32 ? 3 : 2)) k_apply(const float* __restrict__ xc, float* __restrict__ P,
                                                const NucFacet* __restrict__ facets, const float* __restrict__ win,
                                                const float* __restrict__ Mt, int n1, int n2, int L, int Qy, int Qx,
                                                const int* __restrict__ ty_of, const int* __restrict__ tx_of,
                                                float zeta, float* __restrict__ A) {
+  constexpr int BB = LMAX == 32 ? 8 : 4;
   const int c = blockIdx.x * 32 + (threadIdx.x & 31);
   const int r = blockIdx.y * 8 + (threadIdx.x >> 5);
   if (r >= n1 || c >= n2) return;
@@ -610,94 +692,48 @@ __global__ void __launch_bounds__(256) k_apply(const float* __restrict__ xc, flo
   const size_t pix = (size_t)r * n2 + c;
   const int Lp = (L + 3) & ~3;
   const int ty = ty_of[r], tx = tx_of[c];
-  if constexpr (LMAX <= 16) {
-    __shared__ float sacc[LMAX][256];          // this thread's A contributions, per channel
-    float* acc = &sacc[0][threadIdx.x];
-#pragma unroll
-    for (int b = 0; b < LMAX; ++b) acc[b * 256] = 0.f;
-    for (int dy = 0; dy < 2; ++dy) {
-      const int qy = ty + dy;
-      if (qy >= Qy) break;
-      for (int dx = 0; dx < 2; ++dx) {
-        const int qx = tx + dx;
-        if (qx >= Qx) break;
-        const NucFacet f = facets[qy * Qx + qx];
-        if (r < f.r0 || r >= f.r1 || c < f.c0 || c >= f.c1) continue;
-        const int w = f.c1 - f.c0;
-        const int Nq = (f.r1 - f.r0) * w;
-        const int p = (r - f.r0) * w + (c - f.c0);
-        const float d = facet_weight(f, win, r - f.r0, c - f.c0);
-        float* Pq = P + f.p_off;
-        float z[LMAX];
-#pragma unroll
-        for (int l = 0; l < LMAX; ++l) z[l] = (l < L) ? fmaf(d, xc[l * N + pix], Pq[(size_t)l * Nq + p]) : 0.f;
-        const float4* Mq = reinterpret_cast<const float4*>(Mt + (size_t)(qy * Qx + qx) * L * Lp);
-        const float zd = zeta * d;
 #pragma unroll 1
-        for (int b = 0; b < L; ++b) {
-          const float4* row = Mq + (size_t)b * (Lp / 4);
-          float s = 0.f;
+  for (int d4 = 0; d4 < 4; ++d4) {
+    const int qy = ty + (d4 >> 1), qx = tx + (d4 & 1);
+    if (qy >= Qy || qx >= Qx) continue;
+    const NucFacet f = facets[qy * Qx + qx];
+    if (r < f.r0 || r >= f.r1 || c < f.c0 || c >= f.c1) continue;
+    const int w = f.c1 - f.c0;
+    const int Nq = (f.r1 - f.r0) * w;
+    const int p = (r - f.r0) * w + (c - f.c0);
+    const float d = facet_weight(f, win, r - f.r0, c - f.c0);
+    float* Pq = P + f.p_off + p;
+    float z[LMAX];
 #pragma unroll
-          for (int a4 = 0; a4 < LMAX / 4; ++a4) {
-            if (4 * a4 < L) {
-              const float4 m = __ldg(row + a4);
-              s = fmaf(z[4 * a4], m.x, s);
-              s = fmaf(z[4 * a4 + 1], m.y, s);
-              s = fmaf(z[4 * a4 + 2], m.z, s);
-              s = fmaf(z[4 * a4 + 3], m.w, s);
-            }
-          }
-          Pq[(size_t)b * Nq + p] = s;
-          acc[b * 256] = fmaf(zd, s, acc[b * 256]);
+    for (int l = 0; l < LMAX; ++l) z[l] = (l < L) ? fmaf(d, xc[l * N + pix], Pq[(size_t)l * Nq]) : 0.f;
+    const float4* Mq = reinterpret_cast<const float4*>(Mt + (size_t)(qy * Qx + qx) * L * Lp);
+    const float zd = zeta * d;
+#pragma unroll 1
+    for (int b0 = 0; b0 < L; b0 += BB) {
+      float s[BB], a_old[BB];
+#pragma unroll
+      for (int b = 0; b < BB; ++b) {
+        a_old[b] = (b0 + b < L) ? A[(size_t)(b0 + b) * N + pix] : 0.f;
+        s[b] = 0.f;
+      }
+#pragma unroll
+      for (int a4 = 0; a4 < LMAX / 4; ++a4) {
+        if (4 * a4 >= L) break;
+#pragma unroll
+        for (int b = 0; b < BB; ++b) {
+          const float4 m = __ldg(Mq + (size_t)min(b0 + b, L - 1) * (Lp / 4) + a4);
+          s[b] = fmaf(z[4 * a4], m.x, s[b]);
+          s[b] = fmaf(z[4 * a4 + 1], m.y, s[b]);
+          s[b] = fmaf(z[4 * a4 + 2], m.z, s[b]);
+          s[b] = fmaf(z[4 * a4 + 3], m.w, s[b]);
         }
       }
-    }
 #pragma unroll
-    for (int b0 = 0; b0 < LMAX; b0 += 8) {
-      float a_old[8];
-#pragma unroll
-      for (int b = 0; b < 8; ++b) a_old[b] = (b0 + b < L) ? A[(b0 + b) * N + pix] : 0.f;
-#pragma unroll
-      for (int b = 0; b < 8; ++b)
-        if (b0 + b < L) A[(b0 + b) * N + pix] = a_old[b] + acc[(b0 + b) * 256];
-    }
-    return;
-  }
-  for (int dy = 0; dy < 2; ++dy) {
-    int qy = ty + dy;
-    if (qy >= Qy) break;
-    for (int dx = 0; dx < 2; ++dx) {
-      int qx = tx + dx;
-      if (qx >= Qx) break;
-      const NucFacet f = facets[qy * Qx + qx];
-      if (r < f.r0 || r >= f.r1 || c < f.c0 || c >= f.c1) continue;
-      const int w = f.c1 - f.c0;
-      const int Nq = (f.r1 - f.r0) * w;
-      const int p = (r - f.r0) * w + (c - f.c0);
-      const float d = facet_weight(f, win, r - f.r0, c - f.c0);
-      float* Pq = P + f.p_off;
-      float z[LMAX];
-#pragma unroll
-      for (int l = 0; l < LMAX; ++l) z[l] = (l < L) ? fmaf(d, xc[l * N + pix], Pq[(size_t)l * Nq + p]) : 0.f;
-      const float4* Mq = reinterpret_cast<const float4*>(Mt + (size_t)(qy * Qx + qx) * L * Lp);
-      const float zd = zeta * d;
-#pragma unroll 1
-      for (int b = 0; b < L; ++b) {
-        const float4* row = Mq + (size_t)b * (Lp / 4);
-        float s = 0.f;
-#pragma unroll
-        for (int a4 = 0; a4 < LMAX / 4; ++a4) {
-          if (4 * a4 < L) {
-            const float4 m = __ldg(row + a4);
-            s = fmaf(z[4 * a4], m.x, s);
-            s = fmaf(z[4 * a4 + 1], m.y, s);
-            s = fmaf(z[4 * a4 + 2], m.z, s);
-            s = fmaf(z[4 * a4 + 3], m.w, s);
-          }
+      for (int b = 0; b < BB; ++b)
+        if (b0 + b < L) {
+          Pq[(size_t)(b0 + b) * Nq] = s[b];
+          A[(size_t)(b0 + b) * N + pix] = fmaf(zd, s[b], a_old[b]);
         }
-        Pq[(size_t)b * Nq + p] = s;
-        A[b * N + pix] = fmaf(zd, s, A[b * N + pix]);
-      }
     }
   }
 }
@@ -724,11 +760,26 @@ static void gram_cuda_core(fhs_ctx* ctx, const Cube& cb, const float* xcheck, co
 }
 
 // Per-chunk partial Grams of Z_q = D_q S~_q xcheck (+ P_q) into ctx->s.gram: the tcgen05
-// kernel when tc and L <= 32, else the CUDA-core float-float kernel.
-void launch_gram(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, bool tc, cudaStream_t st) {
+// kernel when tc and 8 < L <= 32, k_gram_small when tc and L <= 8, else the CUDA-core
+// float-float kernel.  Returns the partials per facet (at most one per chunk).
+int launch_gram(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, bool tc, cudaStream_t st) {
   const int nch = nchunk_max(cb);
-  if (tc && launch_gram_tc(cb, xcheck, P, ctx->s.gram, nch, st)) return;   // counts its launch
-  gram_cuda_core<false>(ctx, cb, xcheck, P, st);
+  if (tc && cb.L <= 8) {
+    // a wave of eight CTAs per SM over the facets, each adding up its chunks
+    const int Q = cb.Qy * cb.Qx, parts = std::max(1, std::min({(8 * num_sms() + Q - 1) / Q, nch, kEigDirect}));
+    const int use_P = P != nullptr ? 1 : 0;
+    auto go = [&](auto kernel) {
+      kernel<<<dim3(parts, Q), 128, 0, st>>>(xcheck, P, cb.d_facets, cb.d_win, cb.n1, cb.n2, cb.L, use_P, ctx->s.gram,
+                                             nch, parts);
+    };
+    if (cb.L <= 4) go(k_gram_small<4>);
+    else go(k_gram_small<8>);
+    note_launches(1);
+    return parts;
+  }
+  if (!tc || !launch_gram_tc(cb, xcheck, P, ctx->s.gram, nch, st))         // counts its launch
+    gram_cuda_core<false>(ctx, cb, xcheck, P, st);
+  return nch;
 }
 
 void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P,
@@ -736,9 +787,10 @@ void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, 
   const int L = cb.L;
   const int Q = cb.Qy * cb.Qx;
   const int nch = nchunk_max(cb);
+  int parts = nch;
   if (weights_mode) gram_cuda_core<true>(ctx, cb, xcheck, nullptr, st);
-  else launch_gram(ctx, cb, xcheck, P, ctx->path == FHS_PATH_FAST && cb.gram_tc, st);
-  const bool sum = nch > kEigDirect;
+  else parts = launch_gram(ctx, cb, xcheck, P, ctx->path == FHS_PATH_FAST && cb.gram_tc, st);
+  const bool sum = parts > kEigDirect;
   if (sum) {
     k_gram_sum<<<dim3(kEigParts, Q), 256, 0, st>>>(ctx->s.gram, nch, cb.d_facets, L);
     note_launches(1);
@@ -749,7 +801,7 @@ void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, 
     attr = true;
   }
   k_eig<<<Q, eig_threads(L), eig_smem(L, weights_mode), st>>>(
-      ctx->s.gram, nch, sum ? kEigParts : nch, cb.d_facets, L, theta_bar, cb.d_mubar, (float)(1.0 / cb.zeta),
+      ctx->s.gram, nch, sum ? kEigParts : parts, cb.d_facets, L, theta_bar, cb.d_mubar, (float)(1.0 / cb.zeta),
       ctx->s.nucM, theta_bar_out, weights_mode ? 1 : 0, 40);
   note_launches(1);
 }
