@@ -675,8 +675,8 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
 // M_q^T are read as float4 (the same address across the warp, L1) against 4 FMAs a row and
 // load, and the BB accesses to A and to P are in flight together.  One output at a time, with
 // A read and written between the outputs above 16 channels, took 0.744 ms at 1024^2 x 32 (64
-// facets) and 1.50 ms at 4096^2 x 16 (256 facets); now 0.378 and 1.33 ms (4.4 TB/s).  BB = 8
-// and the register limits by measurement: at 16 channels BB = 8 spills (1.74 ms at 64
+// facets) and 1.50 ms at 4096^2 x 16 (256 facets); now 0.378 and 1.33 ms (4.4 TB/s).  BB (8 at
+// 32 channels, else 4) and the register limits by measurement: at 16 channels BB = 8 spills (1.74 ms at 64
 // registers) or loses occupancy (2.89 ms at 154), BB = 2 1.45 ms; at 32 channels BB = 4 0.419.
 template <int LMAX>
 __global__ void __launch_bounds__(256, LMAX == 16 ? 4 : (LMAX == 32 ? 3 : 2)) k_apply(const float* __restrict__ xc, float* __restrict__ P,
