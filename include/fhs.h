@@ -369,7 +369,8 @@ fhs_status fhs_checkpoint_load(fhs_ctx* ctx, const fhs_iterate* it, const char* 
  *                     fixes the internal visibility order, so it is chosen inside
  *                     fhs_create from trial cubes over the first two channels;
  *  degrid_tiled     : 1 tile-staged (TMA) de-gridder, 0 direct per-visibility one;
- *  gram_tc          : 1 tcgen05 error-free facet Gram (L <= 32), 0 CUDA-core float-float;
+ *  gram_tc          : 1 tcgen05 error-free facet Gram (8 < L <= 32; float pairs in registers
+ *                     up to 8 channels), 0 CUDA-core float-float;
  *  sara_fast        : 1 fused SARA tiles, 0 separate analysis / dual / synthesis passes;
  *  prox_ctas_per_sm : CTAs per SM of the fused l2,1 dual pass;
  *  source           : 0 defaults (autotuning off), 1 measured, 2 read from the cache;
