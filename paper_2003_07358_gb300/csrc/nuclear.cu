@@ -286,20 +286,26 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
 // Plane rotation (c, s) that annihilates gpr of [[gpp, gpr], [gpr, grr]] up to the FP32
 // accuracy of its tangent (the remainder is annihilated in the next sweep); c and s are
 // float pairs with c^2 + s^2 = 1 to about 2^-46.  False (identity) when gpr is below the
-// accuracy of the pairs relative to the larger diagonal entry, or not a number.
-__device__ __forceinline__ bool ff_rotation(ff gpp, ff gpr, ff grr, ff& c, ff& s) {
+// accuracy of the pairs relative to the geometric mean of the diagonal, or not a number: the
+// mean and not the larger entry, so that channels many decades fainter than the others keep
+// their own singular vectors.  `more`: gpr lies above that accuracy of the larger entry as
+// well, so a further sweep is due.
+__device__ __forceinline__ bool ff_rotation(ff gpp, ff gpr, ff grr, ff& c, ff& s, bool& more) {
   c = {1.f, 0.f};
   s = {0.f, 0.f};
-  const float g = gpr.h + gpr.l;
-  const float big = fmaxf(fabsf(gpp.h), fabsf(grr.h));
-  if (!(fabsf(g) > 5.7e-14f * big) || !(fabsf(g) > 1e-30f)) return false;       // 2^-44
+  const float g = gpr.h + gpr.l, pp = fabsf(gpp.h), rr = fabsf(grr.h);
+  constexpr float kEps = 5.7e-14f;                                              // 2^-44
+  const bool some = fabsf(g) > 1e-36f;
+  more = some && fabsf(g) > kEps * fmaxf(pp, rr);
+  if (!some || !(fabsf(g) > kEps * (sqrtf(pp) * sqrtf(rr)))) return false;
   const float d = __fadd_rn(__fsub_rn(grr.h, gpp.h), __fsub_rn(grr.l, gpp.l));
-  // tan = g / (|d|/2 + sqrt(d^2/4 + g^2)) with the sign of d; it may be off by a few ulp
-  // and is taken as exact from here on
-  const float h2 = 0.5f * fabsf(d);
+  // tan = g / (|d|/2 + sqrt(d^2/4 + g^2)) with the sign of d, both scaled by a power of two so
+  // that the squares stay in range; it may be off by a few ulp and is taken as exact from here on
+  const float unit = __int_as_float((254 - (__float_as_int(fmaxf(0.5f * fabsf(d), fabsf(g))) >> 23)) << 23);
+  const float h2 = 0.5f * fabsf(d) * unit, gs = g * unit;
   float root;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(h2, h2, g * g)));
-  const float t = __fdividef(copysignf(1.f, d) * g, h2 + root);
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(h2, h2, gs * gs)));
+  const float t = __fdividef(copysignf(1.f, d) * gs, h2 + root);
   // c = (1 + t^2)^-1/2, s = t c
   const float p = __fmul_rn(t, t), pe = __fmaf_rn(t, t, -p);
   const float uh = __fadd_rn(1.f, p);
@@ -391,6 +397,7 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
                                              int weights_mode, int max_sweeps) {
   extern __shared__ __align__(16) unsigned char eig_smem_raw[];
   __shared__ int s_emax;
+  __shared__ volatile int s_more;    // 1 + the last sweep that left a pair for another one
   const int Le = (L + 1) & ~1, H = Le / 2, Ls = Le + 1;
   float4* rot = reinterpret_cast<float4*>(eig_smem_raw);          // [2][H] (c, s) of a round
   int2* pr = reinterpret_cast<int2*>(rot + 2 * H);                // [2][H] index pairs of a round
@@ -407,7 +414,7 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
   const int Nq = (f.r1 - f.r0) * (f.c1 - f.c0);
   const int nch = min((Nq + kGramChunk - 1) / kGramChunk, nparts_max);
   const float mb = mubar[q];
-  if (tid == 0) s_emax = 0;
+  if (tid == 0) { s_emax = 0; s_more = 0; }
   for (int k = tid; k < Le * Ls; k += nt) {
     const int a = k / Ls, b = k - a * Ls;
     G[k] = make_float2(0.f, 0.f);
@@ -543,7 +550,9 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
           gpp = ldp(G, p * Ls + p);
           gpr = ldp(G, p * Ls + r);
           grr = ldp(G, r * Ls + r);
-          mine = ff_rotation(gpp, gpr, grr, c, s) ? 1 : 0;
+          bool more;
+          mine = ff_rotation(gpp, gpr, grr, c, s, more) ? 1 : 0;
+          if (more) s_more = sweep + 1;
           rot[buf * H + tid] = make_float4(c.h, c.l, s.h, s.l);
           pr[buf * H + tid] = make_int2(p, r);
         }
@@ -582,7 +591,8 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
       rows_due = any;
       buf ^= 1;
     }
-    if (!rotated) break;
+    // (s_more only grows, so a thread that reads it late still sees that the sweep was not the last)
+    if (!rotated || (sweep > 0 && s_more <= sweep)) break;
   }
   if (rows_due && wt >= 0) rotate_rows(buf ^ 1);
   __syncthreads();

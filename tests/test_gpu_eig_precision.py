@@ -1,0 +1,70 @@
+"""What the facet Grams and their eigen-solves keep of FP64: singular vectors of channels many
+decades fainter than the others, on both Gram kernels of the fast path (up to 8 channels, and
+tensor cores) and on the CUDA-core one."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle.prox import jacobi_svd
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _context(n, L, mu_bar):
+    from paper_2003_07358_gb300.fhs import Context, CubeParams
+    rng = np.random.default_rng(1)
+    uv = rng.uniform(-1.0, 1.0, (16 * L, 2)).astype(np.float32)
+    return Context([CubeParams(n1=n, n2=n, L=L, Qy=1, Qx=1, overlap=0.1, window="triangular",
+                               M_lb=np.full((L, 1), 16, dtype=np.int64), uv=uv, eta=np.ones(L), mu=0.1,
+                               mu_bar=np.array([mu_bar]), eps=np.ones((L, 1)))])
+
+
+def _sky(n, L, seed):
+    """Non-negative sources with power-law spectra, [L][n][n] in float64: their channels are nearly
+    dependent, the singular values fall to the rounding of FP32."""
+    rng = np.random.default_rng(seed)
+    nu, r = np.linspace(1.0, 2.0, L), np.arange(n)
+    x = np.zeros((L, n, n))
+    for _ in range(60):
+        y0, x0, w, a, index = (rng.uniform(*b) for b in ((0, n), (0, n), (1, 4), (0.1, 1), (-1, 1)))
+        blob = np.exp(-(r - y0) ** 2 / (2 * w * w))[:, None] * np.exp(-(r - x0) ** 2 / (2 * w * w))
+        x += (a * nu ** index)[:, None, None] * blob
+    return x
+
+
+def _dual(x, mu_bar, tb):
+    L, n = x.shape[:2]
+    ctx = _context(n, L, mu_bar)
+    P, A = torch.zeros(L * n * n, device="cuda"), torch.zeros((L, n, n), device="cuda")
+    ctx.fhs_prox_nuclear_facets(0, torch.as_tensor(x, device="cuda"), P, torch.as_tensor(tb[None, :], device="cuda"), A)
+    ctx.close()
+    return P.double().cpu().numpy().reshape(L, n * n).T
+
+
+@pytest.mark.parametrize("L", [2, 4, 7, 8, 12, 20, 37])
+@pytest.mark.parametrize("amps", [(1e-9,), (1e-11,), (1e-13,), (1e-11, 3e-12)])
+def test_faint_channels(L, amps):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    if len(amps) >= L:
+        pytest.skip("a bright channel is needed")
+    n = 64
+    rng = np.random.default_rng(L)
+    x = _sky(n, L, L)
+    faint = [L // 2, L - 1][:len(amps)] if L > 2 else [1]
+    for l, a in zip(faint, amps):
+        x[l] *= a
+    x = (x * (1.0 + 0.2 * rng.standard_normal(x.shape))).astype(np.float32)
+    Z = x.reshape(L, -1).T.astype(np.float64)
+    U, s, V = jacobi_svd(Z)                          # one-sided: small singular values to full relative accuracy
+    tb = np.linspace(0.3, 1.0, L).astype(np.float32)
+    mu_bar = 0.1 * s[0]
+    m = np.minimum(1.0, mu_bar * tb.astype(np.float64) / s)
+    M = (V * m) @ V.T
+    got, ref = _dual(x, mu_bar, tb), Z @ M
+    # FP32 rows times an FP32 matrix: (L + 2) roundings of 2^-24 on the terms of each channel
+    terms = np.linalg.norm(np.abs(Z) @ np.abs(M), axis=0)
+    err = np.linalg.norm(got - ref, axis=0)
+    assert np.all(err <= 2.0 * (L + 2) * 2.0 ** -24 * terms), (err / terms)[faint]
