@@ -5,7 +5,8 @@
 //   (I - prox_{alpha ||.||_*,theta})(Z) = U diag(min(s_j, alpha_j)) V^T = Z V diag(m) V^T,
 //   m_j = min(1, alpha_j / s_j), Z^T Z = V diag(s^2) V^T.
 // Kernels:
-//   k_gram   : partial Gram matrices Z^T Z of pixel chunks (float pairs, staged in smem);
+//   k_gram   : partial Gram matrices Z^T Z of pixel chunks (float pairs, staged in smem;
+//              k_gram_f64 for the weights, k_gram_small up to 8 channels);
 //   k_eig    : FP64 sum of the partials in fixed order (k_gram_sum first where there are
 //              many), cyclic Jacobi eigen-solve of the L x L Gram in float pairs,
 //              M_q = V diag(m) V^T (or weights);
@@ -35,24 +36,17 @@ __device__ __forceinline__ float facet_weight(const NucFacet& f, const float* __
 // sqrt(eps) s_max.)  Thread owns an LB x LB block of G; Lp = L rounded up to a
 // multiple of LB.  Output: FP64 partials [Q][nchunk_max][L][L].
 //
-// W64 (weights mode of Algorithm 1, once per reweighting cycle): z = wy wx x from the FP64
-// windows as a float pair, so that the small singular values entering
-// theta_bar = mu_bar / (s + mu_bar) are not limited by rounding z to FP32; the products
-// take the pairs' cross terms along (1.68 ms in FP64, 0.24 ms at 36 facets of 85^2 pixels and
-// 38 channels).
-template <int LB, bool W64>
+template <int LB>
 __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __restrict__ xc, const float* __restrict__ P,
                                               const NucFacet* __restrict__ facets, const float* __restrict__ win,
-                                              const double* __restrict__ win64,
                                               int n1, int n2, int L, int use_P, double* __restrict__ part,
                                               int nchunk_max) {
   // the staged sub-chunk and, after the last one, the per-group partial sums
   __shared__ union {
-    float z[W64 ? 2 : 1][kGramSub][kMaxL + 1];
+    float z[kGramSub][kMaxL + 1];
     double red[256 * LB * LB];
   } sm;
-  auto& z = sm.z[0];
-  auto& zl = sm.z[W64 ? 1 : 0];
+  auto& z = sm.z;
   auto& red = sm.red;
   const int q = blockIdx.y;
   const NucFacet f = facets[q];
@@ -107,26 +101,13 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
       pre[k] = val;
     }
   };
-  constexpr bool PF = LB <= 2 && !W64;         // prefetch (registers permitting)
+  constexpr bool PF = LB <= 2;                 // prefetch (registers permitting)
   if (PF) fetch(p0);
   for (int s0 = p0; s0 < p1; s0 += kGramSub) {
     if constexpr (PF) {
 #pragma unroll
       for (int k = 0; k < NPT; ++k)
         if (sl0 + 4 * k < Lp) z[spix][sl0 + 4 * k] = pre[k];
-    } else if constexpr (W64) {
-      const int p = s0 + spix;
-      const int rr = p < p1 ? p / w : 0, cc = p < p1 ? p - rr * w : 0;
-      const double d64 = win64[f.wy_off + rr] * win64[f.wx_off + cc];
-      const float dh = (float)d64, dl = (float)(d64 - (double)dh);
-      const size_t xo = (size_t)(f.r0 + rr) * n2 + (f.c0 + cc);
-#pragma unroll 4
-      for (int l = sl0; l < Lp; l += 4) {
-        const float x = p < p1 && l < L ? xc[l * N + xo] : 0.f;
-        const float h = __fmul_rn(dh, x);
-        z[spix][l] = h;
-        zl[spix][l] = __fmaf_rn(dl, x, __fmaf_rn(dh, x, -h));
-      }
     } else {
 #pragma unroll 4
       for (int idx = threadIdx.x; idx < kGramSub * Lp; idx += blockDim.x) {
@@ -151,20 +132,12 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
         for (int i = 0; i < LB; ++i) a[i] = z[pix][ta * LB + i];
 #pragma unroll
         for (int j = 0; j < LB; ++j) b[j] = z[pix][tb * LB + j];
-        float al[LB], bl[LB];
-        if constexpr (W64) {
-#pragma unroll
-          for (int i = 0; i < LB; ++i) al[i] = zl[pix][ta * LB + i];
-#pragma unroll
-          for (int j = 0; j < LB; ++j) bl[j] = zl[pix][tb * LB + j];
-        }
 #pragma unroll
         for (int i = 0; i < LB; ++i)
 #pragma unroll
           for (int j = 0; j < LB; ++j) {
             float pr = __fmul_rn(a[i], b[j]);
             float pe = __fmaf_rn(a[i], b[j], -pr);
-            if constexpr (W64) pe = __fmaf_rn(al[i], b[j], __fmaf_rn(a[i], bl[j], pe));
             float s, e;
             two_sum(hi[i][j], pr, s, e);
             hi[i][j] = s;
@@ -186,6 +159,88 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
     const int pr = k / (LB * LB), ij = k - pr * LB * LB, i = ij / LB, j = ij - i * LB;
     double v = 0.0;
     for (int gg = 0; gg < G; ++gg) v += red[((size_t)gg * npairs + pr) * LB * LB + ij];
+    int xa = 0, xr = pr;
+    while (xr >= nb - xa) { xr -= nb - xa; ++xa; }
+    const int a = xa * LB + i, b = (xa + xr) * LB + j;
+    if (a < L && b < L) {
+      out[a * L + b] = v;
+      out[b * L + a] = v;
+    }
+  }
+}
+
+// Gram of D_q S~_q x in FP64 for the weights of Algorithm 1 (once per reweighting cycle):
+// theta_bar = mu_bar / (s + mu_bar) depends on singular values far below s_max, and an error
+// of the Gram enters them as its square root, so the windows, the products and the sums are
+// FP64 (float pairs, whose low part rounds at about 2^-47 of the sum, were off by 4e-8 of s_max
+// at 38 channels and 1.2e-7 at 64 where these are by 8e-9, and left FP32's range below 1e-18).
+// Blocks of entries and pixel groups over the threads as in k_gram, so that every warp is
+// full: bound by the FP64 pipe, 16 instructions of 64 clk per pixel, warp and 4 x 4 block.
+template <int LB>
+__global__ void __launch_bounds__(256) k_gram_f64(const float* __restrict__ xc, const NucFacet* __restrict__ facets,
+                                                  const double* __restrict__ win64, int n1, int n2, int L,
+                                                  double* __restrict__ part, int nchunk_max) {
+  __shared__ union {
+    double z[kGramSub][kMaxL + 1];
+    double red[256 * LB * LB];
+  } sm;
+  const int q = blockIdx.y;
+  const NucFacet f = facets[q];
+  const int h = f.r1 - f.r0, w = f.c1 - f.c0;
+  const int Nq = h * w;
+  const int p0 = blockIdx.x * kGramChunk;
+  if (p0 >= Nq) return;
+  const int p1 = min(Nq, p0 + kGramChunk);
+  const int nb = (L + LB - 1) / LB, Lp = nb * LB;
+  const int npairs = nb * (nb + 1) / 2;
+  const int G = max(1, (int)blockDim.x / npairs);
+  const int pair = threadIdx.x % npairs, g = threadIdx.x / npairs;
+  const bool active = g < G;
+  int ta = 0, rem = pair;
+  while (rem >= nb - ta) { rem -= nb - ta; ++ta; }
+  const int tb = ta + rem;
+  double acc[LB][LB];
+#pragma unroll
+  for (int i = 0; i < LB; ++i)
+#pragma unroll
+    for (int j = 0; j < LB; ++j) acc[i][j] = 0.0;
+  const size_t N = (size_t)n1 * n2;
+  const int spix = threadIdx.x % kGramSub, sl0 = threadIdx.x / kGramSub;      // pixel, first channel staged
+  for (int s0 = p0; s0 < p1; s0 += kGramSub) {
+    const int p = s0 + spix;
+    const int rr = p < p1 ? p / w : 0, cc = p < p1 ? p - rr * w : 0;
+    const double d = win64[f.wy_off + rr] * win64[f.wx_off + cc];
+    const size_t xo = (size_t)(f.r0 + rr) * n2 + (f.c0 + cc);
+#pragma unroll 4
+    for (int l = sl0; l < Lp; l += 4) sm.z[spix][l] = p < p1 && l < L ? d * (double)xc[l * N + xo] : 0.0;
+    __syncthreads();
+    if (active) {
+      for (int pix = g; pix < min(kGramSub, p1 - s0); pix += G) {
+        double a[LB], b[LB];
+#pragma unroll
+        for (int i = 0; i < LB; ++i) a[i] = sm.z[pix][ta * LB + i];
+#pragma unroll
+        for (int j = 0; j < LB; ++j) b[j] = sm.z[pix][tb * LB + j];
+#pragma unroll
+        for (int i = 0; i < LB; ++i)
+#pragma unroll
+          for (int j = 0; j < LB; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      }
+    }
+    __syncthreads();
+  }
+  if (active) {
+#pragma unroll
+    for (int i = 0; i < LB; ++i)
+#pragma unroll
+      for (int j = 0; j < LB; ++j) sm.red[((size_t)g * npairs + pair) * LB * LB + i * LB + j] = acc[i][j];
+  }
+  __syncthreads();
+  double* out = part + ((size_t)q * nchunk_max + blockIdx.x) * L * L;
+  for (int k = threadIdx.x; k < npairs * LB * LB; k += blockDim.x) {
+    const int pr = k / (LB * LB), ij = k - pr * LB * LB, i = ij / LB, j = ij - i * LB;
+    double v = 0.0;
+    for (int gg = 0; gg < G; ++gg) v += sm.red[((size_t)gg * npairs + pr) * LB * LB + ij];
     int xa = 0, xr = pr;
     while (xr >= nb - xa) { xr -= nb - xa; ++xa; }
     const int a = xa * LB + i, b = (xa + xr) * LB + j;
@@ -756,16 +811,26 @@ void launch_nuclear(fhs_ctx* ctx, const Cube& cb, const float* xcheck, float* P,
   if (!weights_mode) launch_nuclear_apply(ctx, cb, xcheck, P, A, st);
 }
 
-template <bool W64>
 static void gram_cuda_core(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, cudaStream_t st) {
   const int L = cb.L, nch = nchunk_max(cb), use_P = P != nullptr ? 1 : 0;
   dim3 gg(nch, cb.Qy * cb.Qx);
   auto go = [&](auto kernel) {
-    kernel<<<gg, 256, 0, st>>>(xcheck, P, cb.d_facets, cb.d_win, cb.d_win64, cb.n1, cb.n2, L, use_P, ctx->s.gram, nch);
+    kernel<<<gg, 256, 0, st>>>(xcheck, P, cb.d_facets, cb.d_win, cb.n1, cb.n2, L, use_P, ctx->s.gram, nch);
   };
-  if (L <= 4) go(k_gram<1, W64>);
-  else if (L <= 16) go(k_gram<2, W64>);
-  else go(k_gram<4, W64>);
+  if (L <= 4) go(k_gram<1>);
+  else if (L <= 16) go(k_gram<2>);
+  else go(k_gram<4>);
+  note_launches(1);
+}
+
+static void gram_weights(fhs_ctx* ctx, const Cube& cb, const float* x, cudaStream_t st) {
+  const int L = cb.L, nch = nchunk_max(cb);
+  auto go = [&](auto kernel) {
+    kernel<<<dim3(nch, cb.Qy * cb.Qx), 256, 0, st>>>(x, cb.d_facets, cb.d_win64, cb.n1, cb.n2, L, ctx->s.gram, nch);
+  };
+  if (L <= 4) go(k_gram_f64<1>);
+  else if (L <= 16) go(k_gram_f64<2>);
+  else go(k_gram_f64<4>);
   note_launches(1);
 }
 
@@ -788,7 +853,7 @@ int launch_gram(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* 
     return parts;
   }
   if (!tc || !launch_gram_tc(cb, xcheck, P, ctx->s.gram, nch, st))         // counts its launch
-    gram_cuda_core<false>(ctx, cb, xcheck, P, st);
+    gram_cuda_core(ctx, cb, xcheck, P, st);
   return nch;
 }
 
@@ -798,7 +863,7 @@ void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, 
   const int Q = cb.Qy * cb.Qx;
   const int nch = nchunk_max(cb);
   int parts = nch;
-  if (weights_mode) gram_cuda_core<true>(ctx, cb, xcheck, nullptr, st);
+  if (weights_mode) gram_weights(ctx, cb, xcheck, st);
   else parts = launch_gram(ctx, cb, xcheck, P, ctx->path == FHS_PATH_FAST && cb.gram_tc, st);
   const bool sum = parts > kEigDirect;
   if (sum) {

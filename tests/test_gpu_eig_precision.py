@@ -1,6 +1,6 @@
 """What the facet Grams and their eigen-solves keep of FP64: singular vectors of channels many
 decades fainter than the others, on both Gram kernels of the fast path (up to 8 channels, and
-tensor cores) and on the CUDA-core one."""
+tensor cores) and on the CUDA-core one; weights of images far from 1 in scale."""
 from __future__ import annotations
 
 import numpy as np
@@ -68,3 +68,34 @@ def test_faint_channels(L, amps):
     terms = np.linalg.norm(np.abs(Z) @ np.abs(M), axis=0)
     err = np.linalg.norm(got - ref, axis=0)
     assert np.all(err <= 2.0 * (L + 2) * 2.0 ** -24 * terms), (err / terms)[faint]
+
+
+def _weights(x, mu_bar):
+    L, n = x.shape[:2]
+    ctx = _context(n, L, mu_bar)
+    theta, theta_bar = torch.empty(ctx.sizes(0)["n_coef"], device="cuda"), torch.empty(L, device="cuda")
+    ctx.fhs_reweight(0, torch.as_tensor(x, device="cuda"), theta, theta_bar)
+    ctx.close()
+    return theta_bar.double().cpu().numpy()
+
+
+def _weights_tol(s, mu_bar):
+    """Relative error of mu_bar / (s + mu_bar): an eigenvalue of an FP64 Gram is off by a few
+    2^-53 of the largest (4 here), so s by at most 2^-25.5 s_max; theta_bar and mu_bar are FP32."""
+    return 2.0 ** -25.5 * s[0] / (s + mu_bar) + 2.0 ** -23
+
+
+@pytest.mark.parametrize("L", [3, 8, 20, 38, 64])
+@pytest.mark.parametrize("scale", [1e-25, 1e-20, 1e-12, 1e12, 1e18, 1e25])
+def test_weights_at_any_scale(L, scale):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    n = 64
+    rng = np.random.default_rng(L)
+    V, _ = np.linalg.qr(rng.standard_normal((L, L)))
+    Z = (rng.standard_normal((n * n, L)) * np.logspace(0, -3, L)) @ V.T
+    x = np.ascontiguousarray((Z.T * scale).reshape(L, n, n)).astype(np.float32)
+    s = np.linalg.svd(x.reshape(L, -1).T.astype(np.float64), compute_uv=False)
+    mu_bar = 0.01 * s[0]
+    want = mu_bar / (s + mu_bar)
+    assert np.all(np.abs(_weights(x, mu_bar) - want) <= _weights_tol(s, mu_bar) * want)
