@@ -333,27 +333,17 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
 // ------------------------------------------------------------ eigen-solve
 // A GB300 SM issues one FP64 warp instruction per 64 clocks and sub-partition, whatever
 // the number of active lanes (measured: 64 clk per dependent or independent DFMA, 431 for
-// 1/x or rsqrt, 1.7 lanes/clk per SM), 76 times below FP32.  The Jacobi eigen-solve
-// therefore runs on pairs of floats (hi + lo, about 2^-47), and FP64 keeps what the pairs
-// would lose: the sums of the chunk partials, m_j, and, for the weights, the
-// eigenvalues themselves (Rayleigh quotients, whose error is second order in the
-// eigenvectors').
-// Plane rotation (c, s) that annihilates gpr of [[gpp, gpr], [gpr, grr]] up to the FP32
-// accuracy of its tangent (the remainder is annihilated in the next sweep); c and s are
-// float pairs with c^2 + s^2 = 1 to about 2^-46.  False (identity) when gpr is below the
-// accuracy of the pairs relative to the geometric mean of the diagonal, or not a number: the
-// mean and not the larger entry, so that channels many decades fainter than the others keep
-// their own singular vectors.  `more`: gpr lies above that accuracy of the larger entry as
-// well, so a further sweep is due.
-__device__ __forceinline__ bool ff_rotation(ff gpp, ff gpr, ff grr, ff& c, ff& s, bool& more) {
-  c = {1.f, 0.f};
-  s = {0.f, 0.f};
-  const float g = gpr.h + gpr.l, pp = fabsf(gpp.h), rr = fabsf(grr.h);
-  constexpr float kEps = 5.7e-14f;                                              // 2^-44
-  const bool some = fabsf(g) > 1e-36f;
-  more = some && fabsf(g) > kEps * fmaxf(pp, rr);
-  if (!some || !(fabsf(g) > kEps * (sqrtf(pp) * sqrtf(rr)))) return false;
-  const float d = __fadd_rn(__fsub_rn(grr.h, gpp.h), __fsub_rn(grr.l, gpp.l));
+// 1/x or rsqrt, 1.7 lanes/clk per SM), 76 times below FP32.  The rotations are therefore
+// computed on pairs of floats (hi + lo, about 2^-47), and so is the dual update's matrix:
+// what its pairs lose lies below the FP32 rounding of the products Z M that follow.  FP64
+// keeps the sums of the chunk partials and, for the weights, the matrix itself, since
+// theta_bar = mu_bar / (s + mu_bar) shows errors of s that FP32 duals do not.
+
+// Plane rotation (c, s) that annihilates g of [[gpp, g], [g, grr]], d = grr - gpp, up to the
+// FP32 accuracy of its tangent (the remainder is annihilated in the next sweep); c and s are
+// float pairs with c^2 + s^2 = 1 to about 2^-46 (a rotation scales its two rows alike, so the
+// remainder moves an eigenvalue by that much of itself).
+__device__ __forceinline__ void ff_rotation(float g, float d, ff& c, ff& s) {
   // tan = g / (|d|/2 + sqrt(d^2/4 + g^2)) with the sign of d, both scaled by a power of two so
   // that the squares stay in range; it may be off by a few ulp and is taken as exact from here on
   const float unit = __int_as_float((254 - (__float_as_int(fmaxf(0.5f * fabsf(d), fabsf(g))) >> 23)) << 23);
@@ -369,7 +359,26 @@ __device__ __forceinline__ bool ff_rotation(ff gpp, ff gpr, ff grr, ff& c, ff& s
   const float se = __fmaf_rn(t, c.l, __fmaf_rn(t, c.h, -sp));
   s.h = __fadd_rn(sp, se);
   s.l = __fsub_rn(se, __fsub_rn(s.h, sp));
-  return true;
+}
+
+// Whether a pair of the float-pair matrix is rotated: g above the accuracy of the pairs
+// relative to the geometric mean of the diagonal (false for NaN): the mean and not the larger
+// entry, so that channels many decades fainter than the others keep their own singular
+// vectors.  `more`: g lies above that accuracy of the larger entry as well, so a further sweep
+// is due.
+__device__ __forceinline__ bool pair_turns(float pp, float g, float rr, bool& more) {
+  constexpr float kEps = 5.7e-14f;                                              // 2^-44
+  const bool some = fabsf(g) > 1e-36f;
+  more = some && fabsf(g) > kEps * fmaxf(fabsf(pp), fabsf(rr));
+  return some && fabsf(g) > kEps * (sqrtf(fabsf(pp)) * sqrtf(fabsf(rr)));
+}
+
+// Whether a pair of the FP64 matrix is rotated: the rotation would move the smaller diagonal
+// entry, by about g^2 / max(|d|, |g|), by more than 1e-11 of itself.
+__device__ __forceinline__ bool pair_turns64(double gpp, double g64, double grr) {
+  const float g = fabsf((float)g64), d = fabsf((float)(grr - gpp));
+  const float mn = 1e-11f * fminf(fabsf((float)gpp), fabsf((float)grr));
+  return g > 1e-36f && g * __fdividef(g, fmaxf(d, g)) > mn;
 }
 
 constexpr int kEigRows = 3;        // eigenvector-row items per worker thread, at most
@@ -419,6 +428,179 @@ __global__ void __launch_bounds__(256) k_gram_sum(double* __restrict__ part, int
   }
 }
 
+__device__ __forceinline__ ff ldp(const float2* m, int k) {
+  const float2 x = m[k];
+  return ff{x.x, x.y};
+}
+
+// Cyclic Jacobi sweeps by the whole CTA over the symmetric matrix M [Le][Le + 1] in float
+// pairs, whose rotations also go to the rows of V, or (F64) in FP64 without V.  A sweep is
+// Le - 1 rounds of the round-robin tournament over Le indices; a round rotates H = Le/2
+// disjoint pairs at once.  rot, pr: [2][H], c and s (float pairs, or two doubles) and the index
+// pairs of a round; s_more: 1 + the last sweep that left a pair for another one, zero before.
+// Starts and ends with M and V settled (barriers inside).
+template <bool F64>
+__device__ __forceinline__ void eig_sweeps(float2* __restrict__ G, double* __restrict__ G64, float2* __restrict__ V,
+                                           float4* __restrict__ rot, int2* __restrict__ pr, volatile int* s_more,
+                                           int L, int max_sweeps) {
+  const int Le = (L + 1) & ~1, H = Le / 2, Ls = Le + 1, tid = threadIdx.x, nt = blockDim.x;
+  double2* rot64 = reinterpret_cast<double2*>(rot);
+  const int nB = H * (H - 1) / 2, wt = tid - 32, nw = nt - 32;     // worker threads: warps 1 and up
+  int bi = 0, bj = 0;                            // the worker's block: (pair bi) x (pair bj), bi < bj;
+  const bool has_block = wt >= 0 && wt < 2 * nB; // lane parity: the row of pair bi it writes
+  const unsigned block_lanes = __ballot_sync(0xffffffffu, has_block);
+  const int half = wt & 1;
+  if (has_block) {
+    const int t = wt >> 1;
+    bj = (int)((sqrtf(8.f * t + 1.f) + 1.f) * 0.5f);
+    while (bj * (bj - 1) / 2 > t) --bj;
+    while ((bj + 1) * bj / 2 <= t) ++bj;
+    bi = t - bj * (bj - 1) / 2;
+  }
+  int vi[kEigRows], vk[kEigRows];                // its eigenvector rows: (pair, component)
+#pragma unroll
+  for (int m = 0; m < kEigRows; ++m) {
+    const int k = wt + m * nw;
+    vi[m] = wt >= 0 && k < H * L ? k / L : -1;
+    vk[m] = vi[m] >= 0 ? k - vi[m] * L : 0;
+  }
+  auto stg = [&](int a, int b, ff x) { G[a * Ls + b] = G[b * Ls + a] = make_float2(x.h, x.l); };
+  auto stg64 = [&](int a, int b, double x) { G64[a * Ls + b] = G64[b * Ls + a] = x; };
+  // eigenvector rows of the round in buffer `buf` (an identity rotation leaves its pairs as
+  // they are)
+  auto rotate_rows = [&](int buf) {
+    int o[kEigRows], o2[kEigRows];
+    ff vp[kEigRows], vr[kEigRows];
+    float4 r[kEigRows];
+#pragma unroll
+    for (int m = 0; m < kEigRows; ++m) {
+      const int i = max(vi[m], 0);
+      const int2 pi = pr[buf * H + i];
+      r[m] = rot[buf * H + i];
+      o[m] = pi.x * Ls + vk[m];
+      o2[m] = pi.y * Ls + vk[m];
+      vp[m] = ldp(V, o[m]);
+      vr[m] = ldp(V, o2[m]);
+    }
+    bool turn = false;
+#pragma unroll
+    for (int m = 0; m < kEigRows; ++m) turn = turn || r[m].z != 0.f;
+    if (!turn) return;
+#pragma unroll
+    for (int m = 0; m < kEigRows; ++m) {
+      const ff c = {r[m].x, r[m].y}, s = {r[m].z, r[m].w};
+      const ff x = ff_lin(c, vp[m], {-s.h, -s.l}, vr[m]), y = ff_lin(s, vp[m], c, vr[m]);
+      if (vi[m] >= 0) {
+        V[o[m]] = make_float2(x.h, x.l);
+        V[o2[m]] = make_float2(y.h, y.l);
+      }
+    }
+  };
+  int buf = 0, rows_due = 0;
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+    int rotated = 0;
+    for (int rnd = 0; rnd < Le - 1; ++rnd) {
+      int mine = 0, p = 0, r = 0;
+      ff c = {1.f, 0.f}, s = {0.f, 0.f};
+      if (tid < 32) {
+        if (tid < H) {
+          auto player = [&](int k) {
+            int x = k - 1 + rnd;
+            x = x >= Le - 1 ? x - (Le - 1) : x;
+            return k == 0 ? 0 : x + 1;
+          };
+          p = player(tid);
+          r = player(Le - 1 - tid);
+          if (p > r) { const int x = p; p = r; r = x; }
+          bool more;
+          if constexpr (F64) {
+            const double gpp = G64[p * Ls + p], gpr = G64[p * Ls + r], grr = G64[r * Ls + r];
+            more = pair_turns64(gpp, gpr, grr);
+            mine = more ? 1 : 0;
+            if (mine) ff_rotation((float)gpr, (float)(grr - gpp), c, s);
+            rot64[buf * H + tid] = mine ? make_double2(ff_val(c), ff_val(s)) : make_double2(1.0, 0.0);
+          } else {
+            const ff gpp = ldp(G, p * Ls + p), gpr = ldp(G, p * Ls + r), grr = ldp(G, r * Ls + r);
+            mine = pair_turns(gpp.h, gpr.h + gpr.l, grr.h, more) ? 1 : 0;
+            if (mine)
+              ff_rotation(gpr.h + gpr.l, __fadd_rn(__fsub_rn(grr.h, gpp.h), __fsub_rn(grr.l, gpp.l)), c, s);
+            rot[buf * H + tid] = make_float4(c.h, c.l, s.h, s.l);
+          }
+          if (more) *s_more = sweep + 1;
+          pr[buf * H + tid] = make_int2(p, r);
+        }
+      } else if (!F64 && rows_due) {
+        rotate_rows(buf ^ 1);
+      }
+      const int any = __syncthreads_or(mine);
+      if (any) {
+        rotated = 1;
+        if (tid < 32) {
+          if (mine) {                                        // diagonal block
+            if constexpr (F64) {
+              const double2 t = rot64[buf * H + tid];
+              const double gpp = G64[p * Ls + p], gpr = G64[p * Ls + r], grr = G64[r * Ls + r];
+              const double a1 = t.x * gpp - t.y * gpr, b1 = t.x * gpr - t.y * grr;
+              const double c1 = t.y * gpp + t.x * gpr, d1 = t.y * gpr + t.x * grr;
+              stg64(p, p, t.x * a1 - t.y * b1);
+              stg64(p, r, t.y * a1 + t.x * b1);
+              stg64(r, r, t.y * c1 + t.x * d1);
+            } else {
+              const ff gpp = ldp(G, p * Ls + p), gpr = ldp(G, p * Ls + r), grr = ldp(G, r * Ls + r);
+              const ff ns = {-s.h, -s.l};
+              const ff a1 = ff_lin(c, gpp, ns, gpr), b1 = ff_lin(c, gpr, ns, grr);
+              const ff c1 = ff_lin(s, gpp, c, gpr), d1 = ff_lin(s, gpr, c, grr);
+              stg(p, p, ff_lin(c, a1, ns, b1));
+              stg(p, r, ff_lin(s, a1, c, b1));
+              stg(r, r, ff_lin(s, c1, c, d1));
+            }
+          }
+        } else if (has_block) {
+          // the two threads of a block read all of it, then write a row each
+          const int2 pi = pr[buf * H + bi], pj = pr[buf * H + bj];
+          const int row = half ? pi.y : pi.x, other = half ? pi.x : pi.y;
+          if constexpr (F64) {
+            const double2 ri = rot64[buf * H + bi], rj = rot64[buf * H + bj];
+            const bool turn = ri.y != 0.0 || rj.y != 0.0;    // (the same for both threads)
+            double a2 = 0.0, b2 = 0.0;
+            if (turn) {
+              const double ci = ri.x, si = half ? ri.y : -ri.y;
+              const double a = G64[row * Ls + pj.x], b = G64[row * Ls + pj.y];
+              const double d = G64[other * Ls + pj.x], e = G64[other * Ls + pj.y];
+              const double a1 = ci * a + si * d, b1 = ci * b + si * e;
+              a2 = rj.x * a1 - rj.y * b1;
+              b2 = rj.y * a1 + rj.x * b1;
+            }
+            __syncwarp(block_lanes);
+            if (turn) {
+              stg64(row, pj.x, a2);
+              stg64(row, pj.y, b2);
+            }
+          } else {
+            const float4 ri = rot[buf * H + bi], rj = rot[buf * H + bj];
+            const ff ci = {ri.x, ri.y}, si = half ? ff{ri.z, ri.w} : ff{-ri.z, -ri.w};
+            const ff cj = {rj.x, rj.y}, sj = {rj.z, rj.w};
+            const ff a = ldp(G, row * Ls + pj.x), b = ldp(G, row * Ls + pj.y);
+            const ff d = ldp(G, other * Ls + pj.x), e = ldp(G, other * Ls + pj.y);
+            const ff a1 = ff_lin(ci, a, si, d), b1 = ff_lin(ci, b, si, e);
+            const ff a2 = ff_lin(cj, a1, {-sj.h, -sj.l}, b1), b2 = ff_lin(sj, a1, cj, b1);
+            __syncwarp(block_lanes);
+            stg(row, pj.x, a2);
+            stg(row, pj.y, b2);
+          }
+        }
+        __syncthreads();
+      }
+      rows_due = any;
+      buf ^= 1;
+    }
+    // (s_more only grows, so a thread that reads it late still sees that the sweep was not the last)
+    if (!rotated || (sweep > 0 && *s_more <= sweep)) break;
+  }
+  if (!F64 && rows_due && wt >= 0) rotate_rows(buf ^ 1);
+  __syncthreads();
+}
+
 // Threads of k_eig: warp 0 (rotations, diagonal blocks) and two threads per 2 x 2 block of G
 // above the diagonal blocks, which rotate the eigenvector rows as well.
 static int eig_threads(int L) {
@@ -428,16 +610,17 @@ static int eig_threads(int L) {
 }
 static size_t eig_smem(int L, bool weights) {
   const size_t Le = (L + 1) & ~1, H = Le / 2;
-  const size_t b = 2 * Le * (Le + 1) * sizeof(float2) + 2 * H * (sizeof(float4) + sizeof(int2)) +
-                   L * (2 * sizeof(float2) + sizeof(float) + sizeof(int));
-  return ((b + 15) & ~(size_t)15) + (weights ? 3 * (size_t)L * L * sizeof(double) : 0);
+  return (weights ? 3 : 2) * Le * (Le + 1) * sizeof(float2) + 2 * H * (sizeof(float4) + sizeof(int2)) +
+         L * (2 * sizeof(float2) + sizeof(float) + sizeof(int));
 }
 
 // One CTA per facet: G = sum of the partial Grams (FP64, chunk order), cyclic Jacobi
 // eigen-decomposition G = V diag(lambda) V^T in float pairs, s = sqrt(max(lambda, 0))
 // sorted descending, then either M = V diag(m) V^T with m_j = min(1, alpha_j / s_j),
 // alpha_j = (mu_bar_q / zeta) theta_bar_q[rank j] (dual mode), or
-// theta_bar_q[rank] = mu_bar_q / (s + mu_bar_q) (weights mode).
+// theta_bar_q[rank] = mu_bar_q / (s + mu_bar_q) (W, weights mode).  The weights form V^T G V in
+// FP64 and take its diagonal, after further sweeps in FP64 where the pairs left more than
+// rounding beside it (singular values within about 2^-22 of the largest).
 //
 // Bound by the latency of a round: the rotations of H = Le/2 disjoint index pairs (warp 0,
 // about 500 clk), a barrier, every 2 x 2 block of G transformed in place from both
@@ -445,25 +628,25 @@ static size_t eig_smem(int L, bool weights) {
 // beside the next round's rotations.  One warp in FP64 took 1.09 ms at 20
 // channels (16 facets), 3.74 ms at 32 (64 facets) and, for the weights, 6.48 ms at 38 (36
 // facets); this kernel takes 0.098, 0.24 and 0.33 ms (device times of one launch).
+template <bool W>
 __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, int nchunk_max, int nparts_max,
                                              const NucFacet* __restrict__ facets, int L,
                                              const float* __restrict__ theta_bar, const float* __restrict__ mubar,
                                              float inv_zeta, float* __restrict__ Mout, float* __restrict__ tb_out,
-                                             int weights_mode, int max_sweeps) {
+                                             int max_sweeps) {
   extern __shared__ __align__(16) unsigned char eig_smem_raw[];
   __shared__ int s_emax;
-  __shared__ volatile int s_more;    // 1 + the last sweep that left a pair for another one
+  __shared__ volatile int s_more;
   const int Le = (L + 1) & ~1, H = Le / 2, Ls = Le + 1;
   float4* rot = reinterpret_cast<float4*>(eig_smem_raw);          // [2][H] (c, s) of a round
   int2* pr = reinterpret_cast<int2*>(rot + 2 * H);                // [2][H] index pairs of a round
   float2* G = reinterpret_cast<float2*>(pr + 2 * H);              // [Le][Ls] pairs, index L (odd L): zeros
   float2* V = G + Le * Ls;                                        // [Le][Ls], row j = eigenvector j
-  float2* lam = V + Le * Ls;                                      // [L]
+  double* G64 = reinterpret_cast<double*>(V + Le * Ls);           // weights: G in FP64, [Le][Ls]
+  float2* lam = V + (W ? 2 : 1) * Le * Ls;                        // [L]
   float2* tm = lam + L;                                           // [L] m_j
   float* tbq = reinterpret_cast<float*>(tm + L);                  // [L]
   int* rank = reinterpret_cast<int*>(tbq + L);                    // [L]
-  double* G64 = reinterpret_cast<double*>(
-      eig_smem_raw + (((unsigned char*)(rank + L) - eig_smem_raw + 15) & ~(size_t)15));   // weights: [L][L]
   const int q = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const NucFacet f = facets[q];
   const int Nq = (f.r1 - f.r0) * (f.c1 - f.c0);
@@ -474,8 +657,9 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
     const int a = k / Ls, b = k - a * Ls;
     G[k] = make_float2(0.f, 0.f);
     V[k] = make_float2(a == b ? 1.f : 0.f, 0.f);
+    if (W) G64[k] = 0.0;
   }
-  if (!weights_mode)
+  if (!W)
     for (int j = tid; j < L; j += nt) tbq[j] = theta_bar[(size_t)q * L + j];
   __syncthreads();
   // ---- G (upper triangle; the partials are symmetric), kept in FP64 registers until the
@@ -527,212 +711,99 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
     ff x = ff_of(g);
     if (!(fabsf(x.h) < 3e38f)) x = {__int_as_float(0x7fffffff), 0.f};
     G[a * Ls + b] = G[b * Ls + a] = make_float2(x.h, x.l);
-    if (weights_mode) G64[a * L + b] = G64[b * L + a] = g;
+    if (W) G64[a * Ls + b] = G64[b * Ls + a] = g;
   }
   __syncthreads();
-  // ---- one sweep = Le - 1 rounds of the round-robin tournament over Le indices; a round
-  // rotates H disjoint pairs at once
-  const int nB = H * (H - 1) / 2, wt = tid - 32, nw = nt - 32;     // worker threads: warps 1 and up
-  int bi = 0, bj = 0;                            // the worker's block: (pair bi) x (pair bj), bi < bj;
-  const bool has_block = wt >= 0 && wt < 2 * nB; // lane parity: the row of pair bi it writes
-  const unsigned block_lanes = __ballot_sync(0xffffffffu, has_block);
-  const int half = wt & 1;
-  if (has_block) {
-    const int t = wt >> 1;
-    bj = (int)((sqrtf(8.f * t + 1.f) + 1.f) * 0.5f);
-    while (bj * (bj - 1) / 2 > t) --bj;
-    while ((bj + 1) * bj / 2 <= t) ++bj;
-    bi = t - bj * (bj - 1) / 2;
-  }
-  int vi[kEigRows], vk[kEigRows];                // its eigenvector rows: (pair, component)
-#pragma unroll
-  for (int m = 0; m < kEigRows; ++m) {
-    const int k = wt + m * nw;
-    vi[m] = wt >= 0 && k < H * L ? k / L : -1;
-    vk[m] = vi[m] >= 0 ? k - vi[m] * L : 0;
-  }
-  auto ldp = [](const float2* m, int k) {
-    const float2 x = m[k];
-    return ff{x.x, x.y};
-  };
-  auto stg = [&](int a, int b, ff x) { G[a * Ls + b] = G[b * Ls + a] = make_float2(x.h, x.l); };
-  // eigenvector rows of the round in buffer `buf` (an identity rotation leaves its pairs as
-  // they are)
-  auto rotate_rows = [&](int buf) {
-    int o[kEigRows], o2[kEigRows];
-    ff vp[kEigRows], vr[kEigRows];
-    float4 r[kEigRows];
-#pragma unroll
-    for (int m = 0; m < kEigRows; ++m) {
-      const int i = max(vi[m], 0);
-      const int2 pi = pr[buf * H + i];
-      r[m] = rot[buf * H + i];
-      o[m] = pi.x * Ls + vk[m];
-      o2[m] = pi.y * Ls + vk[m];
-      vp[m] = ldp(V, o[m]);
-      vr[m] = ldp(V, o2[m]);
-    }
-    bool turn = false;
-#pragma unroll
-    for (int m = 0; m < kEigRows; ++m) turn = turn || r[m].z != 0.f;
-    if (!turn) return;
-#pragma unroll
-    for (int m = 0; m < kEigRows; ++m) {
-      const ff c = {r[m].x, r[m].y}, s = {r[m].z, r[m].w};
-      const ff x = ff_lin(c, vp[m], {-s.h, -s.l}, vr[m]), y = ff_lin(s, vp[m], c, vr[m]);
-      if (vi[m] >= 0) {
-        V[o[m]] = make_float2(x.h, x.l);
-        V[o2[m]] = make_float2(y.h, y.l);
-      }
-    }
-  };
-  int buf = 0, rows_due = 0;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    int rotated = 0;
-    for (int rnd = 0; rnd < Le - 1; ++rnd) {
-      int mine = 0, p = 0, r = 0;
-      ff gpp, gpr, grr, c, s;
-      if (tid < 32) {
-        if (tid < H) {
-          auto player = [&](int k) {
-            int x = k - 1 + rnd;
-            x = x >= Le - 1 ? x - (Le - 1) : x;
-            return k == 0 ? 0 : x + 1;
-          };
-          p = player(tid);
-          r = player(Le - 1 - tid);
-          if (p > r) { const int x = p; p = r; r = x; }
-          gpp = ldp(G, p * Ls + p);
-          gpr = ldp(G, p * Ls + r);
-          grr = ldp(G, r * Ls + r);
-          bool more;
-          mine = ff_rotation(gpp, gpr, grr, c, s, more) ? 1 : 0;
-          if (more) s_more = sweep + 1;
-          rot[buf * H + tid] = make_float4(c.h, c.l, s.h, s.l);
-          pr[buf * H + tid] = make_int2(p, r);
-        }
-      } else if (rows_due) {
-        rotate_rows(buf ^ 1);
-      }
-      const int any = __syncthreads_or(mine);
-      if (any) {
-        rotated = 1;
-        if (tid < 32) {
-          if (mine) {                                        // diagonal block, from registers
-            const ff ns = {-s.h, -s.l};
-            const ff a1 = ff_lin(c, gpp, ns, gpr), b1 = ff_lin(c, gpr, ns, grr);
-            const ff c1 = ff_lin(s, gpp, c, gpr), d1 = ff_lin(s, gpr, c, grr);
-            stg(p, p, ff_lin(c, a1, ns, b1));
-            stg(p, r, ff_lin(s, a1, c, b1));
-            stg(r, r, ff_lin(s, c1, c, d1));
-          }
-        } else if (has_block) {
-          // the two threads of a block read all of it, then write a row each
-          const float4 ri = rot[buf * H + bi], rj = rot[buf * H + bj];
-          const int2 pi = pr[buf * H + bi], pj = pr[buf * H + bj];
-          const int row = half ? pi.y : pi.x, other = half ? pi.x : pi.y;
-          const ff ci = {ri.x, ri.y}, si = half ? ff{ri.z, ri.w} : ff{-ri.z, -ri.w};
-          const ff cj = {rj.x, rj.y}, sj = {rj.z, rj.w};
-          const ff a = ldp(G, row * Ls + pj.x), b = ldp(G, row * Ls + pj.y);
-          const ff d = ldp(G, other * Ls + pj.x), e = ldp(G, other * Ls + pj.y);
-          const ff a1 = ff_lin(ci, a, si, d), b1 = ff_lin(ci, b, si, e);
-          const ff a2 = ff_lin(cj, a1, {-sj.h, -sj.l}, b1), b2 = ff_lin(sj, a1, cj, b1);
-          __syncwarp(block_lanes);
-          stg(row, pj.x, a2);
-          stg(row, pj.y, b2);
-        }
-        __syncthreads();
-      }
-      rows_due = any;
-      buf ^= 1;
-    }
-    // (s_more only grows, so a thread that reads it late still sees that the sweep was not the last)
-    if (!rotated || (sweep > 0 && s_more <= sweep)) break;
-  }
-  if (rows_due && wt >= 0) rotate_rows(buf ^ 1);
-  __syncthreads();
-  if (weights_mode) {
-    // ---- Rayleigh quotients v^T G v / v^T v in FP64
-    double* V64 = G64 + L * L;                                     // [L][L]
-    double* W64 = V64 + L * L;
-    for (int k = tid; k < L * L; k += nt) {
-      const int j = k / L, a = k - j * L;
-      V64[k] = ff_val(ldp(V, j * Ls + a));
-    }
+  eig_sweeps<false>(G, nullptr, V, rot, pr, &s_more, L, max_sweeps);
+  if constexpr (W) {
+    // ---- B = V^T G V in FP64 over G: V64 over the pairs of G, V64 G over those of V.  Terms of
+    // faint channels are as small as what they add up to, so they keep their relative accuracy
+    double* V64 = reinterpret_cast<double*>(G);
+    double* W64 = reinterpret_cast<double*>(V);
+    for (int k = tid; k < Le * Ls; k += nt) V64[k] = ff_val(ldp(V, k));
+    if (tid == 0) s_more = 0;
     __syncthreads();
     for (int k = tid; k < L * L; k += nt) {
-      const int j = k / L, a = k - j * L;
+      const int j = k / L, b = k - j * L;
       double y = 0.0;
-      for (int b = 0; b < L; ++b) y = fma(G64[b * L + a], V64[j * L + b], y);
-      W64[k] = V64[k] * y;
+      for (int a = 0; a < L; ++a) y = fma(V64[j * Ls + a], G64[a * Ls + b], y);
+      W64[j * Ls + b] = y;
     }
     __syncthreads();
+    for (int e = tid; e < nE; e += nt) {
+      int a, b;
+      entry(e, a, b);
+      double y = 0.0;
+      for (int k = 0; k < L; ++k) y = fma(W64[a * Ls + k], V64[b * Ls + k], y);
+      G64[a * Ls + b] = G64[b * Ls + a] = y;
+    }
+    __syncthreads();
+    int due = 0;
+    for (int e = tid; e < nE; e += nt) {
+      int a, b;
+      entry(e, a, b);
+      if (a != b) due |= pair_turns64(G64[a * Ls + a], G64[a * Ls + b], G64[b * Ls + b]) ? 1 : 0;
+    }
+    if (__syncthreads_or(due)) eig_sweeps<true>(nullptr, G64, nullptr, rot, pr, &s_more, L, max_sweeps);
     for (int j = tid; j < L; j += nt) {
-      double n = 0.0, s = 0.0;
-      for (int a = 0; a < L; ++a) {
-        s += W64[j * L + a];
-        n = fma(V64[j * L + a], V64[j * L + a], n);
+      const double x = G64[j * Ls + j];
+      int rk = 0;
+      for (int k = 0; k < L; ++k) {
+        const double y = G64[k * Ls + k];
+        rk += y > x || (y == x && k < j);
       }
-      const double r = s / n;
-      const ff x = ff_of(r);
-      lam[j] = make_float2(x.h, x.l);
-      G64[j] = r;                                // G64 was last read before the barrier above
+      const double sv = sqrt(fmax(x, 0.0)) * __hiloint2double((1023 + k4) << 20, 0);
+      tb_out[(size_t)q * L + rk] = (float)((double)mb / (sv + (double)mb));
     }
   } else {
     for (int j = tid; j < L; j += nt) lam[j] = G[j * Ls + j];
-  }
-  __syncthreads();
-  for (int j = tid; j < L; j += nt) {
-    const float2 x = lam[j];
-    int rk = 0;
+    __syncthreads();
+    for (int j = tid; j < L; j += nt) {
+      const float2 x = lam[j];
+      int rk = 0;
 #pragma unroll 4
-    for (int k = 0; k < L; ++k) {
-      const float2 y = lam[k];
-      rk += (y.x > x.x) || (y.x == x.x && (y.y > x.y || (y.y == x.y && k < j)));
+      for (int k = 0; k < L; ++k) {
+        const float2 y = lam[k];
+        rk += (y.x > x.x) || (y.x == x.x && (y.y > x.y || (y.y == x.y && k < j)));
+      }
+      rank[j] = rk;
+      // m = min(1, alpha lambda^-1/2) in the scaled units, 1 where lambda is not positive
+      const ff al = ff_of((double)mb * (double)inv_zeta * (double)tbq[rk] * __hiloint2double((1023 - k4) << 20, 0));
+      ff m = {1.f, 0.f};
+      if (x.x > 0.f) {
+        const ff t = ff_mul(al, ff_rsqrt({x.x, x.y}));
+        if (t.h < 1.f || (t.h == 1.f && t.l < 0.f)) m = t;
+      }
+      tm[j] = make_float2(m.h, m.l);
     }
-    rank[j] = rk;
-    if (weights_mode) {
-      const double sv = sqrt(fmax(G64[j], 0.0)) * __hiloint2double((1023 + k4) << 20, 0);
-      tb_out[(size_t)q * L + rk] = (float)((double)mb / (sv + (double)mb));
-      continue;
+    __syncthreads();
+    for (int k = tid; k < L * L; k += nt) {        // diag(m) V^T, over G
+      const int j = k / L, o = j * Ls + k - j * L;
+      const ff w = ff_mul(ldp(tm, j), ldp(V, o));
+      G[o] = make_float2(w.h, w.l);
     }
-    // m = min(1, alpha lambda^-1/2) in the scaled units, 1 where lambda is not positive
-    const ff al = ff_of((double)mb * (double)inv_zeta * (double)tbq[rk] * __hiloint2double((1023 - k4) << 20, 0));
-    ff m = {1.f, 0.f};
-    if (x.x > 0.f) {
-      const ff t = ff_mul(al, ff_rsqrt({x.x, x.y}));
-      if (t.h < 1.f || (t.h == 1.f && t.l < 0.f)) m = t;
-    }
-    tm[j] = make_float2(m.h, m.l);
-  }
-  if (weights_mode) return;
-  __syncthreads();
-  for (int k = tid; k < L * L; k += nt) {        // diag(m) V^T, over G
-    const int j = k / L, o = j * Ls + k - j * L;
-    const ff w = ff_mul(ldp(tm, j), ldp(V, o));
-    G[o] = make_float2(w.h, w.l);
-  }
-  __syncthreads();
-  // M_q^T, rows padded to Lp = L rounded up to 4 (zeros), so that a row is read as float4;
-  // each entry (symmetric) is summed in float pairs and rounded once
-  const int Lp = (L + 3) & ~3;
-  float* Mq = Mout + (size_t)q * L * Lp;
-  for (int e = tid; e < nE; e += nt) {
-    int a, b;
-    entry(e, a, b);
-    ff m0 = {0.f, 0.f}, m1 = {0.f, 0.f};
-    const ff one = {1.f, 0.f};
-    int j = 0;
+    __syncthreads();
+    // M_q^T, rows padded to Lp = L rounded up to 4 (zeros), so that a row is read as float4;
+    // each entry (symmetric) is summed in float pairs and rounded once
+    const int Lp = (L + 3) & ~3;
+    float* Mq = Mout + (size_t)q * L * Lp;
+    for (int e = tid; e < nE; e += nt) {
+      int a, b;
+      entry(e, a, b);
+      ff m0 = {0.f, 0.f}, m1 = {0.f, 0.f};
+      const ff one = {1.f, 0.f};
+      int j = 0;
 #pragma unroll 2
-    for (; j + 2 <= L; j += 2) {
-      m0 = ff_lin(ldp(G, j * Ls + b), ldp(V, j * Ls + a), one, m0);
-      m1 = ff_lin(ldp(G, (j + 1) * Ls + b), ldp(V, (j + 1) * Ls + a), one, m1);
+      for (; j + 2 <= L; j += 2) {
+        m0 = ff_lin(ldp(G, j * Ls + b), ldp(V, j * Ls + a), one, m0);
+        m1 = ff_lin(ldp(G, (j + 1) * Ls + b), ldp(V, (j + 1) * Ls + a), one, m1);
+      }
+      if (j < L) m0 = ff_lin(ldp(G, j * Ls + b), ldp(V, j * Ls + a), one, m0);
+      m0 = ff_lin(one, m0, one, m1);
+      Mq[b * Lp + a] = Mq[a * Lp + b] = m0.h + m0.l;
     }
-    if (j < L) m0 = ff_lin(ldp(G, j * Ls + b), ldp(V, j * Ls + a), one, m0);
-    m0 = ff_lin(one, m0, one, m1);
-    Mq[b * Lp + a] = Mq[a * Lp + b] = m0.h + m0.l;
+    for (int k = tid; k < L * (Lp - L); k += nt) Mq[(k / (Lp - L)) * Lp + L + k % (Lp - L)] = 0.f;
   }
-  for (int k = tid; k < L * (Lp - L); k += nt) Mq[(k / (Lp - L)) * Lp + L + k % (Lp - L)] = 0.f;
 }
 
 // Pixel-driven update: each thread owns one pixel; for every facet covering it,
@@ -870,14 +941,18 @@ void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, 
     k_gram_sum<<<dim3(kEigParts, Q), 256, 0, st>>>(ctx->s.gram, nch, cb.d_facets, L);
     note_launches(1);
   }
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_smem(kMaxL, true));
-    attr = true;
-  }
-  k_eig<<<Q, eig_threads(L), eig_smem(L, weights_mode), st>>>(
-      ctx->s.gram, nch, sum ? kEigParts : parts, cb.d_facets, L, theta_bar, cb.d_mubar, (float)(1.0 / cb.zeta),
-      ctx->s.nucM, theta_bar_out, weights_mode ? 1 : 0, 40);
+  auto go = [&](auto kernel, bool& attr) {
+    if (!attr) {
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_smem(kMaxL, weights_mode));
+      attr = true;
+    }
+    kernel<<<Q, eig_threads(L), eig_smem(L, weights_mode), st>>>(
+        ctx->s.gram, nch, sum ? kEigParts : parts, cb.d_facets, L, theta_bar, cb.d_mubar, (float)(1.0 / cb.zeta),
+        ctx->s.nucM, theta_bar_out, 40);
+  };
+  static bool attr_w = false, attr_d = false;
+  if (weights_mode) go(k_eig<true>, attr_w);
+  else go(k_eig<false>, attr_d);
   note_launches(1);
 }
 

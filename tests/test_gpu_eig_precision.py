@@ -1,6 +1,7 @@
 """What the facet Grams and their eigen-solves keep of FP64: singular vectors of channels many
 decades fainter than the others, on both Gram kernels of the fast path (up to 8 channels, and
-tensor cores) and on the CUDA-core one; weights of images far from 1 in scale."""
+tensor cores) and on the CUDA-core one; weights of images far from 1 in scale, and of nearly
+dependent channels, whose singular values lie below 2^-24 of the largest."""
 from __future__ import annotations
 
 import numpy as np
@@ -99,3 +100,22 @@ def test_weights_at_any_scale(L, scale):
     mu_bar = 0.01 * s[0]
     want = mu_bar / (s + mu_bar)
     assert np.all(np.abs(_weights(x, mu_bar) - want) <= _weights_tol(s, mu_bar) * want)
+
+
+@pytest.mark.parametrize("L,n", [(8, 64), (20, 64), (33, 256), (38, 96), (38, 288), (45, 96), (64, 96), (64, 288)])
+@pytest.mark.parametrize("faint", [False, True])
+def test_weights_of_dependent_channels(L, n, faint):
+    """Both sides of 64 chunks of 1024 pixels (256^2 and 288^2); `faint`: with a channel 1e-9 of the
+    others, whose singular value FP64 rotations keep although it lies below 2^-26 of the largest."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    x = _sky(n, L, L)
+    if faint:
+        x[L // 2] *= 1e-9
+    x = x.astype(np.float32)
+    s = torch.linalg.svdvals(torch.as_tensor(x.reshape(L, -1).T.astype(np.float64), device="cuda")).cpu().numpy()
+    for f in (1e-2, 1e-3, 1e-4):
+        mu_bar = f * s[0]
+        want = mu_bar / (s + mu_bar)
+        got = _weights(x, mu_bar)
+        assert np.all(np.abs(got - want) <= _weights_tol(s, mu_bar) * want), (f, np.max(np.abs(got - want) / want))
