@@ -258,6 +258,10 @@ __global__ void __launch_bounds__(256) k_gram_f64(const float* __restrict__ xc, 
 // blockIdx.x, as k_gram_sum leaves it.  The tensor-core kernel pads such facets to 16
 // channels and pays a chunk's slicing and epilogue all the same: 1.61 ms at 4 channels of
 // 4096^2 (256 facets), here 0.25 ms.
+//
+// The pairs hold while the squares and their rounding errors stay in FP32's range: a CTA that
+// meets a channel whose largest |z| is not zero and lies outside [1e-15, 1e15] goes over
+// its pixels again in FP64.
 template <int LM>
 __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc, const float* __restrict__ P,
                                                     const NucFacet* __restrict__ facets,
@@ -266,31 +270,40 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
   constexpr int NP = LM * (LM + 1) / 2, LD = NP | 1, SH = 128 / NP;   // shares of the final sum
   __shared__ float2 red[128 * LD];
   __shared__ float2 red2[SH * NP];
+  __shared__ unsigned s_nonzero, s_normal;          // channels with |z| > 0, |z| >= 1e-15
   const int q = blockIdx.y, tid = threadIdx.x;
   const NucFacet f = facets[q];
   const int w = f.c1 - f.c0, Nq = (f.r1 - f.r0) * w, nch = (Nq + kGramChunk - 1) / kGramChunk;
   if ((int)blockIdx.x >= nch) return;
   const size_t N = (size_t)n1 * n2;
-  float hi[NP], lo[NP];
+  auto load = [&](int p, float (&z)[LM]) {          // z of pixel p (zero past the facet and from L on)
+    const bool in = p < Nq;
+    const int rr = in ? p / w : 0, cc = in ? p - rr * w : 0;
+    const float d = facet_weight(f, win, rr, cc);
+    const float* xp = xc + (size_t)(f.r0 + rr) * n2 + (f.c0 + cc);
+    const float* pp = P + f.p_off + p;
+    float u[LM];
+#pragma unroll
+    for (int l = 0; l < LM; ++l) {
+      z[l] = in && l < L ? xp[(size_t)l * N] : 0.f;
+      u[l] = in && use_P && l < L ? pp[(size_t)l * Nq] : 0.f;
+    }
+#pragma unroll
+    for (int l = 0; l < LM; ++l) z[l] = fmaf(d, z[l], u[l]);
+  };
+  if (tid == 0) s_nonzero = s_normal = 0;
+  float hi[NP], lo[NP], big[LM];
 #pragma unroll
   for (int e = 0; e < NP; ++e) hi[e] = lo[e] = 0.f;
+#pragma unroll
+  for (int l = 0; l < LM; ++l) big[l] = 0.f;
   for (int c = blockIdx.x; c < nch; c += parts) {
 #pragma unroll 2
     for (int k = 0; k < kGramChunk / 128; ++k) {
-      const int p = c * kGramChunk + k * 128 + tid;
-      const bool in = p < Nq;
-      const int rr = in ? p / w : 0, cc = in ? p - rr * w : 0;
-      const float d = facet_weight(f, win, rr, cc);
-      const float* xp = xc + (size_t)(f.r0 + rr) * n2 + (f.c0 + cc);
-      const float* pp = P + f.p_off + p;
-      float z[LM], u[LM];
+      float z[LM];
+      load(c * kGramChunk + k * 128 + tid, z);
 #pragma unroll
-      for (int l = 0; l < LM; ++l) {
-        z[l] = in && l < L ? xp[(size_t)l * N] : 0.f;
-        u[l] = in && use_P && l < L ? pp[(size_t)l * Nq] : 0.f;
-      }
-#pragma unroll
-      for (int l = 0; l < LM; ++l) z[l] = fmaf(d, z[l], u[l]);
+      for (int l = 0; l < LM; ++l) big[l] = fmaxf(big[l], fabsf(z[l]));
       int e = 0;
 #pragma unroll
       for (int b = 0; b < LM; ++b)
@@ -303,6 +316,55 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
           lo[e] = __fadd_rn(lo[e], __fadd_rn(er, pe));
         }
     }
+  }
+  unsigned nonzero = 0, normal = 0;
+  bool large = false;
+#pragma unroll
+  for (int l = 0; l < LM; ++l) {
+    nonzero |= big[l] > 0.f ? 1u << l : 0u;
+    normal |= big[l] >= 1e-15f ? 1u << l : 0u;
+    large = large || big[l] > 1e15f;
+  }
+  __syncthreads();
+  if (nonzero & ~s_nonzero) atomicOr(&s_nonzero, nonzero);
+  if (normal & ~s_normal) atomicOr(&s_normal, normal);
+  const bool fp64 = __syncthreads_or(large) || s_nonzero != s_normal;
+  const auto entry = [&](int e, double v) {         // entry e of the triangle into the output slot
+    int b = 0;
+    while ((b + 1) * (b + 2) / 2 <= e) ++b;
+    const int a = e - b * (b + 1) / 2;
+    if (b < L) {
+      double* out = part + ((size_t)q * nchunk_max + blockIdx.x) * L * L;
+      out[a * L + b] = out[b * L + a] = v;
+    }
+  };
+  if (fp64) {
+    double* red64 = reinterpret_cast<double*>(red);
+    double acc[NP];
+#pragma unroll
+    for (int e = 0; e < NP; ++e) acc[e] = 0.0;
+#pragma unroll 1
+    for (int c = blockIdx.x; c < nch; c += parts) {
+#pragma unroll 1
+      for (int k = 0; k < kGramChunk / 128; ++k) {
+        float z[LM];
+        load(c * kGramChunk + k * 128 + tid, z);
+        int e = 0;
+#pragma unroll
+        for (int b = 0; b < LM; ++b)
+#pragma unroll
+          for (int a = 0; a <= b; ++a, ++e) acc[e] = fma((double)z[a], (double)z[b], acc[e]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < NP; ++e) red64[tid * LD + e] = acc[e];
+    __syncthreads();
+    if (tid < NP) {
+      double v = 0.0;
+      for (int t = 0; t < 128; ++t) v += red64[t * LD + tid];
+      entry(tid, v);
+    }
+    return;
   }
 #pragma unroll
   for (int e = 0; e < NP; ++e) {
@@ -320,13 +382,7 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
   if (tid < NP) {
     ff s = {0.f, 0.f};
     for (int t = 0; t < SH; ++t) s = ff_add(s, {red2[t * NP + tid].x, red2[t * NP + tid].y});
-    int b = 0;
-    while ((b + 1) * (b + 2) / 2 <= tid) ++b;
-    const int a = tid - b * (b + 1) / 2;
-    if (b < L) {
-      double* out = part + ((size_t)q * nchunk_max + blockIdx.x) * L * L;
-      out[a * L + b] = out[b * L + a] = ff_val(s);
-    }
+    entry(tid, ff_val(s));
   }
 }
 
@@ -911,7 +967,9 @@ static void gram_weights(fhs_ctx* ctx, const Cube& cb, const float* x, cudaStrea
 int launch_gram(fhs_ctx* ctx, const Cube& cb, const float* xcheck, const float* P, bool tc, cudaStream_t st) {
   const int nch = nchunk_max(cb);
   if (tc && cb.L <= 8) {
-    // a wave of eight CTAs per SM over the facets, each adding up its chunks
+    // a wave of eight CTAs per SM over the facets, each adding up its chunks; at most the
+    // kEigDirect partials a facet that k_eig adds itself, so fewer CTAs below 19 facets (one
+    // facet of 4096^2 x 4 still takes 2.1 ms with its update where the tensor-core kernel took 10.2)
     const int Q = cb.Qy * cb.Qx, parts = std::max(1, std::min({(8 * num_sms() + Q - 1) / Q, nch, kEigDirect}));
     const int use_P = P != nullptr ? 1 : 0;
     auto go = [&](auto kernel) {

@@ -1,6 +1,7 @@
 """What the facet Grams and their eigen-solves keep of FP64: singular vectors of channels many
 decades fainter than the others, on both Gram kernels of the fast path (up to 8 channels, and
-tensor cores) and on the CUDA-core one; weights of images far from 1 in scale, and of nearly
+tensor cores) and on the CUDA-core one; duals and
+weights of images far from 1 in scale, and weights of nearly
 dependent channels, whose singular values lie below 2^-24 of the largest."""
 from __future__ import annotations
 
@@ -119,3 +120,25 @@ def test_weights_of_dependent_channels(L, n, faint):
         want = mu_bar / (s + mu_bar)
         got = _weights(x, mu_bar)
         assert np.all(np.abs(got - want) <= _weights_tol(s, mu_bar) * want), (f, np.max(np.abs(got - want) / want))
+
+
+@pytest.mark.parametrize("L", [1, 3, 4, 5, 8, 12])
+@pytest.mark.parametrize("scale", [1e-32, 1e-23, 1e-19, 1e-14, 1e14, 1e18, 1e25])
+def test_dual_at_any_scale(L, scale):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    n = 64
+    rng = np.random.default_rng(L)
+    V, _ = np.linalg.qr(rng.standard_normal((L, L)))
+    Z = (rng.standard_normal((n * n, L)) * np.logspace(0, -3, L)) @ V.T * scale
+    x = np.ascontiguousarray(Z.T.reshape(L, n, n)).astype(np.float32)
+    x[:, : n // 2] *= np.float32(1e-3)               # CTAs on either side of the limits
+    Z = x.reshape(L, -1).T.astype(np.float64)
+    U, s, Vt = np.linalg.svd(Z / scale, full_matrices=False)
+    tb = np.linspace(0.3, 1.0, L).astype(np.float32)
+    m = np.minimum(1.0, 0.05 * s[0] * tb.astype(np.float64) / s)
+    M = (Vt.T * m) @ Vt
+    got = _dual(x, 0.05 * s[0] * scale, tb)
+    # FP32 rows times an FP32 matrix, in units of the scale; below 1e-31 FP32's own spacing too
+    tol = 2.0 * (L + 2) * 2.0 ** -24 * np.linalg.norm(Z / scale) * np.linalg.norm(M) + n * np.sqrt(L) * 2.0 ** -149 / scale
+    assert np.linalg.norm(got / scale - (Z / scale) @ M) <= tol
