@@ -389,11 +389,10 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
 // ------------------------------------------------------------ eigen-solve
 // A GB300 SM issues one FP64 warp instruction per 64 clocks and sub-partition, whatever
 // the number of active lanes (measured: 64 clk per dependent or independent DFMA, 431 for
-// 1/x or rsqrt, 1.7 lanes/clk per SM), 76 times below FP32.  The rotations are therefore
-// computed on pairs of floats (hi + lo, about 2^-47), and so is the dual update's matrix:
-// what its pairs lose lies below the FP32 rounding of the products Z M that follow.  FP64
-// keeps the sums of the chunk partials and, for the weights, the matrix itself, since
-// theta_bar = mu_bar / (s + mu_bar) shows errors of s that FP32 duals do not.
+// 1/x or rsqrt, 1.7 lanes/clk per SM), 76 times below FP32.  The Jacobi sweeps therefore run
+// on pairs of floats (hi + lo, about 2^-47 of the largest entry), and V^T G V is then formed in
+// FP64: its diagonal has FP64's eigenvalues, the entries beside it correct M to first order, and
+// where that would not do (entries below about 1e-7 of the largest) further sweeps run in FP64.
 
 // Plane rotation (c, s) that annihilates g of [[gpp, g], [g, grr]], d = grr - gpp, up to the
 // FP32 accuracy of its tangent (the remainder is annihilated in the next sweep); c and s are
@@ -429,12 +428,25 @@ __device__ __forceinline__ bool pair_turns(float pp, float g, float rr, bool& mo
   return some && fabsf(g) > kEps * (sqrtf(fabsf(pp)) * sqrtf(fabsf(rr)));
 }
 
-// Whether a pair of the FP64 matrix is rotated: the rotation would move the smaller diagonal
-// entry, by about g^2 / max(|d|, |g|), by more than 1e-11 of itself.
-__device__ __forceinline__ bool pair_turns64(double gpp, double g64, double grr) {
+// Whether a pair of the FP64 matrix is rotated: whether that would change a result.  The
+// rotation by about theta = g / max(|d|, |g|) moves the diagonal entries by theta g and their
+// vectors by theta.  tp, tr: (squared threshold, m) of the entries.
+//  weights: an entry moves by more than 1e-11 of itself and of its threshold (1e-8 of mu_bar);
+//  duals: not if both entries stay below their thresholds (m = 1 for any vectors); else if the
+//  second-order change of M exceeds 1e-8 of the larger m (the first order is added to M), or
+//  the smaller entry moves by more than 1e-9 of itself and its threshold.
+template <bool W>
+__device__ __forceinline__ bool pair_turns64(double gpp, double g64, double grr, float2 tp, float2 tr) {
   const float g = fabsf((float)g64), d = fabsf((float)(grr - gpp));
-  const float mn = 1e-11f * fminf(fabsf((float)gpp), fabsf((float)grr));
-  return g > 1e-36f && g * __fdividef(g, fmaxf(d, g)) > mn;
+  const float p = fabsf((float)gpp), r = fabsf((float)grr);
+  const float theta = __fdividef(g, fmaxf(d, g)), move = g * theta;
+  const bool less = p < r;
+  const float small = less ? p : r, ts = less ? tp.x : tr.x, large = less ? r : p, tl = less ? tr.x : tp.x;
+  if (!(g > 1e-36f)) return false;
+  if (W) return move > 1e-11f * fmaxf(small, ts);
+  if (small + move < 0.99f * ts && large + move < 0.99f * tl) return false;
+  return theta * theta * fabsf(tp.y - tr.y) > 1e-8f * fmaxf(tp.y, tr.y) ||
+         move > 1e-9f * fmaxf(small, fminf(ts, large));
 }
 
 constexpr int kEigRows = 3;        // eigenvector-row items per worker thread, at most
@@ -489,18 +501,18 @@ __device__ __forceinline__ ff ldp(const float2* m, int k) {
   return ff{x.x, x.y};
 }
 
-// Cyclic Jacobi sweeps by the whole CTA over the symmetric matrix M [Le][Le + 1] in float
-// pairs, whose rotations also go to the rows of V, or (F64) in FP64 without V.  A sweep is
-// Le - 1 rounds of the round-robin tournament over Le indices; a round rotates H = Le/2
-// disjoint pairs at once.  rot, pr: [2][H], c and s (float pairs, or two doubles) and the index
-// pairs of a round; s_more: 1 + the last sweep that left a pair for another one, zero before.
-// Starts and ends with M and V settled (barriers inside).
-template <bool F64>
+// Cyclic Jacobi sweeps by the whole CTA over the symmetric matrix [Le][Le + 1] in float pairs
+// (G) or, F64, in FP64 (G64, with thr = (squared threshold, m)); the rotations also go to the
+// rows of V.  A sweep is Le - 1 rounds of the round-robin tournament over Le indices; a round
+// rotates H = Le/2 disjoint pairs at once.  rot, rot64, pr: [2][H], c and s in pairs, the same
+// in FP64 and the index pairs of a round; s_more: 1 + the last sweep that left a pair for
+// another one, zero before.  Starts and ends with the matrices settled (barriers inside).
+template <bool F64, bool W>
 __device__ __forceinline__ void eig_sweeps(float2* __restrict__ G, double* __restrict__ G64, float2* __restrict__ V,
-                                           float4* __restrict__ rot, int2* __restrict__ pr, volatile int* s_more,
-                                           int L, int max_sweeps) {
+                                           float4* __restrict__ rot, double2* __restrict__ rot64,
+                                           int2* __restrict__ pr, volatile int* s_more, int L, int max_sweeps,
+                                           const float2* __restrict__ thr) {
   const int Le = (L + 1) & ~1, H = Le / 2, Ls = Le + 1, tid = threadIdx.x, nt = blockDim.x;
-  double2* rot64 = reinterpret_cast<double2*>(rot);
   const int nB = H * (H - 1) / 2, wt = tid - 32, nw = nt - 32;     // worker threads: warps 1 and up
   int bi = 0, bj = 0;                            // the worker's block: (pair bi) x (pair bj), bi < bj;
   const bool has_block = wt >= 0 && wt < 2 * nB; // lane parity: the row of pair bi it writes
@@ -571,10 +583,11 @@ __device__ __forceinline__ void eig_sweeps(float2* __restrict__ G, double* __res
           bool more;
           if constexpr (F64) {
             const double gpp = G64[p * Ls + p], gpr = G64[p * Ls + r], grr = G64[r * Ls + r];
-            more = pair_turns64(gpp, gpr, grr);
+            more = pair_turns64<W>(gpp, gpr, grr, thr[p], thr[r]);
             mine = more ? 1 : 0;
             if (mine) ff_rotation((float)gpr, (float)(grr - gpp), c, s);
             rot64[buf * H + tid] = mine ? make_double2(ff_val(c), ff_val(s)) : make_double2(1.0, 0.0);
+            rot[buf * H + tid] = make_float4(c.h, c.l, s.h, s.l);
           } else {
             const ff gpp = ldp(G, p * Ls + p), gpr = ldp(G, p * Ls + r), grr = ldp(G, r * Ls + r);
             mine = pair_turns(gpp.h, gpr.h + gpr.l, grr.h, more) ? 1 : 0;
@@ -585,7 +598,7 @@ __device__ __forceinline__ void eig_sweeps(float2* __restrict__ G, double* __res
           if (more) *s_more = sweep + 1;
           pr[buf * H + tid] = make_int2(p, r);
         }
-      } else if (!F64 && rows_due) {
+      } else if (rows_due) {
         rotate_rows(buf ^ 1);
       }
       const int any = __syncthreads_or(mine);
@@ -653,7 +666,7 @@ __device__ __forceinline__ void eig_sweeps(float2* __restrict__ G, double* __res
     // (s_more only grows, so a thread that reads it late still sees that the sweep was not the last)
     if (!rotated || (sweep > 0 && *s_more <= sweep)) break;
   }
-  if (!F64 && rows_due && wt >= 0) rotate_rows(buf ^ 1);
+  if (rows_due && wt >= 0) rotate_rows(buf ^ 1);
   __syncthreads();
 }
 
@@ -664,19 +677,17 @@ static int eig_threads(int L) {
   const int work = std::max(2 * nB, (H * L + kEigRows - 1) / kEigRows);
   return 32 + std::max(32, (work + 31) & ~31);
 }
-static size_t eig_smem(int L, bool weights) {
+static size_t eig_smem(int L) {
   const size_t Le = (L + 1) & ~1, H = Le / 2;
-  return (weights ? 3 : 2) * Le * (Le + 1) * sizeof(float2) + 2 * H * (sizeof(float4) + sizeof(int2)) +
-         L * (2 * sizeof(float2) + sizeof(float) + sizeof(int));
+  return 4 * Le * (Le + 1) * sizeof(float2) + 2 * H * (2 * sizeof(float4) + sizeof(int2)) +
+         Le * (3 * sizeof(float2) + sizeof(float));
 }
 
 // One CTA per facet: G = sum of the partial Grams (FP64, chunk order), cyclic Jacobi
 // eigen-decomposition G = V diag(lambda) V^T in float pairs, s = sqrt(max(lambda, 0))
 // sorted descending, then either M = V diag(m) V^T with m_j = min(1, alpha_j / s_j),
 // alpha_j = (mu_bar_q / zeta) theta_bar_q[rank j] (dual mode), or
-// theta_bar_q[rank] = mu_bar_q / (s + mu_bar_q) (W, weights mode).  The weights form V^T G V in
-// FP64 and take its diagonal, after further sweeps in FP64 where the pairs left more than
-// rounding beside it (singular values within about 2^-22 of the largest).
+// theta_bar_q[rank] = mu_bar_q / (s + mu_bar_q) (W, weights mode); lambda in FP64 as above.
 //
 // Bound by the latency of a round: the rotations of H = Le/2 disjoint index pairs (warp 0,
 // about 500 clk), a barrier, every 2 x 2 block of G transformed in place from both
@@ -695,14 +706,17 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
   __shared__ volatile int s_more;
   const int Le = (L + 1) & ~1, H = Le / 2, Ls = Le + 1;
   float4* rot = reinterpret_cast<float4*>(eig_smem_raw);          // [2][H] (c, s) of a round
-  int2* pr = reinterpret_cast<int2*>(rot + 2 * H);                // [2][H] index pairs of a round
+  double2* rot64 = reinterpret_cast<double2*>(rot + 2 * H);       // [2][H] the same in FP64
+  int2* pr = reinterpret_cast<int2*>(rot64 + 2 * H);              // [2][H] index pairs of a round
   float2* G = reinterpret_cast<float2*>(pr + 2 * H);              // [Le][Ls] pairs, index L (odd L): zeros
   float2* V = G + Le * Ls;                                        // [Le][Ls], row j = eigenvector j
-  double* G64 = reinterpret_cast<double*>(V + Le * Ls);           // weights: G in FP64, [Le][Ls]
-  float2* lam = V + (W ? 2 : 1) * Le * Ls;                        // [L]
-  float2* tm = lam + L;                                           // [L] m_j
-  float* tbq = reinterpret_cast<float*>(tm + L);                  // [L]
-  int* rank = reinterpret_cast<int*>(tbq + L);                    // [L]
+  double* G64 = reinterpret_cast<double*>(V + Le * Ls);           // [Le][Ls] G, then V^T G V
+  double* V64 = reinterpret_cast<double*>(G);                     // [Le][Ls] V, once G is solved
+  double* W64 = G64 + Le * Ls;                                    // [Le][Ls] V^T G
+  float2* lam = reinterpret_cast<float2*>(W64 + Le * Ls);         // [Le]
+  float2* tm = lam + Le;                                          // [Le] m_j
+  float2* thr = tm + Le;                                          // [Le] squared threshold, m (duals)
+  float* tbq = reinterpret_cast<float*>(thr + Le);                // [Le]
   const int q = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const NucFacet f = facets[q];
   const int Nq = (f.r1 - f.r0) * (f.c1 - f.c0);
@@ -713,7 +727,7 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
     const int a = k / Ls, b = k - a * Ls;
     G[k] = make_float2(0.f, 0.f);
     V[k] = make_float2(a == b ? 1.f : 0.f, 0.f);
-    if (W) G64[k] = 0.0;
+    G64[k] = 0.0;
   }
   if (!W)
     for (int j = tid; j < L; j += nt) tbq[j] = theta_bar[(size_t)q * L + j];
@@ -767,75 +781,109 @@ __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, i
     ff x = ff_of(g);
     if (!(fabsf(x.h) < 3e38f)) x = {__int_as_float(0x7fffffff), 0.f};
     G[a * Ls + b] = G[b * Ls + a] = make_float2(x.h, x.l);
-    if (W) G64[a * Ls + b] = G64[b * Ls + a] = g;
+    G64[a * Ls + b] = G64[b * Ls + a] = g;
   }
   __syncthreads();
-  eig_sweeps<false>(G, nullptr, V, rot, pr, &s_more, L, max_sweeps);
-  if constexpr (W) {
-    // ---- B = V^T G V in FP64 over G: V64 over the pairs of G, V64 G over those of V.  Terms of
-    // faint channels are as small as what they add up to, so they keep their relative accuracy
-    double* V64 = reinterpret_cast<double*>(G);
-    double* W64 = reinterpret_cast<double*>(V);
-    for (int k = tid; k < Le * Ls; k += nt) V64[k] = ff_val(ldp(V, k));
-    if (tid == 0) s_more = 0;
-    __syncthreads();
-    for (int k = tid; k < L * L; k += nt) {
-      const int j = k / L, b = k - j * L;
-      double y = 0.0;
-      for (int a = 0; a < L; ++a) y = fma(V64[j * Ls + a], G64[a * Ls + b], y);
-      W64[j * Ls + b] = y;
-    }
-    __syncthreads();
-    for (int e = tid; e < nE; e += nt) {
-      int a, b;
-      entry(e, a, b);
-      double y = 0.0;
-      for (int k = 0; k < L; ++k) y = fma(W64[a * Ls + k], V64[b * Ls + k], y);
-      G64[a * Ls + b] = G64[b * Ls + a] = y;
-    }
-    __syncthreads();
-    int due = 0;
-    for (int e = tid; e < nE; e += nt) {
-      int a, b;
-      entry(e, a, b);
-      if (a != b) due |= pair_turns64(G64[a * Ls + a], G64[a * Ls + b], G64[b * Ls + b]) ? 1 : 0;
-    }
-    if (__syncthreads_or(due)) eig_sweeps<true>(nullptr, G64, nullptr, rot, pr, &s_more, L, max_sweeps);
+  eig_sweeps<false, W>(G, nullptr, V, rot, rot64, pr, &s_more, L, max_sweeps, nullptr);
+  // ---- V^T G V in FP64.  Terms of faint channels are as small as what they add up to, so
+  // they keep their relative accuracy
+  for (int k = tid; k < Le * Ls; k += nt) V64[k] = ff_val(ldp(V, k));
+  if (tid == 0) s_more = 0;
+  __syncthreads();
+  for (int k = tid; k < L * L; k += nt) {
+    const int j = k / L, b = k - j * L;
+    double y = 0.0;
+    for (int a = 0; a < L; ++a) y = fma(V64[j * Ls + a], G64[a * Ls + b], y);
+    W64[j * Ls + b] = y;
+  }
+  __syncthreads();
+  for (int e = tid; e < nE; e += nt) {
+    int a, b;
+    entry(e, a, b);
+    double y = 0.0;
+    for (int k = 0; k < L; ++k) y = fma(W64[a * Ls + k], V64[b * Ls + k], y);
+    G64[a * Ls + b] = G64[b * Ls + a] = y;
+  }
+  __syncthreads();
+  auto diagonal = [&]() {
     for (int j = tid; j < L; j += nt) {
-      const double x = G64[j * Ls + j];
-      int rk = 0;
-      for (int k = 0; k < L; ++k) {
-        const double y = G64[k * Ls + k];
-        rk += y > x || (y == x && k < j);
-      }
-      const double sv = sqrt(fmax(x, 0.0)) * __hiloint2double((1023 + k4) << 20, 0);
-      tb_out[(size_t)q * L + rk] = (float)((double)mb / (sv + (double)mb));
+      const ff x = ff_of(G64[j * Ls + j]);
+      lam[j] = make_float2(x.h, x.l);
     }
-  } else {
-    for (int j = tid; j < L; j += nt) lam[j] = G[j * Ls + j];
     __syncthreads();
-    for (int j = tid; j < L; j += nt) {
-      const float2 x = lam[j];
-      int rk = 0;
+  };
+  auto rank_of = [&](int j) {
+    const float2 x = lam[j];
+    int rk = 0;
 #pragma unroll 4
-      for (int k = 0; k < L; ++k) {
-        const float2 y = lam[k];
-        rk += (y.x > x.x) || (y.x == x.x && (y.y > x.y || (y.y == x.y && k < j)));
-      }
-      rank[j] = rk;
+    for (int k = 0; k < L; ++k) {
+      const float2 y = lam[k];
+      rk += (y.x > x.x) || (y.x == x.x && (y.y > x.y || (y.y == x.y && k < j)));
+    }
+    return rk;
+  };
+  // squared thresholds of the entries: duals, the smallest alpha from the entry's rank on;
+  // weights, (3e-3 mu_bar)^2
+  const double unit = __hiloint2double((1023 - k4) << 20, 0);
+  diagonal();
+  for (int j = tid; j < Le; j += nt) {
+    float t = 3e-3f, m = 1.f;
+    if (!W && j < L) {
+      const int rk = rank_of(j);
+      t = INFINITY;
+      for (int k = rk; k < L; ++k) t = fminf(t, tbq[k]);
+      const float al = (float)((double)mb * (double)inv_zeta * (double)tbq[rk] * unit);
+      m = fminf(1.f, al * rsqrtf(fmaxf(lam[j].x, 1e-37f)));
+    }
+    t = (float)((double)mb * (W ? 1.0 : (double)inv_zeta) * (double)t * unit);
+    thr[j] = make_float2(t * t, m);
+  }
+  __syncthreads();
+  int due = 0;
+  for (int e = tid; e < nE; e += nt) {
+    int a, b;
+    entry(e, a, b);
+    if (a != b && pair_turns64<W>(G64[a * Ls + a], G64[a * Ls + b], G64[b * Ls + b], thr[a], thr[b])) due = 1;
+  }
+  if (__syncthreads_or(due)) {
+    eig_sweeps<true, W>(nullptr, G64, V, rot, rot64, pr, &s_more, L, max_sweeps, thr);
+    diagonal();
+  }
+  for (int j = tid; j < L; j += nt) {
+    const int rk = rank_of(j);
+    if constexpr (W) {
+      const double sv = sqrt(fmax(G64[j * Ls + j], 0.0)) * __hiloint2double((1023 + k4) << 20, 0);
+      tb_out[(size_t)q * L + rk] = (float)((double)mb / (sv + (double)mb));
+    } else {
       // m = min(1, alpha lambda^-1/2) in the scaled units, 1 where lambda is not positive
-      const ff al = ff_of((double)mb * (double)inv_zeta * (double)tbq[rk] * __hiloint2double((1023 - k4) << 20, 0));
+      const ff al = ff_of((double)mb * (double)inv_zeta * (double)tbq[rk] * unit), x = ldp(lam, j);
       ff m = {1.f, 0.f};
-      if (x.x > 0.f) {
-        const ff t = ff_mul(al, ff_rsqrt({x.x, x.y}));
+      if (x.h > 0.f) {
+        const ff t = ff_mul(al, ff_rsqrt(x));
         if (t.h < 1.f || (t.h == 1.f && t.l < 0.f)) m = t;
       }
       tm[j] = make_float2(m.h, m.l);
     }
+  }
+  if constexpr (!W) {
     __syncthreads();
-    for (int k = tid; k < L * L; k += nt) {        // diag(m) V^T, over G
-      const int j = k / L, o = j * Ls + k - j * L;
-      const ff w = ff_mul(ldp(tm, j), ldp(V, o));
+    // first order of what the pairs left beside the diagonal: M = V (diag(m) + F) V^T with
+    // F_ij = B_ij (m_i - m_j) / (lambda_i - lambda_j), B = V^T G V (F over V^T G, then
+    // (diag(m) + F) V^T over G)
+    float* F = reinterpret_cast<float*>(W64);
+    for (int k = tid; k < L * L; k += nt) {
+      const int i = k / L, j = k - i * L;
+      const float dm = __fadd_rn(__fsub_rn(tm[i].x, tm[j].x), __fsub_rn(tm[i].y, tm[j].y));
+      const float d = __fadd_rn(__fsub_rn(lam[i].x, lam[j].x), __fsub_rn(lam[i].y, lam[j].y));
+      F[k] = dm != 0.f && d != 0.f ? (float)G64[i * Ls + j] / d * dm : 0.f;
+    }
+    __syncthreads();
+    for (int k = tid; k < L * L; k += nt) {
+      const int j = k / L, c = k - j * L, o = j * Ls + c;
+      float first = 0.f;
+#pragma unroll 4
+      for (int i = 0; i < L; ++i) first = fmaf(F[j * L + i], V[i * Ls + c].x, first);
+      const ff w = ff_add(ff_mul(ldp(tm, j), ldp(V, o)), {first, 0.f});
       G[o] = make_float2(w.h, w.l);
     }
     __syncthreads();
@@ -1001,10 +1049,10 @@ void launch_nuclear_gram_eig(fhs_ctx* ctx, const Cube& cb, const float* xcheck, 
   }
   auto go = [&](auto kernel, bool& attr) {
     if (!attr) {
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_smem(kMaxL, weights_mode));
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_smem(kMaxL));
       attr = true;
     }
-    kernel<<<Q, eig_threads(L), eig_smem(L, weights_mode), st>>>(
+    kernel<<<Q, eig_threads(L), eig_smem(L), st>>>(
         ctx->s.gram, nch, sum ? kEigParts : parts, cb.d_facets, L, theta_bar, cb.d_mubar, (float)(1.0 / cb.zeta),
         ctx->s.nucM, theta_bar_out, 40);
   };

@@ -142,3 +142,30 @@ def test_dual_at_any_scale(L, scale):
     # FP32 rows times an FP32 matrix, in units of the scale; below 1e-31 FP32's own spacing too
     tol = 2.0 * (L + 2) * 2.0 ** -24 * np.linalg.norm(Z / scale) * np.linalg.norm(M) + n * np.sqrt(L) * 2.0 ** -149 / scale
     assert np.linalg.norm(got / scale - (Z / scale) @ M) <= tol
+
+
+@pytest.mark.parametrize("L", [2, 4, 7, 8, 10, 16, 24, 32, 36, 64])
+def test_dual_beside_a_bright_pixel(L):
+    """A bright pixel whose values have 7 bits (every Gram kernel forms their products exactly) and
+    independent faint noise elsewhere: s_1 is about 6e4 times the others, whose thresholds and vectors
+    show in the faint pixels (their own products with M are accurate to FP32)."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    n = 64
+    rng = np.random.default_rng(2000 + L)
+    x = rng.standard_normal((L, n, n))
+    x[:, :16] = 0.0                                  # the source has a Gram chunk of its own
+    x[:, 0, 0] = rng.integers(96, 128, L) * 2.0 ** np.floor(np.log2(6e4 * np.sqrt(48.0 * n / L) / 112))
+    x = x.astype(np.float32)
+    Z = x.reshape(L, -1).T.astype(np.float64)
+    U, s, Vt = np.linalg.svd(Z, full_matrices=False)
+    tb = np.linspace(0.3, 1.0, L).astype(np.float32)
+    mu_bar = float(s[L // 2])
+    m = np.minimum(1.0, mu_bar * tb.astype(np.float64) / s)
+    M = (Vt.T * m) @ Vt
+    got, ref, faint = _dual(x, mu_bar, tb), Z @ M, slice(16 * n, None)
+    # FP32 rows times an FP32 matrix, and an FP64 solve: about 8 sweeps of L rotations of a row, two
+    # roundings each, 2^-53 of the largest eigenvalue and adding up at random
+    tol = 2.0 * (L + 2) * 2.0 ** -24 * np.linalg.norm(np.abs(Z[faint]) @ np.abs(M))
+    tol += 4.0 * np.sqrt(L) * 2.0 ** -53 * (s[0] / s[-1]) ** 2 * np.linalg.norm(ref[faint])
+    assert np.linalg.norm(got[faint] - ref[faint]) <= tol
