@@ -391,7 +391,8 @@ typedef struct {
 /* Process-wide switch for the contexts created afterwards.  mode 0: defaults (tile 64,
  * tile-staged de-gridder, tcgen05 Gram, fused SARA, 16 CTAs per SM); 1: read each
  * cube's choices from the cache file when it holds the cube's key (device name,
- * compute capability, n1 x n2, L, Qy x Qx, B, total visibilities), else measure them in
+ * compute capability, n1 x n2, L, Qy x Qx, B, total visibilities, generation of the kernels:
+ * entries measured on older kernels stay unread), else measure them in
  * fhs_create (pattern inputs, CUDA events: one warm-up, three timed launches per
  * candidate) and write them to the file; 2: always measure, then write.  cache_path:
  * a JSON object of objects of numbers, or NULL for no file.  The file is replaced

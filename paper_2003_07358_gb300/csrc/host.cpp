@@ -1218,6 +1218,11 @@ std::mutex g_tune_mu;
 std::string g_tune_path;
 using TuneFile = std::map<std::string, std::map<std::string, double>>;
 
+// Generation of the kernels that the choices stand for: raised when a choice comes to select
+// another kernel or its candidates change speed (2: gram_tc selects k_gram_small up to 8
+// channels; new SARA, Gram and l2,1 kernels), so that older measurements are taken again.
+constexpr int kTuneGeneration = 2;
+
 std::string tune_key(const fhs_cube_desc& d) {
   int dev = 0;
   cudaDeviceProp p;
@@ -1228,9 +1233,9 @@ std::string tune_key(const fhs_cube_desc& d) {
   std::string name = p.name;
   for (char& ch : name)
     if (ch == '"' || ch == '\\' || (unsigned char)ch < 32) ch = '_';
-  char buf[320];
-  snprintf(buf, sizeof(buf), "%s|sm_%d%d|n=%dx%d|L=%d|Q=%dx%d|B=%d|M=%lld", name.c_str(), p.major, p.minor, d.n1,
-           d.n2, d.L, d.Qy, d.Qx, d.B, (long long)m);
+  char buf[352];
+  snprintf(buf, sizeof(buf), "%s|sm_%d%d|n=%dx%d|L=%d|Q=%dx%d|B=%d|M=%lld|kernels=%d", name.c_str(), p.major, p.minor,
+           d.n1, d.n2, d.L, d.Qy, d.Qx, d.B, (long long)m, kTuneGeneration);
   return buf;
 }
 
