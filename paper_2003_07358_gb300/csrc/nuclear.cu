@@ -175,7 +175,11 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
 // FP64 (float pairs, whose low part rounds at about 2^-47 of the sum, were off by 4e-8 of s_max
 // at 38 channels and 1.2e-7 at 64 where these are by 8e-9, and left FP32's range below 1e-18).
 // Blocks of entries and pixel groups over the threads as in k_gram, so that every warp is
-// full: bound by the FP64 pipe, 16 instructions of 64 clk per pixel, warp and 4 x 4 block.
+// full; blockIdx.z takes a share of the blocks (at most kGramShare), so that the CTAs of a facet
+// balance over the SMs: bound by the FP64 pipe, 16 instructions of 64 clk per pixel, warp
+// and 4 x 4 block.
+constexpr int kGramShare = 28;     // blocks of entries per CTA of k_gram_f64
+
 template <int LB>
 __global__ void __launch_bounds__(256) k_gram_f64(const float* __restrict__ xc, const NucFacet* __restrict__ facets,
                                                   const double* __restrict__ win64, int n1, int n2, int L,
@@ -192,11 +196,13 @@ __global__ void __launch_bounds__(256) k_gram_f64(const float* __restrict__ xc, 
   if (p0 >= Nq) return;
   const int p1 = min(Nq, p0 + kGramChunk);
   const int nb = (L + LB - 1) / LB, Lp = nb * LB;
-  const int npairs = nb * (nb + 1) / 2;
+  // this CTA's blocks first .. first + npairs - 1 of the upper triangle
+  const int all = nb * (nb + 1) / 2, share = (all + gridDim.z - 1) / gridDim.z;
+  const int first = blockIdx.z * share, npairs = min(share, all - first);
   const int G = max(1, (int)blockDim.x / npairs);
   const int pair = threadIdx.x % npairs, g = threadIdx.x / npairs;
   const bool active = g < G;
-  int ta = 0, rem = pair;
+  int ta = 0, rem = first + pair;
   while (rem >= nb - ta) { rem -= nb - ta; ++ta; }
   const int tb = ta + rem;
   double acc[LB][LB];
@@ -241,7 +247,7 @@ __global__ void __launch_bounds__(256) k_gram_f64(const float* __restrict__ xc, 
     const int pr = k / (LB * LB), ij = k - pr * LB * LB, i = ij / LB, j = ij - i * LB;
     double v = 0.0;
     for (int gg = 0; gg < G; ++gg) v += sm.red[((size_t)gg * npairs + pr) * LB * LB + ij];
-    int xa = 0, xr = pr;
+    int xa = 0, xr = first + pr;
     while (xr >= nb - xa) { xr -= nb - xa; ++xa; }
     const int a = xa * LB + i, b = (xa + xr) * LB + j;
     if (a < L && b < L) {
@@ -1000,12 +1006,13 @@ static void gram_cuda_core(fhs_ctx* ctx, const Cube& cb, const float* xcheck, co
 
 static void gram_weights(fhs_ctx* ctx, const Cube& cb, const float* x, cudaStream_t st) {
   const int L = cb.L, nch = nchunk_max(cb);
-  auto go = [&](auto kernel) {
-    kernel<<<dim3(nch, cb.Qy * cb.Qx), 256, 0, st>>>(x, cb.d_facets, cb.d_win64, cb.n1, cb.n2, L, ctx->s.gram, nch);
+  auto go = [&](auto kernel, int LB) {
+    const int nb = (L + LB - 1) / LB, z = (nb * (nb + 1) / 2 + kGramShare - 1) / kGramShare;
+    kernel<<<dim3(nch, cb.Qy * cb.Qx, z), 256, 0, st>>>(x, cb.d_facets, cb.d_win64, cb.n1, cb.n2, L, ctx->s.gram, nch);
   };
-  if (L <= 4) go(k_gram_f64<1>);
-  else if (L <= 16) go(k_gram_f64<2>);
-  else go(k_gram_f64<4>);
+  if (L <= 4) go(k_gram_f64<1>, 1);
+  else if (L <= 16) go(k_gram_f64<2>, 2);
+  else go(k_gram_f64<4>, 4);
   note_launches(1);
 }
 
