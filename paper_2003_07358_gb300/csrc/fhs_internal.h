@@ -153,9 +153,8 @@ struct Scratch {
 // Streams, events and scratch of one further lane of an iteration.
 struct Lane {
   Scratch s;
-  cudaStream_t stream = nullptr, aux = nullptr, aux2 = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;   // this lane's fork to its aux streams, join from aux
-  cudaEvent_t ev_join2 = nullptr;                     // join from aux2
+  cudaStream_t stream = nullptr, aux = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;   // this lane's fork to / join from its aux stream
   cudaEvent_t ev_done = nullptr;                      // the lane's last work (joined by the first lane)
 };
 

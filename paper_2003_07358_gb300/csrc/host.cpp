@@ -647,7 +647,6 @@ void free_scratch(Scratch& s) {
 void free_lane(fhs_ctx* ctx, Lane& x, int slot) {
   if (x.stream) cudaStreamSynchronize(x.stream);
   if (x.aux) cudaStreamSynchronize(x.aux);
-  if (x.aux2) cudaStreamSynchronize(x.aux2);
   Scratch& s = x.s;
   void* ps[] = {s.grid, s.pack, s.coef, s.t0, s.t1, s.t2, s.t3, s.img, s.vis, s.vis2, s.red, s.gram, s.nucM,
                 s.blk_scale, s.blk_out, s.ll1, s.ll2, s.ll3};
@@ -656,8 +655,7 @@ void free_lane(fhs_ctx* ctx, Lane& x, int slot) {
   s = Scratch();
   if (x.stream) cudaStreamDestroy(x.stream);
   if (x.aux) cudaStreamDestroy(x.aux);
-  if (x.aux2) cudaStreamDestroy(x.aux2);
-  for (cudaEvent_t e : {x.ev_fork, x.ev_join, x.ev_join2, x.ev_done})
+  for (cudaEvent_t e : {x.ev_fork, x.ev_join, x.ev_done})
     if (e) cudaEventDestroy(e);
   x = Lane();
   for (Cube& cb : ctx->cubes) cb.tm_grid[slot] = nullptr;
@@ -739,8 +737,6 @@ bool make_lane(fhs_ctx* ctx) {
   if (ok) {
     ok = cudaStreamCreateWithFlags(&x.stream, cudaStreamNonBlocking) == cudaSuccess &&
          cudaStreamCreateWithFlags(&x.aux, cudaStreamNonBlocking) == cudaSuccess &&
-         cudaStreamCreateWithFlags(&x.aux2, cudaStreamNonBlocking) == cudaSuccess &&
-         cudaEventCreateWithFlags(&x.ev_join2, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&x.ev_fork, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&x.ev_join, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&x.ev_done, cudaEventDisableTiming) == cudaSuccess;
@@ -801,15 +797,6 @@ const Cube& get_cube(fhs_ctx* ctx, int32_t c) {
 }
 
 // ------------------------------------------------------ composite steps
-// Per-basis offsets of the synthesised LL1 bands used by the fused SARA path.
-void set_ll1_offsets(fhs_ctx* ctx, const Cube& cb) {
-  int64_t off = 0;
-  for (int b = 0; b < 8; ++b) {
-    ctx->s.ll1_off[b] = off;
-    off += (int64_t)cb.L * cb.sara.rows[b][1] * cb.sara.cols[b][1];
-  }
-}
-
 // The plain path's [L][I] coefficient buffer, allocated on first use.
 void ensure_coef(fhs_ctx* ctx) {
   if (!ctx->s.coef) ctx->s.coef = dalloc<float>(ctx->s.coef_elems);
@@ -833,7 +820,6 @@ void sara_dual(fhs_ctx* ctx, const Cube& cb, const float* xcheck, float* W, cons
   cudaStream_t st = ctx->stream;
   if (use_fast(ctx, cb) && cb.sara_fast) {
     ensure_coef(ctx);
-    set_ll1_offsets(ctx, cb);
     launch_sara_fast(ctx, cb, xcheck, W, theta, A, nullptr, false, st);
   } else {
     ensure_coef(ctx);
@@ -943,8 +929,6 @@ void swap_lane(fhs_ctx* ctx, Lane& x) {
   std::swap(ctx->s, x.s);
   std::swap(ctx->stream, x.stream);
   std::swap(ctx->aux, x.aux);
-  std::swap(ctx->aux2, x.aux2);
-  std::swap(ctx->ev_join2, x.ev_join2);
   std::swap(ctx->ev_fork, x.ev_fork);
   std::swap(ctx->ev_join, x.ev_join);
 }
