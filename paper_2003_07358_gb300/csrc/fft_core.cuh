@@ -72,12 +72,27 @@ static __constant__ float2 c_w32[16] = {
     {-9.238795325e-01f, -3.826834324e-01f}, {-9.807852804e-01f, -1.950903220e-01f},
 };
 
-// In-place R-point DFT of v (natural order in and out), R = 2^a, radix-2 decimation in time
-// down to the 8-, 4- and 2-point kernels; sign exp(-2 pi i / R), INV flips it.
+// exp(-2 pi i j / 48), j < 24
+static __constant__ float2 c_w48[24] = {
+    {1.000000000e+00f, 0.000000000e+00f}, {9.914448614e-01f, -1.305261922e-01f}, {9.659258263e-01f, -2.588190451e-01f},
+    {9.238795325e-01f, -3.826834324e-01f}, {8.660254038e-01f, -5.000000000e-01f}, {7.933533403e-01f, -6.087614290e-01f},
+    {7.071067812e-01f, -7.071067812e-01f}, {6.087614290e-01f, -7.933533403e-01f}, {5.000000000e-01f, -8.660254038e-01f},
+    {3.826834324e-01f, -9.238795325e-01f}, {2.588190451e-01f, -9.659258263e-01f}, {1.305261922e-01f, -9.914448614e-01f},
+    {0.000000000e+00f, -1.000000000e+00f}, {-1.305261922e-01f, -9.914448614e-01f}, {-2.588190451e-01f, -9.659258263e-01f},
+    {-3.826834324e-01f, -9.238795325e-01f}, {-5.000000000e-01f, -8.660254038e-01f}, {-6.087614290e-01f, -7.933533403e-01f},
+    {-7.071067812e-01f, -7.071067812e-01f}, {-7.933533403e-01f, -6.087614290e-01f}, {-8.660254038e-01f, -5.000000000e-01f},
+    {-9.238795325e-01f, -3.826834324e-01f}, {-9.659258263e-01f, -2.588190451e-01f}, {-9.914448614e-01f, -1.305261922e-01f},
+};
+
+// In-place R-point DFT of v (natural order in and out), R = 2^a or 3 2^a, radix-2
+// decimation in time down to the 8-, 4-, 3- and 2-point kernels; sign exp(-2 pi i / R),
+// INV flips it.
 template <int R, bool INV>
 __device__ __forceinline__ void rdft(float2* v) {
   if constexpr (R == 2) {
     dft2(v[0], v[1]);
+  } else if constexpr (R == 3) {
+    dft3(v[0], v[1], v[2], INV);
   } else if constexpr (R == 4) {
     dft4(v[0], v[1], v[2], v[3], INV);
   } else if constexpr (R == 8) {
@@ -100,7 +115,7 @@ __device__ __forceinline__ void rdft(float2* v) {
       } else if (2 * k == H) {               // w = -i (forward), +i (inverse)
         t = INV ? make_float2(-o[k].y, o[k].x) : make_float2(o[k].y, -o[k].x);
       } else {
-        float2 w = c_w32[k * (32 / R)];
+        float2 w = R % 3 ? c_w32[k * (32 / R)] : c_w48[k * (48 / R)];
         if (INV) w.y = -w.y;
         t = cmul(o[k], w);
       }

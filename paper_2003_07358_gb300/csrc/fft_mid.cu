@@ -19,9 +19,6 @@
 // adjoint at 16 channels of 1024^2, these 32 + 41 and 43 + 25 us.  What bounds them now is
 // DRAM for the columns and the rows' latency (two exchanges, 94 registers a thread).
 #include <cuda_runtime.h>
-#include <math.h>
-
-#include <vector>
 
 #include "fft_core.cuh"
 #include "fhs_internal.h"
@@ -67,138 +64,40 @@ bool mid_side(int K) {
   return K == 128 || K == 96;
 }
 
-// ------------------------------------------------------------- register DFTs
-// exp(-2 pi i j / 48), j < 24
-static __constant__ float2 c_w48[24] = {
-    {1.000000000e+00f, 0.000000000e+00f}, {9.914448614e-01f, -1.305261922e-01f}, {9.659258263e-01f, -2.588190451e-01f},
-    {9.238795325e-01f, -3.826834324e-01f}, {8.660254038e-01f, -5.000000000e-01f}, {7.933533403e-01f, -6.087614290e-01f},
-    {7.071067812e-01f, -7.071067812e-01f}, {6.087614290e-01f, -7.933533403e-01f}, {5.000000000e-01f, -8.660254038e-01f},
-    {3.826834324e-01f, -9.238795325e-01f}, {2.588190451e-01f, -9.659258263e-01f}, {1.305261922e-01f, -9.914448614e-01f},
-    {0.000000000e+00f, -1.000000000e+00f}, {-1.305261922e-01f, -9.914448614e-01f}, {-2.588190451e-01f, -9.659258263e-01f},
-    {-3.826834324e-01f, -9.238795325e-01f}, {-5.000000000e-01f, -8.660254038e-01f}, {-6.087614290e-01f, -7.933533403e-01f},
-    {-7.071067812e-01f, -7.071067812e-01f}, {-7.933533403e-01f, -6.087614290e-01f}, {-8.660254038e-01f, -5.000000000e-01f},
-    {-9.238795325e-01f, -3.826834324e-01f}, {-9.659258263e-01f, -2.588190451e-01f}, {-9.914448614e-01f, -1.305261922e-01f},
-};
-
-// 8-point DFT with the eighth roots folded into the last butterflies (one rounding of their
-// products less than a complex product, and fewer instructions).
-template <bool INV>
-__device__ __forceinline__ void mid_dft8(float2* v) {
-  float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
-  float2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-  dft4(e0, e1, e2, e3, INV);
-  dft4(o0, o1, o2, o3, INV);
-  const float c = 0.70710678118654752440f;
-  // (o1 w, o3 w^3) / c and o2 w^2, w = (1 -+ i) c
-  const float2 t1 = INV ? make_float2(o1.x - o1.y, o1.y + o1.x) : make_float2(o1.x + o1.y, o1.y - o1.x);
-  const float2 t3 = INV ? make_float2(-o3.x - o3.y, o3.x - o3.y) : make_float2(o3.y - o3.x, -o3.y - o3.x);
-  const float2 t2 = INV ? make_float2(-o2.y, o2.x) : make_float2(o2.y, -o2.x);
-  v[0] = cadd(e0, o0);
-  v[4] = csub(e0, o0);
-  v[1] = make_float2(fmaf(c, t1.x, e1.x), fmaf(c, t1.y, e1.y));
-  v[5] = make_float2(fmaf(-c, t1.x, e1.x), fmaf(-c, t1.y, e1.y));
-  v[2] = cadd(e2, t2);
-  v[6] = csub(e2, t2);
-  v[3] = make_float2(fmaf(c, t3.x, e3.x), fmaf(c, t3.y, e3.y));
-  v[7] = make_float2(fmaf(-c, t3.x, e3.x), fmaf(-c, t3.y, e3.y));
-}
-
-// x exp(-2 pi i j / R) (INV: +), 0 <= j < R, j known at compile time.
+// v[k] *= w^k, w = exp(-+2 pi i b / len) (table step `step` per unit of b): the powers w^1 ..
+// w^(S-1) and w^S, w^2S, ... come from the table and the others are one product of two of
+// them.  (Products over the set bits of k, up to four, had a 1.1 times larger error; a load
+// for every power took 1.6 to 1.8 times as long for the rows.)
 template <int R, bool INV>
-__device__ __forceinline__ float2 mid_root(float2 x, int j) {
-  if (j == 0) return x;
-  if (4 * j == R) return INV ? make_float2(-x.y, x.x) : make_float2(x.y, -x.x);
-  if (2 * j == R) return make_float2(-x.x, -x.y);
-  if (4 * j == 3 * R) return INV ? make_float2(x.y, -x.x) : make_float2(-x.y, x.x);
-  const bool neg = 2 * j > R;
-  const int h = neg ? j - R / 2 : j;
-  float2 w = R % 3 ? c_w32[h * (32 / R)] : c_w48[h * (48 / R)];
-  if (INV) w.y = -w.y;
-  if (neg) w = make_float2(-w.x, -w.y);
-  return cmul(x, w);
-}
-
-// In-place R-point DFT (natural order in and out), R = 3, 4, 8 or A B with 4 x 3, 4 x 4, 8 x 3,
-// 4 x 8: DFTs of A over stride B, twiddles, DFTs of B.  One level of twiddles below a pass
-// where a radix-2 recursion has two or three, whose products round as often.
-template <int R, bool INV>
-__device__ __forceinline__ void mid_dft(float2* v) {
-  if constexpr (R == 3) {
-    dft3(v[0], v[1], v[2], INV);
-  } else if constexpr (R == 4) {
-    dft4(v[0], v[1], v[2], v[3], INV);
-  } else if constexpr (R == 8) {
-    mid_dft8<INV>(v);
-  } else {
-    constexpr int A = R == 24 ? 8 : 4, B = R / A;
-    static_assert(A * B == R && (B == 3 || B == 4 || B == 8), "register DFT");
-    float2 u[B][A];
+__device__ __forceinline__ void mid_twiddle(float2* v, int b, int len, const float2* __restrict__ tw, int step) {
+  constexpr int S = R >= 24 ? 8 : 4;
+  float2 lo[S], hi[(R + S - 1) / S];
+  int e = 0;
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
-#pragma unroll
-      for (int a = 0; a < A; ++a) u[b][a] = v[b + B * a];
-      mid_dft<A, INV>(u[b]);
-    }
-#pragma unroll
-    for (int k = 0; k < A; ++k) {
-      float2 z[B];
-#pragma unroll
-      for (int b = 0; b < B; ++b) z[b] = mid_root<R, INV>(u[b][k], b * k);
-      mid_dft<B, INV>(z);
-#pragma unroll
-      for (int m = 0; m < B; ++m) v[k + A * m] = z[m];
-    }
+  for (int j = 1; j < S && j < R; ++j) {
+    e = e + b >= len ? e + b - len : e + b;
+    lo[j] = __ldg(&tw[(size_t)e * step]);
+    if (INV) lo[j].y = -lo[j].y;
   }
-}
-
-// Twiddles exp(-+2 pi i k b / len) of a pass of R-point DFTs: the powers k < S and the multiples
-// of S come from the table, roots rounded to FP32 (x, y) and what the rounding left (z, w),
-// neighbouring b adjacent; the others are one product of two of them, rounded once.
-// Products of the rounded roots under radix-2 register DFTs put the adjoint of 768^2 at 2.4e-7
-// and of 1536^2 at 2.3e-7 from 64 bits, measuring at 1.23e-7 and 1.32e-7; with these, the
-// register DFTs above and mid_scaled below 2.20 and 1.99e-7, 1.00 and 1.00e-7 (mixed-radix transforms:
-// 2.04 and 1.74e-7, 0.97 and 0.99e-7; what is left of the adjoint's is the two-for-one packing,
-// whose halves share each rounding).  A load for every power is no more accurate and took
-// longer (k_mid_row_adj<1536> 121 -> 139 us, k_mid_col_adj 69 -> 82 us at 23 channels).
-__host__ __device__ constexpr int mid_step(int R) { return R >= 24 ? 8 : 4; }
-__host__ __device__ constexpr int mid_rows(int R) { return mid_step(R) - 1 + (R - 1) / mid_step(R); }
-
-// v[k] *= the twiddle of k; t: the pass's table [mid_rows(R)][LD] at b.
-template <int R, int LD, bool INV>
-__device__ __forceinline__ void mid_twiddle(float2* v, const float4* __restrict__ t) {
-  constexpr int S = mid_step(R);
-  auto root = [&](int row) {
-    float4 w = __ldg(t + row * LD);
-    if (INV) { w.y = -w.y; w.w = -w.w; }
-    return w;
-  };
-  float4 lo[S], hi[(R - 1) / S + 1];
+  const int eS = (e + b) % len;
+  e = 0;
 #pragma unroll
-  for (int j = 1; j < S; ++j) lo[j] = root(j - 1);
-#pragma unroll
-  for (int j = 1; j <= (R - 1) / S; ++j) hi[j] = root(S - 2 + j);
+  for (int j = 1; j < (R + S - 1) / S; ++j) {
+    e = e + eS >= len ? e + eS - len : e + eS;
+    hi[j] = __ldg(&tw[(size_t)e * step]);
+    if (INV) hi[j].y = -hi[j].y;
+  }
 #pragma unroll
   for (int k = 1; k < R; ++k) {
-    const float4 p = hi[k / S], q = lo[k % S];
-    float2 w;
-    if (k % S == 0) {
-      w = make_float2(p.x, p.y);
-    } else if (k < S) {
-      w = make_float2(q.x, q.y);
-    } else {
-      const float rx = fmaf(p.z, q.x, fmaf(-p.w, q.y, fmaf(p.x, q.z, -p.y * q.w)));
-      const float ry = fmaf(p.z, q.y, fmaf(p.w, q.x, fmaf(p.x, q.w, p.y * q.z)));
-      w = make_float2(fmaf(p.x, q.x, fmaf(-p.y, q.y, rx)), fmaf(p.x, q.y, fmaf(p.y, q.x, ry)));
-    }
-    v[k] = cmul(v[k], w);
+    const int r = k % S, q = k / S;
+    v[k] = cmul(v[k], r == 0 ? hi[q] : (q == 0 ? lo[r] : cmul(hi[q], lo[r])));
   }
 }
 
 // DFTs of W sequences of length N by the NT threads of the CTA: load(n, w) gives element n
 // of sequence w, store(k, w, v) takes output k.  SEQ: tasks enumerated along a sequence
 // (rows); otherwise across the sequences (columns).  With n = b + NB a, b = d + R3 c and
-// k = ka + R1 (kc + R2 kd): pass 1 over a, pass 2 over c, pass 3 over d.  tw: the length's
-// tables (mid_tables).  Shared memory
+// k = ka + R1 (kc + R2 kd): pass 1 over a, pass 2 over c, pass 3 over d.  Shared memory
 // mid_smem<N, W, SEQ>() bytes; rows of NB + 1 elements per (w, ka) keep the exchanges of a
 // sequence free of bank conflicts.
 template <int N, int W, bool SEQ>
@@ -208,7 +107,8 @@ __host__ __device__ constexpr int mid_smem() {
 }
 
 template <int N, int W, bool SEQ, int NT, bool INV, class Load, class Store>
-__device__ __forceinline__ void mid_fft(float2* sm, const float4* __restrict__ tw, Load load, Store store) {
+__device__ __forceinline__ void mid_fft(float2* sm, const float2* __restrict__ tw, int twstride, Load load,
+                                        Store store) {
   constexpr int R1 = MidCfg<N>::R1, R2 = MidCfg<N>::R2, R3 = MidCfg<N>::R3;
   constexpr int NB = R2 * R3, LD = NB + 1;
   static_assert(R1 * NB == N, "factorisation");
@@ -219,8 +119,8 @@ __device__ __forceinline__ void mid_fft(float2* sm, const float4* __restrict__ t
     float2 v[R1];
 #pragma unroll
     for (int a = 0; a < R1; ++a) v[a] = load(b + NB * a, w);
-    mid_dft<R1, INV>(v);
-    mid_twiddle<R1, NB, INV>(v, tw + b);
+    rdft<R1, INV>(v);
+    mid_twiddle<R1, INV>(v, b, N, tw, twstride);
 #pragma unroll
     for (int a = 0; a < R1; ++a) sm[at(w, a, b)] = v[a];
   }
@@ -232,8 +132,8 @@ __device__ __forceinline__ void mid_fft(float2* sm, const float4* __restrict__ t
       float2 u[R2];
 #pragma unroll
       for (int c = 0; c < R2; ++c) u[c] = sm[at(w, ka, d + R3 * c)];
-      mid_dft<R2, INV>(u);
-      mid_twiddle<R2, R3, INV>(u, tw + mid_rows(R1) * NB + d);
+      rdft<R2, INV>(u);
+      mid_twiddle<R2, INV>(u, d, NB, tw, twstride * R1);
 #pragma unroll
       for (int c = 0; c < R2; ++c) sm[at(w, ka, d + R3 * c)] = u[c];
     }
@@ -244,7 +144,7 @@ __device__ __forceinline__ void mid_fft(float2* sm, const float4* __restrict__ t
       float2 z[R3];
 #pragma unroll
       for (int d = 0; d < R3; ++d) z[d] = sm[at(w, ka, d + R3 * kc)];
-      mid_dft<R3, INV>(z);
+      rdft<R3, INV>(z);
 #pragma unroll
       for (int d = 0; d < R3; ++d) store(ka + R1 * (kc + R2 * d), w, z[d]);
     }
@@ -255,7 +155,7 @@ __device__ __forceinline__ void mid_fft(float2* sm, const float4* __restrict__ t
       float2 z[R2];
 #pragma unroll
       for (int c = 0; c < R2; ++c) z[c] = sm[at(w, ka, c)];
-      mid_dft<R2, INV>(z);
+      rdft<R2, INV>(z);
 #pragma unroll
       for (int c = 0; c < R2; ++c) store(ka + R1 * c, w, z[c]);
     }
@@ -281,37 +181,25 @@ template <int N> struct MidRow {
   static constexpr int SMEM_ADJ = SMEM + W * (N / 2) * (int)sizeof(float2);
 };
 
-// Pairs (rounded value and what the rounding left) of the deapodisation factors: x a b rounded
-// once, where a b in FP32 would round the factors, their product and x's the same way in all
-// channels (5e-8 of an image's 1.5e-7).
-__device__ __forceinline__ float2 mid_pair_mul(float2 a, float2 b) {
-  const float p = __fmul_rn(a.x, b.x);
-  return make_float2(p, __fmaf_rn(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ float mid_scaled(float x, float2 a, float2 b) {
-  const float2 p = mid_pair_mul(a, b);
-  return fmaf(x, p.x, x * p.y);
-}
-
 // Z and column DFT of W packed columns of channel blockIdx.y -> P [L][K1][n2/2].
 template <int N>
 __global__ void __launch_bounds__(MidCol<N>::NT) k_mid_col_fwd(const float* __restrict__ x, float2* __restrict__ P,
-                                                               const float2* __restrict__ sr,
-                                                               const float2* __restrict__ sc, int n1, int n2,
-                                                               const float4* __restrict__ tw) {
+                                                               const float* __restrict__ sr,
+                                                               const float* __restrict__ sc, int n1, int n2,
+                                                               const float2* __restrict__ tw, int twstride) {
   constexpr int W = MidCol<N>::W;
   extern __shared__ float2 sm[];
   const int hp = n2 / 2, h1 = n1 / 2, l = blockIdx.y, j0 = blockIdx.x * W;
   const float* xl = x + (size_t)l * n1 * n2;
   float2* pl = P + (size_t)l * N * hp;
   mid_fft<N, W, false, MidCol<N>::NT, false>(
-      sm, tw,
+      sm, tw, twstride,
       [&](int i, int w) {
         const int r = i < h1 ? i + h1 : (i >= N - h1 ? i - (N - h1) : -1), j = j0 + w;
         if (r < 0 || j >= hp) return make_float2(0.f, 0.f);
-        const float2 s = sr[r];
+        const float s = sr[r];
         const float* xr = xl + (size_t)r * n2;
-        return make_float2(mid_scaled(xr[j + hp], s, sc[j + hp]), mid_scaled(xr[j], s, sc[j]));
+        return make_float2(xr[j + hp] * s * sc[j + hp], xr[j] * s * sc[j]);
       },
       [&](int k, int w, float2 v) {
         if (j0 + w < hp) pl[(size_t)k * hp + j0 + w] = v;
@@ -322,10 +210,10 @@ __global__ void __launch_bounds__(MidCol<N>::NT) k_mid_col_fwd(const float* __re
 // out[l][r][c] (+)= eta_l s_r s_c Re(...).
 template <int N>
 __global__ void __launch_bounds__(MidCol<N>::NT) k_mid_col_adj(const float2* __restrict__ P, float* __restrict__ out,
-                                                               const float2* __restrict__ sr,
-                                                               const float2* __restrict__ sc,
+                                                               const float* __restrict__ sr,
+                                                               const float* __restrict__ sc,
                                                                const float* __restrict__ eta, int accumulate, int n1,
-                                                               int n2, const float4* __restrict__ tw) {
+                                                               int n2, const float2* __restrict__ tw, int twstride) {
   constexpr int W = MidCol<N>::W;
   extern __shared__ float2 sm[];
   const int hp = n2 / 2, h1 = n1 / 2, l = blockIdx.y, j0 = blockIdx.x * W;
@@ -333,14 +221,14 @@ __global__ void __launch_bounds__(MidCol<N>::NT) k_mid_col_adj(const float2* __r
   const float el = eta ? eta[l] : 1.f;
   float* ol = out + (size_t)l * n1 * n2;
   mid_fft<N, W, false, MidCol<N>::NT, true>(
-      sm, tw,
+      sm, tw, twstride,
       [&](int i, int w) { return j0 + w < hp ? pl[(size_t)i * hp + j0 + w] : make_float2(0.f, 0.f); },
       [&](int k, int w, float2 v) {
         const int r = k < h1 ? k + h1 : (k >= N - h1 ? k - (N - h1) : -1), j = j0 + w;
         if (r < 0 || j >= hp) return;
-        const float2 s = sr[r], e = make_float2(el, 0.f);
+        const float s = sr[r];
         float* o = ol + (size_t)r * n2 + j;
-        const float va = mid_scaled(v.x, s, mid_pair_mul(e, sc[j + hp])), vb = mid_scaled(v.y, s, mid_pair_mul(e, sc[j]));
+        const float va = el * sc[j + hp] * s * v.x, vb = el * sc[j] * s * v.y;
         o[hp] = accumulate ? o[hp] + va : va;
         o[0] = accumulate ? o[0] + vb : vb;
       });
@@ -350,7 +238,7 @@ __global__ void __launch_bounds__(MidCol<N>::NT) k_mid_col_adj(const float2* __r
 // columns: sequence 2 m is row k of pair m, sequence 2 m + 1 row K1 - k.
 template <int N>
 __global__ void __launch_bounds__(MidRow<N>::NT) k_mid_row_fwd(float2* __restrict__ grid, const float2* __restrict__ P,
-                                                               int K1, const float4* __restrict__ tw) {
+                                                               int K1, const float2* __restrict__ tw, int twstride) {
   constexpr int W = MidRow<N>::W, HP = N / 4;
   extern __shared__ float2 sm[];
   const int l = blockIdx.y, k0 = blockIdx.x * (W / 2);
@@ -363,7 +251,7 @@ __global__ void __launch_bounds__(MidRow<N>::NT) k_mid_row_fwd(float2* __restric
     return k == 0 || 2 * k == K1 ? -1 : K1 - k;
   };
   mid_fft<N, W, true, MidRow<N>::NT, false>(
-      sm, tw,
+      sm, tw, twstride,
       [&](int n, int w) {
         const int k = row(w);
         if (k < 0 || (n >= HP && n < N - HP)) return make_float2(0.f, 0.f);
@@ -382,7 +270,7 @@ __global__ void __launch_bounds__(MidRow<N>::NT) k_mid_row_fwd(float2* __restric
 // the outputs of rows k and -k, c_j[k] = H_j + i H_{N-HP+j}, H_n = (A_n[k] + conj(A_n[-k])) / 2.
 template <int N>
 __global__ void __launch_bounds__(MidRow<N>::NT) k_mid_row_adj(const float2* __restrict__ grid, float2* __restrict__ P,
-                                                               int K1, const float4* __restrict__ tw) {
+                                                               int K1, const float2* __restrict__ tw, int twstride) {
   constexpr int W = MidRow<N>::W, HP = N / 4;
   extern __shared__ float2 sm[];
   float2* keep = sm + MidRow<N>::SMEM / sizeof(float2);            // [W][2 HP]: columns j, then N - HP + j
@@ -390,7 +278,7 @@ __global__ void __launch_bounds__(MidRow<N>::NT) k_mid_row_adj(const float2* __r
   const float2* gl = grid + (size_t)l * K1 * N;
   float2* pl = P + (size_t)l * K1 * HP;
   mid_fft<N, W, true, MidRow<N>::NT, true>(
-      sm, tw,
+      sm, tw, twstride,
       [&](int n, int w) {
         const int k = k0 + (w >> 1);
         if (k > K1 / 2) return make_float2(0.f, 0.f);
@@ -415,66 +303,43 @@ __global__ void __launch_bounds__(MidRow<N>::NT) k_mid_row_adj(const float2* __r
 }
 
 template <int N>
-void mid_col_fwd(const Cube& cb, const float* x, float2* P, const float4* tw, cudaStream_t st) {
+void mid_col_fwd(const Cube& cb, const float* x, float2* P, const float2* tw, int Kmax, cudaStream_t st) {
   using C = MidCol<N>;
   static bool attr = false;
   if (!attr) { cudaFuncSetAttribute(k_mid_col_fwd<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM); attr = true; }
   k_mid_col_fwd<N><<<dim3((cb.n2 / 2 + C::W - 1) / C::W, cb.L), C::NT, C::SMEM, st>>>(
-      x, P, cb.d_scale_r2, cb.d_scale_c2, cb.n1, cb.n2, tw);
+      x, P, cb.d_scale_r, cb.d_scale_c, cb.n1, cb.n2, tw, Kmax / N);
 }
 
 template <int N>
-void mid_col_adj(const Cube& cb, const float2* P, float* out, const float* eta, bool acc, const float4* tw,
+void mid_col_adj(const Cube& cb, const float2* P, float* out, const float* eta, bool acc, const float2* tw, int Kmax,
                  cudaStream_t st) {
   using C = MidCol<N>;
   static bool attr = false;
   if (!attr) { cudaFuncSetAttribute(k_mid_col_adj<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM); attr = true; }
   k_mid_col_adj<N><<<dim3((cb.n2 / 2 + C::W - 1) / C::W, cb.L), C::NT, C::SMEM, st>>>(
-      P, out, cb.d_scale_r2, cb.d_scale_c2, eta, acc ? 1 : 0, cb.n1, cb.n2, tw);
+      P, out, cb.d_scale_r, cb.d_scale_c, eta, acc ? 1 : 0, cb.n1, cb.n2, tw, Kmax / N);
 }
 
 template <int N>
-void mid_row_fwd(const Cube& cb, float2* grid, const float2* P, const float4* tw, cudaStream_t st) {
+void mid_row_fwd(const Cube& cb, float2* grid, const float2* P, const float2* tw, int Kmax, cudaStream_t st) {
   using C = MidRow<N>;
   static bool attr = false;
   if (!attr) { cudaFuncSetAttribute(k_mid_row_fwd<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM); attr = true; }
-  k_mid_row_fwd<N><<<dim3((cb.K1 / 2 + C::W / 2) / (C::W / 2), cb.L), C::NT, C::SMEM, st>>>(grid, P, cb.K1, tw);
+  k_mid_row_fwd<N><<<dim3((cb.K1 / 2 + C::W / 2) / (C::W / 2), cb.L), C::NT, C::SMEM, st>>>(grid, P, cb.K1, tw,
+                                                                                          Kmax / N);
 }
 
 template <int N>
-void mid_row_adj(const Cube& cb, const float2* grid, float2* P, const float4* tw, cudaStream_t st) {
+void mid_row_adj(const Cube& cb, const float2* grid, float2* P, const float2* tw, int Kmax, cudaStream_t st) {
   using C = MidRow<N>;
   static bool attr = false;
   if (!attr) { cudaFuncSetAttribute(k_mid_row_adj<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_ADJ); attr = true; }
-  k_mid_row_adj<N><<<dim3((cb.K1 / 2 + C::W / 2) / (C::W / 2), cb.L), C::NT, C::SMEM_ADJ, st>>>(grid, P, cb.K1, tw);
-}
-
-// Tables of the passes of length N (mid_twiddle): of the first, then, with three passes, of
-// the second.
-template <int N>
-void mid_tables_n(std::vector<float4>& t) {
-  constexpr int R1 = MidCfg<N>::R1, R2 = MidCfg<N>::R2, R3 = MidCfg<N>::R3, NB = N / R1;
-  auto pass = [&](int R, int LD, int len) {
-    const int S = mid_step(R);
-    for (int row = 0; row < mid_rows(R); ++row) {
-      const int k = row < S - 1 ? row + 1 : (row - (S - 2)) * S;
-      for (int b = 0; b < LD; ++b) {
-        const double a = -2.0 * 3.14159265358979323846 * (double)(k * b % len) / len, c = cos(a), s = sin(a);
-        t.push_back(make_float4((float)c, (float)s, (float)(c - (double)(float)c), (float)(s - (double)(float)s)));
-      }
-    }
-  };
-  pass(R1, NB, N);
-  if (R3 > 1) pass(R2, R3, NB);
+  k_mid_row_adj<N><<<dim3((cb.K1 / 2 + C::W / 2) / (C::W / 2), cb.L), C::NT, C::SMEM_ADJ, st>>>(grid, P, cb.K1, tw,
+                                                                                              Kmax / N);
 }
 
 }  // namespace
-
-std::vector<float4> mid_tables(int K) {
-  std::vector<float4> t;
-  FHS_MID_SWITCH(K, mid_tables_n, t)
-  return t;
-}
 
 // One-pass columns (natural row order) and both sides among the instantiated lengths.  Grids
 // with a side of 32 or 64 cells (images of 16 and 32) keep the transforms they had: 2 to 13 us
@@ -485,15 +350,15 @@ bool fft_mid_supported(const Cube& cb) {
 }
 
 void launch_fft_forward_mid(fhs_ctx* ctx, const Cube& cb, const float* x, float2* grid, cudaStream_t st) {
-  FHS_MID_SWITCH(cb.K1, mid_col_fwd, cb, x, ctx->s.pack, ctx->d_mid_tw + cb.mid_tw1, st)
-  FHS_MID_SWITCH(cb.K2, mid_row_fwd, cb, grid, ctx->s.pack, ctx->d_mid_tw + cb.mid_tw2, st)
+  FHS_MID_SWITCH(cb.K1, mid_col_fwd, cb, x, ctx->s.pack, ctx->d_tw, ctx->Kmax, st)
+  FHS_MID_SWITCH(cb.K2, mid_row_fwd, cb, grid, ctx->s.pack, ctx->d_tw, ctx->Kmax, st)
   note_launches(2);
 }
 
 void launch_fft_adjoint_mid(fhs_ctx* ctx, const Cube& cb, const float2* grid, float* out, const float* eta,
                             bool accumulate, cudaStream_t st) {
-  FHS_MID_SWITCH(cb.K2, mid_row_adj, cb, grid, ctx->s.pack, ctx->d_mid_tw + cb.mid_tw2, st)
-  FHS_MID_SWITCH(cb.K1, mid_col_adj, cb, ctx->s.pack, out, eta, accumulate, ctx->d_mid_tw + cb.mid_tw1, st)
+  FHS_MID_SWITCH(cb.K2, mid_row_adj, cb, grid, ctx->s.pack, ctx->d_tw, ctx->Kmax, st)
+  FHS_MID_SWITCH(cb.K1, mid_col_adj, cb, ctx->s.pack, out, eta, accumulate, ctx->d_tw, ctx->Kmax, st)
   note_launches(2);
 }
 

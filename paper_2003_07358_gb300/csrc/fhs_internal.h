@@ -60,7 +60,6 @@ struct Cube {
   std::vector<double> eta, mu_bar, eps;     // host copies
   int K1, K2;
   int N1c, N2c;                              // column FFT factorisation K1 = N1c * N2c
-  int64_t mid_tw1 = 0, mid_tw2 = 0;          // mid-size transforms: tables of K1 and K2 in ctx->d_mid_tw
   SaraLayout sara;
   std::vector<NucFacet> facets;
   int64_t n_facet_pix;
@@ -85,8 +84,6 @@ struct Cube {
   double* d_win64 = nullptr;                 // window tables in FP64 (reweighting Gram)
   float* d_scale_r = nullptr;                // [n1] deapodisation s_r
   float* d_scale_c = nullptr;                // [n2]
-  float2* d_scale_r2 = nullptr;              // [n1] s_r rounded and the remainder (mid-size transforms)
-  float2* d_scale_c2 = nullptr;              // [n2]
   double* d_eps = nullptr;                   // [L*B]
   int64_t* d_M_lb = nullptr;                 // [L*B] visibilities per (channel, block)
   // preconditioned data duals (Section 3.2): n_sub forward-backward sub-iterations
@@ -165,7 +162,6 @@ struct fhs_ctx {
   std::vector<fhs::Cube> cubes;
   fhs::Scratch s;
   float2* d_tw = nullptr;          // twiddles exp(-2 pi i k / Kmax), k < Kmax
-  float4* d_mid_tw = nullptr;      // tables of the mid-size transforms (mid_tables)
   int Kmax = 0;
   std::string err;
   bool broken = false;
@@ -219,7 +215,6 @@ void launch_fft_forward_fast(fhs_ctx* ctx, const Cube& cb, const float* x, float
 bool fft_forward_packed(const Cube& cb);
 // two-for-one transforms of grid sides 2^a and 3 2^a with one-pass columns (fft_mid.cu)
 bool fft_mid_supported(const Cube& cb);
-std::vector<float4> mid_tables(int K);   // twiddle tables of a length
 void launch_fft_forward_mid(fhs_ctx* ctx, const Cube& cb, const float* x, float2* grid, cudaStream_t st);
 void launch_fft_adjoint_mid(fhs_ctx* ctx, const Cube& cb, const float2* grid, float* out, const float* eta,
                             bool accumulate, cudaStream_t st);

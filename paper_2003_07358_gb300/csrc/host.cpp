@@ -419,17 +419,8 @@ void build_cube(Cube& cb, const fhs_cube_desc& d, cudaStream_t st, int tile) {
 
   // deapodisation s = 1 / phi_hat(2 pi p / K), p = i - n/2
   std::vector<float> sr(d.n1), sc(d.n2);
-  std::vector<float2> sr2(d.n1), sc2(d.n2);                     // rounded, and the remainder
-  for (int i = 0; i < d.n1; ++i) {
-    const double v = 1.0 / kb_phi_hat(2.0 * kPi * (i - d.n1 / 2) / cb.K1);
-    sr[i] = (float)v;
-    sr2[i] = make_float2(sr[i], (float)(v - (double)sr[i]));
-  }
-  for (int i = 0; i < d.n2; ++i) {
-    const double v = 1.0 / kb_phi_hat(2.0 * kPi * (i - d.n2 / 2) / cb.K2);
-    sc[i] = (float)v;
-    sc2[i] = make_float2(sc[i], (float)(v - (double)sc[i]));
-  }
+  for (int i = 0; i < d.n1; ++i) sr[i] = (float)(1.0 / kb_phi_hat(2.0 * kPi * (i - d.n1 / 2) / cb.K1));
+  for (int i = 0; i < d.n2; ++i) sc[i] = (float)(1.0 / kb_phi_hat(2.0 * kPi * (i - d.n2 / 2) / cb.K2));
 
   // visibilities: per-channel tile sort (counting sort, stable)
   cb.M_lb.assign(d.M, d.M + d.L * d.B);
@@ -533,8 +524,6 @@ void build_cube(Cube& cb, const fhs_cube_desc& d, cudaStream_t st, int tile) {
   cb.d_tile_of = dalloc<int>(tile_of.size());
   cb.d_scale_r = dalloc<float>(d.n1);
   cb.d_scale_c = dalloc<float>(d.n2);
-  cb.d_scale_r2 = dalloc<float2>(d.n1);
-  cb.d_scale_c2 = dalloc<float2>(d.n2);
   cb.d_eps = dalloc<double>(cb.eps.size());
   cb.d_eta = dalloc<float>(d.L);
   cb.d_mubar = dalloc<float>(cb.mu_bar.size());
@@ -551,8 +540,6 @@ void build_cube(Cube& cb, const fhs_cube_desc& d, cudaStream_t st, int tile) {
   upload(cb.d_tile_of, tile_of.data(), tile_of.size(), st);
   upload(cb.d_scale_r, sr.data(), sr.size(), st);
   upload(cb.d_scale_c, sc.data(), sc.size(), st);
-  upload(cb.d_scale_r2, sr2.data(), sr2.size(), st);
-  upload(cb.d_scale_c2, sc2.data(), sc2.size(), st);
   upload(cb.d_eps, cb.eps.data(), cb.eps.size(), st);
   upload(cb.d_eta, eta_f.data(), eta_f.size(), st);
   upload(cb.d_mubar, mub_f.data(), mub_f.size(), st);
@@ -567,7 +554,7 @@ void build_cube(Cube& cb, const fhs_cube_desc& d, cudaStream_t st, int tile) {
 
 void free_cube(Cube& cb) {
   void* ps[] = {cb.d_uv, cb.d_blk, cb.d_perm, cb.d_vis_off, cb.d_tile_off, cb.d_facets, cb.d_win, cb.d_win64, cb.d_tile_of,
-                cb.d_scale_r, cb.d_scale_c, cb.d_scale_r2, cb.d_scale_c2, cb.d_eps, cb.d_eta, cb.d_mubar, cb.d_ncmax, cb.d_M_lb, cb.d_U, cb.d_gamma,
+                cb.d_scale_r, cb.d_scale_c, cb.d_eps, cb.d_eta, cb.d_mubar, cb.d_ncmax, cb.d_M_lb, cb.d_U, cb.d_gamma,
                 cb.d_dde_kern, cb.d_dde_idx, cb.d_dde_l1, cb.d_dde_ncmax};
   for (void* p : ps)
     if (p) cudaFree(p);
@@ -1517,25 +1504,6 @@ fhs_status fhs_create(const fhs_cube_desc* cubes, int32_t ncubes, void* stream, 
     }
     ctx->d_tw = dalloc<float2>(kmax);
     upload(ctx->d_tw, tw.data(), tw.size(), ctx->stream);
-    std::map<int, int64_t> mid_at;                             // tables of the mid-size transforms, one per length
-    std::vector<float4> mid_tw;
-    auto mid_table = [&](int K) {
-      auto it = mid_at.find(K);
-      if (it != mid_at.end()) return it->second;
-      const int64_t at = mid_at[K] = (int64_t)mid_tw.size();
-      const std::vector<float4> t = mid_tables(K);
-      mid_tw.insert(mid_tw.end(), t.begin(), t.end());
-      return at;
-    };
-    for (Cube& cb : ctx->cubes)
-      if (fft_mid_supported(cb)) {
-        cb.mid_tw1 = mid_table(cb.K1);
-        cb.mid_tw2 = mid_table(cb.K2);
-      }
-    if (!mid_tw.empty()) {
-      ctx->d_mid_tw = dalloc<float4>(mid_tw.size());
-      upload(ctx->d_mid_tw, mid_tw.data(), mid_tw.size(), ctx->stream);
-    }
     alloc_scratch(ctx);
     encode_degrid_maps(ctx);
     FHS_CUDA(cudaStreamCreateWithFlags(&ctx->gstream, cudaStreamNonBlocking));
@@ -1554,7 +1522,6 @@ fhs_status fhs_create(const fhs_cube_desc* cubes, int32_t ncubes, void* stream, 
     for (Cube& cb : ctx->cubes) free_cube(cb);
     free_scratch(ctx->s);
     if (ctx->d_tw) cudaFree(ctx->d_tw);
-    if (ctx->d_mid_tw) cudaFree(ctx->d_mid_tw);
     if (ctx->gstream) cudaStreamDestroy(ctx->gstream);
     if (ctx->aux) cudaStreamDestroy(ctx->aux);
     if (ctx->aux2) cudaStreamDestroy(ctx->aux2);
@@ -1592,7 +1559,6 @@ fhs_status fhs_destroy(fhs_ctx* ctx) {
   for (Cube& cb : ctx->cubes) free_cube(cb);
   free_scratch(ctx->s);
   if (ctx->d_tw) cudaFree(ctx->d_tw);
-  if (ctx->d_mid_tw) cudaFree(ctx->d_mid_tw);
   delete ctx;
   return FHS_OK;
 }
