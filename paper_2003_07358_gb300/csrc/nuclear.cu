@@ -260,7 +260,9 @@ __global__ void __launch_bounds__(256) k_gram_f64(const float* __restrict__ xc, 
 // Partial Grams of up to LM <= 8 channels: a thread streams pixels (chunks blockIdx.x,
 // blockIdx.x + parts, ... of the facet) and keeps every entry of the upper triangle as a
 // float pair in registers (the products and sums of k_gram), so a pixel is read once and
-// nothing is staged; the CTA adds its threads' pairs in a fixed order.  Output slot
+// nothing is staged; the CTA adds its threads' pairs in a fixed order.  The pairs are normalised
+// after each chunk (8 products a thread), as one facet of 4096^2 adds 2048 of them in a thread,
+// over which a low part that grows would round at 2^-41 of the sum instead of 2^-44.  Output slot
 // blockIdx.x, as k_gram_sum leaves it.  The tensor-core kernel pads such facets to 16
 // channels and pays a chunk's slicing and epilogue all the same: 1.61 ms at 4 channels of
 // 4096^2 (256 facets), here 0.25 ms.
@@ -322,6 +324,12 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
           lo[e] = __fadd_rn(lo[e], __fadd_rn(er, pe));
         }
     }
+#pragma unroll
+    for (int e = 0; e < NP; ++e) {                  // the low part back below the high one's rounding
+      const float h = __fadd_rn(hi[e], lo[e]);
+      lo[e] = __fsub_rn(lo[e], __fsub_rn(h, hi[e]));
+      hi[e] = h;
+    }
   }
   unsigned nonzero = 0, normal = 0;
   bool large = false;
@@ -373,10 +381,7 @@ __global__ void __launch_bounds__(128) k_gram_small(const float* __restrict__ xc
     return;
   }
 #pragma unroll
-  for (int e = 0; e < NP; ++e) {
-    const float h = __fadd_rn(hi[e], lo[e]);
-    red[tid * LD + e] = make_float2(h, __fsub_rn(lo[e], __fsub_rn(h, hi[e])));
-  }
+  for (int e = 0; e < NP; ++e) red[tid * LD + e] = make_float2(hi[e], lo[e]);
   __syncthreads();
   if (tid < SH * NP) {
     const int e = tid % NP;

@@ -169,3 +169,34 @@ def test_dual_beside_a_bright_pixel(L):
     tol = 2.0 * (L + 2) * 2.0 ** -24 * np.linalg.norm(np.abs(Z[faint]) @ np.abs(M))
     tol += 4.0 * np.sqrt(L) * 2.0 ** -53 * (s[0] / s[-1]) ** 2 * np.linalg.norm(ref[faint])
     assert np.linalg.norm(got[faint] - ref[faint]) <= tol
+
+
+@pytest.mark.parametrize("L", [2, 4, 8])
+def test_dual_of_one_large_facet(L):
+    """A facet of 4096^2 pixels, where a thread of the Gram kernel adds thousands of products:
+    channels that differ by 1e-6, whose dual is that much of them, scaled by alpha / s_j."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    n = 4096
+    g = torch.Generator(device="cuda").manual_seed(L)
+    b = torch.rand((1, n * n), generator=g, device="cuda", dtype=torch.float64) ** 4
+    c = torch.linspace(0.6, 1.4, L, device="cuda", dtype=torch.float64)[:, None]
+    x = (b * c + 1e-6 * b.square().mean().sqrt() * torch.randn((L, n * n), generator=g, device="cuda")).float()
+    # the singular values through a basis whose first vector is the spectrum c: its Gram is graded, and so
+    # are its Cholesky factor's entries, which one-sided rotations keep
+    basis = torch.linalg.qr(torch.cat([c, torch.eye(L, device="cuda", dtype=torch.float64)[:, 1:]], 1))[0]
+    Y = basis.T @ x.double()
+    R = np.linalg.cholesky((Y @ Y.T).cpu().numpy()).T
+    U, s, V = jacobi_svd(R)
+    V = basis.cpu().numpy() @ V
+    alpha = 0.5 * float(s[-1])
+    ctx = _context(n, L, alpha)
+    P, A = torch.zeros(L * n * n, device="cuda"), torch.zeros((L, n, n), device="cuda")
+    ctx.fhs_prox_nuclear_facets(0, x.view(L, n, n), P, torch.ones((1, L), device="cuda"), A)
+    ctx.close()
+    for j in range(1, L):
+        v = torch.as_tensor(np.ascontiguousarray(V[:, j]), device="cuda")
+        z, p = v @ x.double(), v @ P.view(L, -1).double()
+        m = float((p @ z) / (z @ z)) / (alpha / s[j])
+        # s_j^2 from a Gram to 2^-47 of s_1^2 (float pairs), and 2^-10 for the solve and FP32
+        assert abs(m - 1.0) <= 0.5 * 2.0 ** -47 * (s[0] / s[j]) ** 2 + 2.0 ** -10, (j, m - 1.0, s[0] / s[j])
