@@ -814,7 +814,7 @@ def main():
                 "vs_baseline": None, "dtype": "f32", "data": "synthetic",
                 "config": {"workload": spec.name, "n": spec.n, "L": spec.L, "subcubes": spec.C,
                            "facets": f"{spec.Q}x{spec.Q}", "vis_per_channel": spec.M, "blocks": spec.B,
-                           "path": "FP32 fused kernels (FP64 reductions)", "lanes": lanes,
+                           "path": "FP32 fused kernels (reductions in float pairs and FP64)", "lanes": lanes,
                            "l2": "working set ~100 GB >> 129 MB L2; no flush"},
                 "roofline": roofline, "operators": ops, "cpu_baseline": cpu, "e2e": e2e,
                 "plain_fp32_path": plain, "snr_gap_vs_fp64": gaps, "dde_degridding": dde_line, "mixed_size_batch": batch_line,

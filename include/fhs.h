@@ -180,7 +180,7 @@ fhs_status fhs_prox_l21_sara_facets(fhs_ctx* ctx, int32_t cube, const float* xch
 /* Low-rankness duals of every facet (Algorithm 2, P update, Table 2 row 2):
  * P_q <- (I - prox_{zeta^-1 mu_bar_q ||.||_{*,theta_bar_q}})(P_q + D_q S~_q Xcheck),
  * then A += zeta S~_q^T D_q P_q.  The prox is computed as P_q <- Z V diag(m) V^T
- * with Z^T Z = V diag(s^2) V^T (FP64 eigen-solve) and m_j = min(1, alpha_j / s_j). */
+ * with Z^T Z = V diag(s^2) V^T (eigenvalues to FP64's accuracy) and m_j = min(1, alpha_j / s_j). */
 fhs_status fhs_prox_nuclear_facets(fhs_ctx* ctx, int32_t cube, const float* xcheck,
                                    float* P, const float* theta_bar, float* A);
 /* Data duals with U = I (Table 2 row 4): for every (l, b),

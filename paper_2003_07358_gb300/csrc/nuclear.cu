@@ -8,8 +8,8 @@
 //   k_gram   : partial Gram matrices Z^T Z of pixel chunks (float pairs, staged in smem;
 //              k_gram_f64 for the weights, k_gram_small up to 8 channels);
 //   k_eig    : FP64 sum of the partials in fixed order (k_gram_sum first where there are
-//              many), cyclic Jacobi eigen-solve of the L x L Gram in float pairs,
-//              M_q = V diag(m) V^T (or weights);
+//              many), cyclic Jacobi eigen-solve of the L x L Gram in float pairs, finished
+//              in FP64, M_q = V diag(m) V^T (or weights);
 //   k_apply  : pixel-driven: for each pixel and each facet covering it,
 //              P_q <- Z_q M_q and A += zeta D_q P_q (every A pixel written once).
 #include <cuda_runtime.h>
@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(256, LB == 4 ? 1 : 3) k_gram(const float* __re
 // Blocks of entries and pixel groups over the threads as in k_gram, so that every warp is
 // full; blockIdx.z takes a share of the blocks (at most kGramShare), so that the CTAs of a facet
 // balance over the SMs: bound by the FP64 pipe, 16 instructions of 64 clk per pixel, warp
-// and 4 x 4 block.
+// and 4 x 4 block.  0.69 ms at 36 facets of 85^2 pixels and 38 channels (1.68 ms in the earlier FP64
+// kernel, whose warps were partly filled, 0.24 ms in float pairs).
 constexpr int kGramShare = 28;     // blocks of entries per CTA of k_gram_f64
 
 template <int LB>
@@ -705,7 +706,8 @@ static size_t eig_smem(int L) {
 // sides by two threads, a barrier; the eigenvector rows of a round are rotated
 // beside the next round's rotations.  One warp in FP64 took 1.09 ms at 20
 // channels (16 facets), 3.74 ms at 32 (64 facets) and, for the weights, 6.48 ms at 38 (36
-// facets); this kernel takes 0.098, 0.24 and 0.33 ms (device times of one launch).
+// facets); this kernel takes 0.125, 0.29 and 0.35 ms (device times of one launch; 0.098, 0.24
+// and 0.33 without the FP64 stage).
 template <bool W>
 __global__ void __launch_bounds__(1024) k_eig(const double* __restrict__ part, int nchunk_max, int nparts_max,
                                              const NucFacet* __restrict__ facets, int L,
